@@ -284,13 +284,13 @@ LNBNN_API lnbnn_status lnbnn_classify_fp8_ws(lnbnn_index *index, lnbnn_workspace
  * lists, so longer lists favour fewer splits.  A launch with at least one
  * wave of query tiles also takes at least as many splits as keep each
  * split's reference bytes in L2 for the FP8 coarse pass (48 MB a split), and
- * 4 (lists of 17..32 entries) or 8 (heaps) for the exact scan; the splits of
+ * 4 (lists of 17..32 keys) or 8 (more than 64) for the exact scan; the splits of
  * a row then run one after another, and each starts from the row's lists of
  * the previous split when that split has finished (the results never depend
  * on whether it has).  A launch of few query tiles with an automatic split
  * count takes the claimed-chunk form instead of splits (the FP8 coarse pass
  * while there are at least 8 SMs per query tile, the exact scan for a lone
- * query tile; lists of up to 32 entries or heaps): each of P / T CTAs per
+ * query tile; lists of up to 32 or more than 64 keys): each of P / T CTAs per
  * query tile keeps that tile's lists for the whole launch and claims short
  * reference chunks, in increasing order, from a counter the tile's CTAs
  * share, so that the reference ranges holding a query's own class, where
@@ -349,9 +349,9 @@ LNBNN_API lnbnn_status lnbnn_plan_splits(const lnbnn_index *index, int64_t n_que
  * of the FP8 shortlist search (fp8 != 0; k1 = the shortlist length).  Nothing
  * is launched.  Fields: the reference splits of the launch and references per
  * split; the sorted lists per query row the scan writes (merged afterwards
- * when more than one); where each list lives (list_storage 0: registers, 1:
- * shared memory, 2: a heap in global memory) and how many entries it holds
- * (16, 24, 32 or 64; k1 for a heap); the tile of query rows x references one CTA
+ * when more than one); where each list is kept while it grows (list_storage 0:
+ * registers, 2: global memory; 1 is not used) and how many keys it has room
+ * for (16, 24, 32 or 64; k1 in global memory); the tile of query rows x references one CTA
  * computes per step (tile_m query rows x tile_n references); persistent = 1
  * when a fixed grid of CTAs takes (query tiles, split) work items from a
  * queue instead of one CTA per item; bound_per_tile: how the lists of a row

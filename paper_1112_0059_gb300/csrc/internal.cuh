@@ -57,11 +57,11 @@ __host__ __device__ __forceinline__ bool row_layout_ok(int row_bytes, int loc_w)
 
 // Reference preparation (rows of row_bytes bytes): exact BF16 copy of the
 // centred appearance coordinates x - 128 (padding rows up to n_pad: zero),
-// squared norms as fp32 (padding rows get kPadNorm) and the K-extension
+// squared norms as fp32 (padding rows get kPadNorm; not if null) and the K-extension
 // [n_pad, kExt] (norm digits, location columns).
 cudaError_t launch_prep_ref(const uint8_t* ref, int64_t n_ref, int64_t n_pad, int row_bytes, int loc_w,
                             __nv_bfloat16* ref_bf, float* rnorm, __nv_bfloat16* ref_ext, cudaStream_t s);
-// Query preparation: squared norms (int32) and, when qbf != nullptr, the BF16
+// Query preparation: squared norms (int32; not if null) and, when qbf != nullptr, the BF16
 // operand -2 (q - 128) (padding rows up to m_pad: zero) and its K-extension
 // [m_pad, kExt] (the weights of the reference's norm digits, the query's norm
 // digits, the location cross-term columns).
@@ -83,13 +83,12 @@ cudaError_t launch_fill_float(float* dst, int64_t n, float v, cudaStream_t s);
 // Merge `splits` sorted lists per row into one sorted list of K1 keys
 // (at most 32 * kMaxListsPerLane lists).  With `chain.done` set (the scan's
 // per-work-item flags of a launch whose splits carried their lists), a row
-// whose last split reports 2 merges only that split's lists_per_split lists.
-constexpr int kMaxListsPerLane = 20;
+// whose last split reports 2 takes that split's list as it is.
+constexpr int kMaxListsPerLane = 10;
 struct MergeChain {
   const uint32_t* done = nullptr;
   int64_t T = 0;              // query-tile groups: work item x + y T is split y of group x
   int64_t rows_per_item = 0;  // query rows per group
-  int lists_per_split = 0;
 };
 cudaError_t launch_merge_lists(const uint64_t* lists, int splits, int64_t m, int64_t list_stride_rows,
                                int K1, uint64_t* out, cudaStream_t s, const MergeChain& chain = MergeChain{});

@@ -35,18 +35,17 @@
 //                        the last chunk of each tile)
 //   warp 1, one thread : tcgen05.mma issuer (9 MMAs of 128x256x16 per tile);
 //                        warp 1 also owns the TMEM allocation; with QT = 2 a
-//                        second issuer (the warp after the epilogue warps)
-//                        issues the second query tile's MMAs
-//   warps 2-9          : epilogue: two warps per TMEM lane quarter, each
+//                        second issuer (warp 2) issues the second query
+//                        tile's MMAs
+//   warps 4-11         : epilogue: two warps per TMEM lane quarter, each
 //                        taking a 128-column half of every tile (QT = 2: its
 //                        query tile's 128 x 128 block) with one thread per
-//                        query row (TMEM lane); each keeps its own sorted
-//                        list of the k+1 nearest (in registers for k+1 <= 64,
-//                        otherwise a heap in global memory; for 33..64 one
-//                        warp per quarter takes all 256 columns, to have the
-//                        registers); two 256-column FP32 accumulators in
-//                        flight; each 32-column load also returns the
-//                        columns' minimum
+//                        query row (TMEM lane); two 256-column FP32
+//                        accumulators in flight; each 32-column load also
+//                        returns the columns' minimum, and groups whose
+//                        minimum is below the row's limit are passed on
+//   warps 12-15        : inserters, one per TMEM lane quarter: the rows' lists
+//                        of the k+1 nearest (not in the NBNN scan)
 // Every wait is bounded; on expiry the CTA records a timeout in the index's
 // device error word, drains what it issued and returns.
 #include <cudaTypedefs.h>
@@ -81,21 +80,29 @@ struct Shape {
   static constexpr uint32_t kStageBytes = kBChunkBytes + kBExtBytes;
 };
 
-// Threads of a CTA whose epilogue has `epq` warps per TMEM lane quarter and
-// which computes `qt` query tiles: the producer warp, one MMA warp per query
-// tile (the second after the epilogue warps) and 4 * epq epilogue warps.
-constexpr int warps_for(int epq, int qt) { return 1 + qt + 4 * epq; }
-constexpr int threads_for(int epq, int qt) { return 32 * warps_for(epq, qt); }
-// Registers per thread above which the CTA's warps cannot share one SM (the
-// sub-partition holding the most warps has 16,384 registers).
-constexpr int max_regs_for(int epq, int qt) {
-  return (16384 / (32 * ((warps_for(epq, qt) + 3) / 4))) / 8 * 8 > 255
-             ? 255
-             : (16384 / (32 * ((warps_for(epq, qt) + 3) / 4))) / 8 * 8;
-}
+// Warps of a CTA, in warpgroups of four: warp 0 the TMA producer, warp 1 the
+// MMA issuer (and the TMEM allocation's owner), warp 2 the second query tile's
+// issuer (QT = 2), warp 3 unused; then eight epilogue warps, two per TMEM lane
+// quarter; then, for lists kept in registers, four inserter warps.
+constexpr int kEpiWarp0 = 4;
+constexpr int kEpiWarps = 8;
+constexpr int kInsWarp0 = kEpiWarp0 + kEpiWarps;
+template <class Epilogue>
+constexpr int kThreadsOf = 32 * (kInsWarp0 + Epilogue::kInserterWarps);
+// Registers a thread of a launch can have (the SM's 65,536 over its threads).
+template <class Epilogue>
+constexpr int kMaxRegsOf = 65536 / kThreadsOf<Epilogue> / 8 * 8;
+// Lists of more than 64 registers a thread: the inserter warps take registers
+// that the first warpgroup, whose roles need few, gives up (the epilogue's two
+// warpgroups keep theirs).
+template <class Epilogue, int QT>
+constexpr bool kWideLists = Epilogue::KMAX * QT > 32;
+constexpr int kRegsFirst = 72, kRegsLaunch = 128, kRegsInserter = 184;
+static_assert(kRegsFirst + 2 * kRegsLaunch + kRegsInserter <= 4 * kRegsLaunch, "what is taken has been given up");
 constexpr uint32_t kAccCols = kTcRefTile;  // FP32 columns per accumulator (one step)
 constexpr uint32_t kTmemCols = 2 * kAccCols;
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per wait
+constexpr uint64_t kItemLimitNs = 60 * kWaitLimitNs;  // a work item, for the warps that wait through all of it
 
 // Shared-memory layout of one CTA: QT query tiles (each AChunks
 // 128-byte-swizzle chunks + the 32-byte-swizzle extension), the reference
@@ -110,10 +117,11 @@ struct Layout {
   static constexpr uint32_t kOffA = 0;  // query tile q at kOffA + q * kAQueryBytes; its extension after its chunks
   static constexpr uint32_t kOffB = QT * kAQueryBytes;
   static constexpr uint32_t kOffBar = kOffB + Stages * S::kStageBytes;
-  // full, empty per stage; tmem full, tmem empty per accumulator; A full, A
-  // empty, drain; item full, item empty per item slot; lists written
-  static constexpr int kNumBars = 2 * Stages + 2 + 2 + 3 + 2 + 2 + 1;
-  // TMEM address, abort flag, 2 item slots, 2 "an earlier split was not carried" words
+  // full, empty per stage; tmem empty per accumulator; A full, A empty,
+  // drain; item full, item empty per item slot; lists written; warm-up done,
+  // the rows' limits posted, the columns of an item all queued
+  static constexpr int kNumBars = 2 * Stages + 2 + 3 + 2 + 2 + 1 + 3;
+  // TMEM address, abort flag, 2 item slots, 2 "an earlier split was not carried" words, work slot
   static constexpr uint32_t kOffMisc = kOffBar + 8 * kNumBars;
   static constexpr uint32_t kOffList = (kOffMisc + 48 + 1023) / 1024 * 1024;
   static constexpr uint32_t kSmemBytes = kOffList + ListBytes + 1024;  // + alignment slack
@@ -145,26 +153,23 @@ struct Bars {
   uint32_t base;
   __device__ uint32_t full(int s) const { return base + 8 * s; }
   __device__ uint32_t empty(int s) const { return base + 8 * (kStages + s); }
-  __device__ uint32_t tfull(int b) const { return base + 8 * (2 * kStages + b); }
-  __device__ uint32_t tempty(int b) const { return base + 8 * (2 * kStages + 2 + b); }
-  __device__ uint32_t afull() const { return base + 8 * (2 * kStages + 4); }
-  __device__ uint32_t aempty() const { return base + 8 * (2 * kStages + 5); }
-  __device__ uint32_t drain() const { return base + 8 * (2 * kStages + 6); }
-  __device__ uint32_t ifull(int i) const { return base + 8 * (2 * kStages + 7 + i); }
-  __device__ uint32_t iempty(int i) const { return base + 8 * (2 * kStages + 9 + i); }
-  __device__ uint32_t lists_done() const { return base + 8 * (2 * kStages + 11); }
+  __device__ uint32_t tempty(int b) const { return base + 8 * (2 * kStages + b); }
+  __device__ uint32_t afull() const { return base + 8 * (2 * kStages + 2); }
+  __device__ uint32_t aempty() const { return base + 8 * (2 * kStages + 3); }
+  __device__ uint32_t drain() const { return base + 8 * (2 * kStages + 4); }
+  __device__ uint32_t ifull(int i) const { return base + 8 * (2 * kStages + 5 + i); }
+  __device__ uint32_t iempty(int i) const { return base + 8 * (2 * kStages + 7 + i); }
+  __device__ uint32_t lists_done() const { return base + 8 * (2 * kStages + 9); }
+  __device__ uint32_t limits() const { return base + 8 * (2 * kStages + 10); }
+  __device__ uint32_t queued() const { return base + 8 * (2 * kStages + 11); }
+  __device__ uint32_t warmed() const { return base + 8 * (2 * kStages + 12); }
 };
 
-// The layout of a kernel instantiation: the format's query chunks; ring
-// stages for two tiles of 256 references (BF16: four chunks, E4M3: two), as
-// many as fit when the epilogue's lists take shared memory (BF16 two, E4M3
-// three), and three or four times as many tiles of 128 references for QT = 2
-// (BF16 six stages, E4M3 eight).
+// The layout of a kernel instantiation: the format's query chunks; four ring
+// stages (two tiles of 256 references in BF16, four in E4M3), for QT = 2 three
+// or eight tiles of 128 references (BF16 six stages, E4M3 eight).
 template <class Fmt, class Epilogue, int QT>
-using LayoutOf = Layout<Fmt::kChunks,
-                        QT == 2 ? (Fmt::kChunks == 2 ? 6 : 8)
-                                : (Epilogue::kListBytes ? (Fmt::kChunks == 2 ? 2 : 3) : 4),
-                        Epilogue::kListBytes, QT>;
+using LayoutOf = Layout<Fmt::kChunks, QT == 2 ? (Fmt::kChunks == 2 ? 6 : 8) : 4, Epilogue::kListBytes, QT>;
 
 __device__ __forceinline__ void flag_timeout(volatile uint32_t* abort_flag, uint32_t* dev_err) {
   *abort_flag = 1u;
@@ -184,65 +189,6 @@ __device__ __forceinline__ bool wait_gate(const uint32_t* gate, uint64_t limit_n
   }
 }
 
-// Sorted list of the K1 smallest (distance, row) pairs seen so far, held in
-// registers: ascending in slots [KMAX-K1, KMAX); the slots below hold the
-// distance -1, which no real distance displaces, so the list always has K1
-// live entries and its largest is slot KMAX-1.  Every list receives its
-// columns in increasing row order, so comparing distances strictly is exact
-// for (distance, row) order: a later row at an equal distance sorts after.
-template <int KMAX>
-struct RegList {
-  int32_t d[KMAX];
-  uint32_t r[KMAX];
-
-  __device__ __forceinline__ void init(int K1) {
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i) {
-      d[i] = i < KMAX - K1 ? -1 : INT32_MAX;
-      r[i] = 0xFFFFFFFFu;
-    }
-  }
-  __device__ __forceinline__ int32_t worst() const { return d[KMAX - 1]; }
-  // Start from a finished list of K1 ascending keys (kEmptyKey: no entry).
-  __device__ __forceinline__ void seed(const uint64_t* src, int K1) {
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i) {
-      if (i >= KMAX - K1) {
-        const uint64_t k = __ldcg(src + (i - (KMAX - K1)));
-        d[i] = k == kEmptyKey ? INT32_MAX : (int32_t)key_dist(k);
-        r[i] = key_row(k);
-      }
-      // at most four keys in flight: the list itself holds the registers
-      if ((i & 3) == 3) asm volatile("" ::: "memory");
-    }
-  }
-  // new[i] = old[i-1] if x sorts before it, else min(x, old[i]); requires x < worst().
-  __device__ __forceinline__ void insert(int32_t x, uint32_t row) {
-#pragma unroll
-    for (int i = KMAX - 1; i > 0; --i) {
-      const bool shift = x < d[i - 1];
-      const bool place = !shift && x < d[i];
-      const int32_t nd = shift ? d[i - 1] : (place ? x : d[i]);
-      const uint32_t nr = shift ? r[i - 1] : (place ? row : r[i]);
-      d[i] = nd;
-      r[i] = nr;
-    }
-    if (x < d[0]) {
-      d[0] = x;
-      r[0] = row;
-    }
-  }
-  // Writes the K1 live entries ascending (unfilled slots as kEmptyKey).
-  __device__ __forceinline__ void store(uint64_t* out, int K1) const {
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i)
-      if (i >= KMAX - K1) out[i - (KMAX - K1)] = d[i] == INT32_MAX ? kEmptyKey : make_key((uint32_t)d[i], r[i]);
-  }
-};
-
-// Bits of a non-negative float (or -0) as int32; ordered like the float.
-__device__ __forceinline__ int32_t thr_bits(int32_t dist) { return __float_as_int((float)dist); }
-
 // v[j] for a run-time j without dynamic register indexing (no local memory):
 // a 5-level select tree on the bits of j.
 __device__ __forceinline__ int32_t select32(const uint32_t (&v)[32], int j) {
@@ -258,23 +204,9 @@ __device__ __forceinline__ int32_t select32(const uint32_t (&v)[32], int j) {
   return (int32_t)((j & 16) ? t[1] : t[0]);
 }
 
-// Bit j set when column j's distance is below the threshold.
-__device__ __forceinline__ uint32_t hit_mask(const uint32_t (&v)[32], int32_t thr) {
-  uint32_t mask = 0;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) mask |= ((int32_t)v[j] < thr ? 1u : 0u) << j;
-  return mask;
-}
-
-template <>
-struct RegList<0> {
-  __device__ __forceinline__ void init(int) {}
-};
-
-// KMAX > 0: per-row lists in registers (K1 <= KMAX); KMAX = 0: heaps in global memory.
-// What the epilogue writes (see the two epilogues below).
+// What the scan writes (see the epilogues below).
 struct ScanOut {
-  uint64_t* lists;           // kNN: sorted lists, [splits * lists per split][stride][K1]
+  uint64_t* lists;           // kNN: sorted lists, [splits][stride][K1]
   int64_t stride;
   int K1;
   int32_t* mins;             // NBNN: per (query row, class) minimum distance, [m_pad][C], atomicMin
@@ -287,277 +219,354 @@ struct ScanOut {
                              // lists are written, 2 if they also hold every earlier split's keys (zero
                              // before the launch), or null
   int64_t T;                 // query-tile groups of the launch (work item w - T is the same rows' previous split)
-  int lists_per_split;
+  char* work;                // kNN: candidate buffers of the lists in progress, work_slots x tc_work_bytes(entries)
+  int64_t work_slots;
+  int entries;
+  uint32_t* slot_used;       // one word per slot, zero before the launch; null if the grid has no more CTAs than slots
 };
 
-// kNN epilogue: the K1 smallest (distance, row) keys of the columns one
-// thread sees (Alg. 2's NN(d, k+1) restricted to a slice of the references).
+// A work slot of the launch for this CTA: its own number where the grid has no
+// more CTAs than slots.  Otherwise there is a slot per SM, a CTA fills an SM
+// (its shared memory), and so one of the slots is always free.
+__device__ __forceinline__ int32_t acquire_slot(const ScanOut& out) {
+  if (out.slot_used == nullptr) return (int32_t)blockIdx.x;
+  int32_t s = (int32_t)(blockIdx.x % out.work_slots);
+  const uint64_t t0 = globaltimer_ns();
+  while (atomicExch(out.slot_used + s, 1u) != 0u) {
+    s = s + 1 < out.work_slots ? s + 1 : 0;
+    if (s == 0 && globaltimer_ns() - t0 > kWaitLimitNs) return -1;
+  }
+  __threadfence();
+  return s;
+}
+__device__ __forceinline__ void release_slot(const ScanOut& out, int32_t s) {
+  if (out.slot_used == nullptr || s < 0) return;
+  __threadfence();
+  atomicExch(out.slot_used + s, 0u);
+}
+
+// kNN (Alg. 2's NN(d, k+1) restricted to the columns one CTA sees): the lists
+// are kept by warps of their own.  An epilogue warp that inserted its own
+// candidates held up its tile, and with it the other seven and the
+// accumulator's return to the MMAs, for as long as the insert took (101-class
+// data, k = 50: 3,660 cycles a step against the MMAs' 1,152; k = 100 and
+// FP8 shortlist 128 on the 256-class data, heaps: 4,680 and 4,180).
 //
-// The lists (here and in KnnSmemEpilogue) share a bound per query row with the other lists of that row
-// (the other column half, the other reference splits): row_thr[row] holds the
-// bit pattern of a distance at or below which some list already holds K1
-// entries, so a column farther than it cannot be among the row's K1 nearest
-// and is not offered (a column at exactly the bound still is: it may win on
-// its row).  When the lists of a row run at the same time (few query tiles,
-// many splits), a full list publishes its K1-th distance with an atomic
-// minimum after each tile that improved it, and reads the word once per tile
-// (the read issued at the end of one tile is taken in at the end of the
-// next).  When they run one after another (many query tiles: the splits of a
-// row are work items far apart), a list reads the word once when it starts
-// and publishes once when it ends.  Which columns a list drops depends on
-// timing; the K1 nearest of the row never are, so the merged result does not.
-template <int KMAX>
-struct KnnEpilogue {
-  static constexpr int kWarpsPerQuarter = KMAX == kTcWideRegListMax ? 1 : 2;
-  static constexpr bool kSeeds = true;  // can start from the previous split's list of its rows
-  static constexpr bool kClaimsChunks = true;  // can keep its lists across claimed reference chunks
-  static constexpr uint32_t kListBytes = 0;
-  RegList<KMAX> L;
-  TopK top;
-  int32_t thr;      // bit pattern of this list's K1-th distance (INT32_MAX's while not full)
-  int32_t shared;   // the row's shared bound as last read (bit pattern)
-  int32_t pending;  // the read in flight for the next tile
-  int32_t* rthr;    // the row's shared bound, or null
-  bool per_tile;    // share the bound every tile (else at start and end)
-  bool active;
-  int K1;
-  uint64_t* out;
-  __device__ __forceinline__ KnnEpilogue(const ScanOut& o, int list, int64_t row, bool act, int64_t, uint8_t*, int)
-      : top(o.lists + ((int64_t)list * o.stride + (act ? row : 0)) * o.K1, o.K1),
-        thr(thr_bits(INT32_MAX)),
-        shared(kNoBound),
-        pending(kNoBound),
-        rthr(act && o.row_thr ? o.row_thr + row : nullptr),
-        per_tile(o.bound_per_tile),
-        active(act),
-        K1(o.K1),
-        out(o.lists + ((int64_t)list * o.stride + (act ? row : 0)) * o.K1) {
-    L.init(K1);
-    if (rthr && !per_tile) shared = __ldcg(rthr);
+// An epilogue warp compares the least value of each 32-column group (which the
+// TMEM load returns) with its rows' limits; each of its threads appends the
+// octets of columns that hold one below its row's limit to a buffer.  One
+// inserter warp per TMEM lane quarter takes the buffers of the quarter's two
+// epilogue warps when they are handed over, sorts their columns into the rows'
+// lists (registers, or merge_rows) and posts the rows' new limits; the epilogue
+// goes on in a second set of buffers meanwhile.  The buffers are in global
+// memory (L2): a hit costs the epilogue about 300 cycles of predicated stores
+// (copying single columns 1,000), whatever the list length.  The limit may be
+// read late: that changes which columns are appended, never which K1 keys the
+// list ends with, since keys are compared by (distance, row) and a column at
+// the limit passes.  Measured, whole calls before and after (one GB300):
+// 101-class data, 200k rows, k = 50 121.6 / 64.2 ms; 256-class data, 15k rows,
+// k = 100 95.0 / 37.5 ms, FP8 shortlist 128 84.5 / 28.0 ms, shortlist 24 on
+// one image of 632 rows 1.31 / 0.90 ms.
+//
+// The lists of a row in other reference splits share a bound with it:
+// row_thr[row] holds the bit pattern of a distance at or below which some list
+// already holds K1 entries, so a column farther than it cannot be among the
+// row's K1 nearest.  When the lists of a row run at the same time (few query
+// tiles, many splits), a merge publishes an improved K1-th distance with an
+// atomic minimum, and the inserters read the word every few polls.  When they
+// run one after another (many query tiles: the splits of a row are work items
+// far apart), a list reads the word once when it starts and publishes once
+// when it ends.  Which columns a list drops depends on timing; the K1 nearest
+// of the row never are, so the merged result does not.
+//
+// Warm-up: a list that starts empty would copy every column until its first
+// merge.  So the first `warm_tiles` tiles of an item are run twice, first for
+// a limit alone: their columns fall into at least K1 groups (the row's columns
+// of one tile and column half, or of 32 columns where the item is short), each
+// group's least value is the distance of another column, and the largest of
+// them therefore bounds the K1-th smallest distance.
+constexpr int32_t kNoBound = 0x7F7F7F7F;  // row_thr's initial value: above every distance
+
+struct WarmUp {
+  int tiles;  // tiles run twice
+  bool fine;  // groups of 32 columns
+};
+template <int QT>
+__device__ __forceinline__ WarmUp warm_up(int ntiles, int K1) {
+  constexpr int kHalves = QT == 2 ? 1 : 2;  // column halves of a row per tile
+  const int wide = (K1 + kHalves - 1) / kHalves, fine = (K1 + 4 * kHalves - 1) / (4 * kHalves);
+  if (ntiles >= 2 * wide) return {wide, false};
+  if (ntiles >= fine) return {fine, true};
+  return {0, false};
+}
+
+// Shared memory of the hand-over between epilogue and inserter warps.
+struct HandOver {
+  static constexpr uint32_t kGiven = 0;                     // hand-overs made, per epilogue warp (8)
+  static constexpr uint32_t kDone = kGiven + 8 * 4;         // hand-overs merged, per epilogue warp
+  static constexpr uint32_t kCount = kDone + 8 * 4;         // candidates handed over, per epilogue thread (256)
+  static constexpr uint32_t kWarm = kCount + 256 * 4;       // warm-up bound, per epilogue thread
+  static constexpr uint32_t kLim = kWarm + 256 * 4;         // limit, per query row (256)
+  static constexpr uint32_t kBytes = kLim + 256 * 4;
+  uint32_t base;
+  __device__ uint32_t given(uint32_t w) const { return base + kGiven + 4 * w; }
+  __device__ uint32_t done(uint32_t w) const { return base + kDone + 4 * w; }
+  __device__ uint32_t count(uint32_t t) const { return base + kCount + 4 * t; }
+  __device__ uint32_t warm(uint32_t t) const { return base + kWarm + 4 * t; }
+  __device__ uint32_t lim(uint32_t row) const { return base + kLim + 4 * row; }
+};
+
+// The epilogue warps' side: each thread collects its row's candidates, eight
+// neighbouring columns at a time: what is in the epilogue's path is then one
+// compare and three predicated stores per octet, and the columns are sorted
+// out by the inserters, whose 32 lanes each have a row's to sort.
+struct Collector {
+  HandOver ho;
+  uint32_t w, lane;         // epilogue warp, half * 4 + quarter
+  uint32_t lim_at;          // its row's limit in shared memory
+  const char* mine;         // this thread's two buffers of `cap` entries
+  uint32_t cap;
+  uint32_t soft;            // entries worth a merge if the inserter is free
+  volatile uint32_t* abort_flag;
+  uint32_t* dev_err;
+  const char* start;        // the buffer being filled
+  uint32_t n = 0;           // entries in it
+  uint32_t given = 0;       // hand-overs made
+  int32_t lim = INT32_MIN;  // a column enters below it (bit pattern)
+  __device__ __forceinline__ void read_limit() { lim = (int32_t)ld_shared_u32(lim_at); }
+  // Hands the warp's buffers over and goes on with the other ones, once the
+  // hand-over before has been merged (without `wait`: only if it has).
+  // False when the CTA gives up.
+  __device__ __forceinline__ bool hand_over(bool wait) {
+    if (ld_shared_acquire(ho.done(w)) != given) {
+      if (!wait) return true;
+      const uint64_t t0 = globaltimer_ns();
+      for (uint32_t it = 1; ld_shared_acquire(ho.done(w)) != given; ++it) {
+        if ((it & 63u) == 0 && __any_sync(0xffffffffu, *abort_flag != 0u || globaltimer_ns() - t0 > kWaitLimitNs)) {
+          flag_timeout(abort_flag, dev_err);
+          n = 0;  // (the candidates are lost: the call reports the timeout)
+          return false;
+        }
+        __nanosleep(40);  // (the inserters need the issue slots)
+      }
+    }
+    st_shared_u32(ho.count(w * 32 + lane), n);
+    __threadfence_block();
+    __syncwarp();
+    ++given;
+    if (lane == 0) st_shared_release(ho.given(w), given);
+    start = mine + (given & 1u) * cap * kTcEntryBytes;
+    n = 0;
+    read_limit();
+    return true;
   }
-  static constexpr int32_t kNoBound = 0x7F7F7F7F;  // the word's initial value: above every distance
-  // One 32-column group: one compare of the group's minimum bit pattern (mn,
-  // from the reducing TMEM load); on a hit, the columns below the limit are
-  // offered in column order, each checked again as the limit tightens.  A
-  // column at exactly the list's K1-th distance cannot enter: its row is
-  // higher than every kept row's.
-  __device__ __forceinline__ void group(const uint32_t (&v)[32], uint32_t mn, int64_t col0) {
-    int32_t lim = min(thr, shared + 1);  // strictly below: own K1-th, at or below: the shared bound
-    const bool hit = active && (int32_t)mn < lim;
-    if (__any_sync(0xffffffffu, hit)) {
-      if (hit) {
-        for (uint32_t mask = hit_mask(v, lim); mask; mask &= mask - 1) {
-          const int j = __ffs(mask) - 1;
-          const int32_t bits = select32(v, j);
-          if (bits < lim) {
-            const int32_t d = __float2int_rn(__int_as_float(bits));
-            if constexpr (KMAX > 0) {
-              L.insert(d, (uint32_t)(col0 + j));
-              thr = thr_bits(L.worst());
-            } else {
-              top.push(make_key((uint32_t)d, (uint32_t)(col0 + j)));
-              thr = thr_bits(top.threshold);
-            }
-            lim = min(thr, shared + 1);
-          }
+  // 32 columns, some below some row's limit.
+  __device__ __forceinline__ void group(const uint32_t (&v)[32], uint32_t col) {
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const uint32_t* x = v + 8 * o;
+      const int32_t a = __vimin3_s32((int32_t)x[0], (int32_t)x[1], (int32_t)x[2]);
+      const int32_t b = __vimin3_s32((int32_t)x[3], (int32_t)x[4], (int32_t)x[5]);
+      const int32_t c = __vimin3_s32(a, (int32_t)x[6], (int32_t)x[7]);
+      push_octet_if_less(start, n, min(b, c), lim, x, col + 8u * o);
+    }
+  }
+  // Two 32-column groups with their minima (mn, from the reducing TMEM load).
+  __device__ __forceinline__ void round(const uint32_t (&v0)[32], uint32_t mn0, const uint32_t (&v1)[32], uint32_t mn1,
+                                        int64_t col0) {
+    if (!__any_sync(0xffffffffu, (int32_t)min(mn0, mn1) < lim)) return;
+    // the limit is read again only here, where it matters (a read per tile cost
+    // the FP8 pass 4%)
+    read_limit();
+    if (__any_sync(0xffffffffu, n + 8 > cap)) hand_over(true);
+    if (__any_sync(0xffffffffu, (int32_t)mn0 < lim)) group(v0, (uint32_t)col0);
+    if (__any_sync(0xffffffffu, (int32_t)mn1 < lim)) group(v1, (uint32_t)col0 + 32u);
+    if (__any_sync(0xffffffffu, n >= soft)) hand_over(false);
+  }
+};
+
+// The inserter warps' side: warp `quarter` has the 32 rows of its TMEM lane
+// quarter (QT = 2: of each query tile); lane l holds the state of row l.
+template <int KMAX, int QT>
+struct Inserter {
+  // Lists of up to 64 keys are a thread's registers, and a hand-over's
+  // candidates go in one per row and step: a step is a network of 6 KMAX
+  // instructions for 32 rows.  Longer ones are in global memory (merge_rows).
+  static constexpr bool kRegs = KMAX > 0;
+  RegList<kRegs ? KMAX : 0> L[QT];
+  HandOver ho;
+  uint32_t quarter, lane;
+  int K1, cap;
+  char* cand;              // this CTA's candidate buffers: [256 epilogue threads][2][cap] entries
+  uint32_t done0 = 0, done1 = 0;  // hand-overs merged of the quarter's two epilogue warps
+  uint64_t* list[QT];      // the lists of the 32 rows: K1 keys each
+  const uint64_t* seed[QT];  // the lists they start from, or null
+  uint32_t listed[QT];     // rows whose list has been written
+  int32_t kth[QT];         // the list's K1-th distance (INT32_MAX: not full)
+  int32_t shared[QT];      // the row's shared bound as last read
+  int32_t lim[QT];         // min(kth, shared) + 1; INT32_MIN: no row here
+  int32_t* rthr[QT];       // the row's shared bound, or null
+  __device__ __forceinline__ void post_limit(int q) {
+    if (lim[q] != INT32_MIN) lim[q] = min(kth[q], shared[q]) + 1;  // at the bound a column may still win on its row
+    st_shared_u32(ho.lim(q * kBM + quarter * 32 + lane), (uint32_t)lim[q]);
+  }
+  // Merges what the epilogue warp of half h has handed over; false if nothing.
+  __device__ __forceinline__ bool take(int h, bool publish) {
+    const uint32_t w = (uint32_t)h * 4 + quarter;
+    const int q = QT == 2 ? h : 0;
+    const uint32_t done = h == 0 ? done0 : done1;
+    if (ld_shared_acquire(ho.given(w)) == done) return false;
+    const int n = (int)ld_shared_u32(ho.count(w * 32 + lane));
+    uint32_t* from =
+        reinterpret_cast<uint32_t*>(cand) + ((int64_t)w * 64 + (done & 1u)) * cap * kEntryWords;
+    const int stride = 2 * cap * kEntryWords;
+    if constexpr (kRegs) {
+      insert_all(L[q], from + lane * stride, n, lim[q]);
+      kth[q] = L[q].worst();
+    } else {
+      const int keys = pack(from + lane * stride, n, lim[q]);
+      const uint32_t rows = __ballot_sync(0xffffffffu, keys > 0);
+      const uint64_t* packed = reinterpret_cast<const uint64_t*>(from);
+      if (K1 <= 128) {
+        kth[q] = merge_rows<4, 2>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
+      } else {
+        kth[q] = merge_rows<8, 1>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
+      }
+      listed[q] |= rows;
+    }
+    if (publish && rthr[q] && kth[q] < shared[q]) {
+      atomicMin(rthr[q], kth[q]);
+      shared[q] = kth[q];
+    }
+    post_limit(q);
+    if (h == 0) done0 = done + 1;
+    else done1 = done + 1;
+    __syncwarp();
+    if (lane == 0) st_shared_release(ho.done(w), done + 1);
+    return true;
+  }
+  // Brings a lane's n entries into L1 (about 1,000 cycles for each one alone,
+  // from L2 while the operands stream); returns the warp's largest n.
+  __device__ __forceinline__ int fetch(const uint32_t* from, int n) const {
+    const int most = (int)__reduce_max_sync(0xffffffffu, (uint32_t)n);
+#pragma unroll 1
+    for (int e = 0; e < most; e += 4) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (e + i < n) {
+          prefetch_l1(from + (e + i) * kEntryWords);
+          prefetch_l1(from + (e + i) * kEntryWords + 8);
         }
       }
-      __syncwarp();
     }
+    return most;
   }
-  // Start from the same rows' finished list of the previous split (K1
-  // ascending keys of lower reference rows than any column to come, so the
-  // strict distance tests keep exact (distance, row) order): the list then
-  // holds the best keys so far and offers only columns that improve on them.
-  __device__ __forceinline__ void seed(const uint64_t* src) {
-    if (!active) return;
-    if constexpr (KMAX > 0) {
-      L.seed(src, K1);
-      thr = thr_bits(L.worst());
-    } else {
-      for (int i = 0; i < K1; ++i) {
-        const uint64_t k = __ldcg(src + i);
-        if (k != kEmptyKey) top.push(k);
+  // The columns below `limit` of a lane's n entries into its list: each step
+  // takes the least column left of every lane's entry.  The next entry is
+  // loaded meanwhile.
+  template <class List>
+  __device__ __forceinline__ void insert_all(List& list, const uint32_t* from, int n, int32_t limit) const {
+    const int most = fetch(from, n);
+    uint4 a = make_uint4(0, 0, 0, 0), b = a;
+    uint32_t col = 0;
+    if (n > 0) {
+      a = ld_global_v4(from);
+      b = ld_global_v4(from + 4);
+      col = ld_global_u32(from + 8);
+    }
+#pragma unroll 1
+    for (int e = 0; e < most; ++e) {
+      int32_t v[8] = {(int32_t)a.x, (int32_t)a.y, (int32_t)a.z, (int32_t)a.w,
+                      (int32_t)b.x, (int32_t)b.y, (int32_t)b.z, (int32_t)b.w};
+      const uint32_t c = col;
+      const int32_t bound = e < n ? limit : INT32_MIN;
+      if (e + 1 < n) {
+        const uint32_t* p = from + (e + 1) * kEntryWords;
+        a = ld_global_v4(p);
+        b = ld_global_v4(p + 4);
+        col = ld_global_u32(p + 8);
       }
-      thr = thr_bits(top.threshold);
-    }
-  }
-  __device__ __forceinline__ bool full() const {
-    if constexpr (KMAX > 0) {
-      return L.worst() != INT32_MAX;
-    } else {
-      return top.size == top.cap;
-    }
-  }
-  // After each tile: publish an improved K1-th distance of a full list, take
-  // in the bound read a tile ago (its latency hidden behind a whole tile), and
-  // start the next read.
-  __device__ __forceinline__ void tile_end() {
-    if (rthr && per_tile) {
-      if (full() && thr < shared) {
-        atomicMin(rthr, thr);
-        shared = thr;
+#pragma unroll 1
+      for (;;) {
+        const int32_t m = min(__vimin3_s32(__vimin3_s32(v[0], v[1], v[2]), v[3], v[4]), __vimin3_s32(v[5], v[6], v[7]));
+        const bool in = m < bound && m <= list.worst();
+        if (!__any_sync(0xffffffffu, in)) break;
+        uint32_t j = 0;
+#pragma unroll
+        for (int i = 7; i >= 0; --i)
+          if (v[i] == m) j = (uint32_t)i;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (j == (uint32_t)i) v[i] = INT32_MAX;
+        list.insert(in ? m : INT32_MAX, in ? c + j : 0xFFFFFFFFu);
       }
-      shared = min(shared, pending);
-      pending = __ldcg(rthr);
     }
   }
-  __device__ __forceinline__ void finish() {
-    if (!active) return;
-    if (rthr && !per_tile && full() && thr < shared) atomicMin(rthr, thr);
-    if constexpr (KMAX > 0) {
-      L.store(out, K1);
-    } else {
-      top.finish();
+  // The columns below `limit` of a lane's n entries, packed in place (an entry
+  // takes as many bytes as eight pairs): (column, distance bits) pairs, as many
+  // as returned.
+  __device__ __forceinline__ int pack(uint32_t* from, int n, int32_t limit) const {
+    const int most = fetch(from, n);
+    uint64_t* at = reinterpret_cast<uint64_t*>(from);
+    uint64_t* const first = at;
+    uint4 a = make_uint4(0, 0, 0, 0), b = a;
+    uint32_t col = 0;
+    if (n > 0) {
+      a = ld_global_v4(from);
+      b = ld_global_v4(from + 4);
+      col = ld_global_u32(from + 8);
+    }
+#pragma unroll 1
+    for (int e = 0; e < most; ++e) {
+      const uint32_t v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+      const uint32_t c = col;
+      const int32_t bound = e < n ? limit : INT32_MIN;
+      if (e + 1 < n) {
+        const uint32_t* p = from + (e + 1) * kEntryWords;
+        a = ld_global_v4(p);
+        b = ld_global_v4(p + 4);
+        col = ld_global_u32(p + 8);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) push_global_if_less(at, (int32_t)v[i], bound, c + (uint32_t)i);
+    }
+    __syncwarp();
+    return (int)(at - first);
+  }
+  // The rows' shared bounds, read again.
+  __device__ __forceinline__ void read_bounds() {
+#pragma unroll
+    for (int q = 0; q < QT; ++q) {
+      const int32_t b = rthr[q] ? min(shared[q], __ldcg(rthr[q])) : shared[q];
+      if (b != shared[q]) {
+        shared[q] = b;
+        post_limit(q);
+      }
+    }
+  }
+  // Writes the rows' lists (those in global memory: of the rows that had no
+  // candidate).
+  __device__ __forceinline__ void finish(int q, uint32_t n_rows) {
+    if constexpr (kRegs) {
+      if (lane < n_rows) L[q].store(list[q] + lane * K1, K1);
+      return;
+    }
+#pragma unroll 1
+    for (uint32_t r = 0; r < n_rows; ++r) {
+      if ((listed[q] >> r) & 1u) continue;
+      for (int e = (int)lane; e < K1; e += 32)
+        list[q][r * K1 + e] = seed[q] ? __ldcg(seed[q] + r * K1 + e) : kEmptyKey;
     }
   }
 };
 
-// kNN epilogue with the lists in shared memory, for lists of up to KM = 64
-// entries on the one-warp-per-quarter layout (register lists that long leave
-// the insert as the bottleneck: a 64-wide insertion network per list and
-// only four warps to hide it).  Each epilogue warp keeps its 32 rows' lists
-// in shared memory, list by list, as float bit patterns and rows, and inserts
-// with the whole warp: lane i computes entries i and i + 32 of the list
-// (shifted, the new key, or unchanged) from their predecessors, so an insert
-// is a few instructions per lane whatever the list length.  Candidates are
-// taken lane by lane (the lowest lane with a hit first) and, within a lane,
-// in column order, so each list still receives its columns in increasing row
-// order.
-template <int KM>
-struct KnnSmemEpilogue {
-  static constexpr int kWarpsPerQuarter = 1;
-  static constexpr bool kSeeds = false;
-  static constexpr bool kClaimsChunks = false;
-  static constexpr int kPerLane = KM / 32;  // list entries each lane computes in an insert
-  static constexpr uint32_t kListBytes = 4 * kWarpsPerQuarter * 32 * KM * 8;
-  static constexpr int32_t kInf = 0x7F800000;  // bits of +inf, above every distance
-  static constexpr int32_t kNoBound = 0x7F7F7F7F;  // the shared bound's initial value
-  static_assert(KM % 32 == 0 && KM <= 64, "entries i and i + 32 per lane");
-  __device__ __forceinline__ void seed(const uint64_t*) {}
-  uint32_t* D;  // this warp's lists: D[list * KM + i] bit patterns, R[list * KM + i] rows
-  uint32_t* R;
-  int32_t thr;      // bit pattern of this lane's list's K1-th entry
-  int32_t shared;   // the row's shared bound as last read (as in KnnEpilogue)
-  int32_t pending;  // the read in flight
-  int32_t* rthr;    // the row's shared bound, or null
-  bool per_tile;    // share the bound every tile (else at start and end)
-  bool active;
-  int K1;
-  int lane;
-  uint64_t* out;
-  __device__ __forceinline__ KnnSmemEpilogue(const ScanOut& o, int list, int64_t row, bool act, int64_t,
-                                             uint8_t* smem_list, int epi_warp)
-      : D(reinterpret_cast<uint32_t*>(smem_list) + (size_t)epi_warp * 32 * KM * 2),
-        R(D + 32 * KM),
-        thr(kInf),
-        shared(kNoBound),
-        pending(kNoBound),
-        rthr(act && o.row_thr ? o.row_thr + row : nullptr),
-        per_tile(o.bound_per_tile),
-        active(act),
-        K1(o.K1),
-        lane((int)(threadIdx.x & 31)),
-        out(o.lists + ((int64_t)list * o.stride + (act ? row : 0)) * o.K1) {
-    if (rthr && !per_tile) shared = __ldcg(rthr);
-    __syncwarp();  // the previous work item's lists have been read out
-    for (int l = 0; l < 32; ++l)
-#pragma unroll
-      for (int e = 0; e < kPerLane; ++e) {
-        D[l * KM + e * 32 + lane] = (uint32_t)kInf;
-        R[l * KM + e * 32 + lane] = 0xFFFFFFFFu;
-      }
-    __syncwarp();
-  }
-  // Insert (x, row) into list L; every lane takes part.  Requires x below the
-  // list's K1-th entry.
-  __device__ __forceinline__ void insert(int L, int32_t x, uint32_t row) {
-    uint32_t* d = D + L * KM;
-    uint32_t* r = R + L * KM;
-    int32_t a[kPerLane];
-    uint32_t ra[kPerLane];
-#pragma unroll
-    for (int e = 0; e < kPerLane; ++e) {
-      a[e] = (int32_t)d[e * 32 + lane];
-      ra[e] = r[e * 32 + lane];
-    }
-    int32_t nd[kPerLane];
-#pragma unroll
-    for (int e = 0; e < kPerLane; ++e) {
-      // predecessor of entry e * 32 + lane: lane - 1 of the same half, or
-      // lane 31 of the previous half for lane 0
-      const int32_t up = __shfl_up_sync(0xffffffffu, a[e], 1);
-      const uint32_t upr = __shfl_up_sync(0xffffffffu, ra[e], 1);
-      int32_t b = up;
-      uint32_t rb = upr;
-      bool has_pred = lane > 0;
-      if (e > 0) {
-        const int32_t w = __shfl_sync(0xffffffffu, a[e - 1], 31);
-        const uint32_t wr = __shfl_sync(0xffffffffu, ra[e - 1], 31);
-        if (lane == 0) {
-          b = w;
-          rb = wr;
-          has_pred = true;
-        }
-      }
-      const bool shift = has_pred && x < b;
-      const bool place = !shift && x < a[e];
-      nd[e] = shift ? b : (place ? x : a[e]);
-      const uint32_t nr = shift ? rb : (place ? row : ra[e]);
-      if (e * 32 + lane < K1) {
-        d[e * 32 + lane] = (uint32_t)nd[e];
-        r[e * 32 + lane] = nr;
-      }
-    }
-    // the list's new K1-th entry
-    const int last = K1 - 1;
-    int32_t v = nd[0];
-#pragma unroll
-    for (int e = 1; e < kPerLane; ++e)
-      if ((last >> 5) == e) v = nd[e];
-    const int32_t nt = __shfl_sync(0xffffffffu, v, last & 31);
-    if (lane == L) thr = nt;
-    __syncwarp();
-  }
-  __device__ __forceinline__ void group(const uint32_t (&v)[32], uint32_t mn, int64_t col0) {
-    // strictly below the list's K1-th entry, at or below the row's shared bound
-    const bool hit = active && (int32_t)mn < min(thr, shared + 1);
-    if (!__any_sync(0xffffffffu, hit)) return;
-    uint32_t mask = hit ? hit_mask(v, min(thr, shared + 1)) : 0u;
-    for (;;) {
-      const uint32_t who = __ballot_sync(0xffffffffu, mask != 0u);
-      if (who == 0u) break;
-      const int L = __ffs(who) - 1;
-      const int j = mask ? __ffs(mask) - 1 : 0;
-      const int32_t x = __shfl_sync(0xffffffffu, select32(v, j), L);
-      const int jl = __shfl_sync(0xffffffffu, j, L);
-      const int32_t tl = __shfl_sync(0xffffffffu, min(thr, shared + 1), L);
-      if (lane == L) mask &= mask - 1;
-      if (x < tl) insert(L, x, (uint32_t)(col0 + jl));  // warp-uniform
-    }
-  }
-  // As in KnnEpilogue: publish a full list's improved K1-th entry, take in the
-  // read from a tile ago, start the next one.
-  __device__ __forceinline__ void tile_end() {
-    if (rthr && per_tile) {
-      if (thr != kInf && thr < shared) {
-        atomicMin(rthr, thr);
-        shared = thr;
-      }
-      shared = min(shared, pending);
-      pending = __ldcg(rthr);
-    }
-  }
-  __device__ __forceinline__ void finish() {
-    __syncwarp();
-    if (!active) return;
-    if (rthr && !per_tile && thr != kInf && thr < shared) atomicMin(rthr, thr);
-    for (int i = 0; i < K1; ++i) {
-      const uint32_t bits = D[lane * KM + i];
-      out[i] = (int32_t)bits == kInf ? kEmptyKey
-                                      : make_key((uint32_t)__float2int_rn(__uint_as_float(bits)), R[lane * KM + i]);
-    }
-  }
+// KMAX: the longest list (16, 24, 32 or 64 keys; 0: up to 256).
+template <int KMAX_>
+struct KnnEpilogue {
+  static constexpr int KMAX = KMAX_;
+  static constexpr int kInserterWarps = 4;
+  static constexpr bool kClaimsChunks = true;  // can keep its lists across claimed reference chunks
+  static constexpr uint32_t kListBytes = HandOver::kBytes;
 };
 
 // NBNN epilogue (Alg. 1's NN_C for every class C): the columns are the
@@ -567,12 +576,10 @@ struct KnnSmemEpilogue {
 // class).  All lanes of a warp see the same columns, so the class bookkeeping
 // is uniform across the warp.
 struct NbnnEpilogue {
-  static constexpr int kWarpsPerQuarter = 2;
-  static constexpr bool kSeeds = false;
+  static constexpr int KMAX = 0;
+  static constexpr int kInserterWarps = 0;
   static constexpr bool kClaimsChunks = false;
-  __device__ __forceinline__ void seed(const uint64_t*) {}
   static constexpr uint32_t kListBytes = 0;
-  __device__ __forceinline__ void tile_end() {}
   int32_t* dst;          // mins + row * C
   const int64_t* class_off;
   int64_t n_ref;
@@ -581,8 +588,7 @@ struct NbnnEpilogue {
   int64_t next;          // first row of the next class
   int32_t run;           // float bits of the running minimum over cls
   bool active;
-  __device__ __forceinline__ NbnnEpilogue(const ScanOut& o, int, int64_t row, bool act, int64_t j_begin, uint8_t*,
-                                          int)
+  __device__ __forceinline__ NbnnEpilogue(const ScanOut& o, int64_t row, bool act, int64_t j_begin)
       : dst(o.mins + (act ? row : 0) * (int64_t)o.C), class_off(o.class_off), n_ref(o.class_off[o.C]), C(o.C),
         run(INT32_MAX), active(act) {
     // class of j_begin: the last c with class_off[c] <= j_begin
@@ -615,6 +621,11 @@ struct NbnnEpilogue {
       run = min(run, select32(v, j));
     }
   }
+  __device__ __forceinline__ void round(const uint32_t (&v0)[32], uint32_t mn0, const uint32_t (&v1)[32], uint32_t mn1,
+                                        int64_t col0) {
+    group(v0, mn0, col0);
+    group(v1, mn1, col0 + 32);
+  }
   __device__ __forceinline__ void finish() { flush(); }
 };
 
@@ -643,7 +654,7 @@ struct Work {
 // Claim: the claimed-chunk form (Work::group > 0), a separate instantiation
 // so that the split form's kernels carry none of its code.
 template <class Fmt, class Epilogue, int QT, bool Claim>
-__global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1)
+__global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
     tc_scan_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_qe,
                    const __grid_constant__ CUtensorMap tmap_r, const __grid_constant__ CUtensorMap tmap_re, int64_t m,
                    int64_t n_ref, Work work, ScanOut out, uint32_t* __restrict__ dev_err,
@@ -654,17 +665,16 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
   using L = LayoutOf<Fmt, Epilogue, QT>;
   constexpr int kStages = L::kStages;
   // The epilogue learns that a tile's MMAs are done from the commit that
-  // frees the tile's last ring stage, where that stage is not reused within
+  // frees the tile's last ring stage: that stage is not reused within
   // two tiles (its next phase then needs this tile's accumulator back, so a
   // parity wait cannot miss a phase); a separate accumulator-full commit per
-  // tile cost the MMA thread 2-10% of a step.  With a two-stage ring the
-  // stage comes back within a tile and the separate commit stays.
-  constexpr bool kStageSignalsTile = kStages >= 2 * KC;
-  constexpr int kEpiPerQuarter = Epilogue::kWarpsPerQuarter;  // epilogue warps per TMEM lane quarter
-  constexpr int kEpiWarps = 4 * kEpiPerQuarter;
+  // tile cost the MMA thread 2-10% of a step.
+  static_assert(kStages >= 2 * KC, "the ring holds two tiles");
+  constexpr bool kAsync = Epilogue::kInserterWarps > 0;  // lists kept by inserter warps
+  constexpr int kListWarps = 4;                        // inserter warps
+  constexpr int kEpiPerQuarter = kEpiWarps / 4;
   constexpr int kEpiCols = kAccCols / kEpiPerQuarter;  // accumulator columns per epilogue warp
   constexpr int kRounds = kEpiCols / 64;               // rounds of two 32-column loads per tile
-  static_assert(QT == 1 || kEpiPerQuarter == 2, "two query tiles need one epilogue warp per tile and quarter");
   static_assert(KC <= kKChunks, "the query tile fits the chunks shared memory is laid out for");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -674,6 +684,7 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
   volatile uint32_t* abort_flag = tmem_slot + 1;
   volatile int64_t* item_slot = reinterpret_cast<volatile int64_t*>(smem + L::kOffMisc + 16);
   volatile uint32_t* chain_broken = reinterpret_cast<volatile uint32_t*>(smem + L::kOffMisc + 32);
+  volatile int32_t* work_slot = reinterpret_cast<volatile int32_t*>(smem + L::kOffMisc + 40);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -682,7 +693,7 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
   // after the epilogue warps), each issuing its tile's MMAs into its half of
   // the accumulator, so that no single thread issues all of a step's MMAs.
   constexpr int kIssuers = QT;
-  constexpr int kSecondIssuerWarp = 2 + kEpiWarps;
+  constexpr int kSecondIssuerWarp = 2;
   const bool issuer = warp == 1 || (kIssuers == 2 && warp == kSecondIssuerWarp);
   // A timeout reported earlier and not yet collected by lnbnn_sync: scan no
   // tiles (every item's lists are still written, empty).
@@ -694,18 +705,28 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
       mbar_init(bars.empty(s), kIssuers);  // the MMA completions that free the stage
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(bars.tfull(b), kIssuers);
       mbar_init(bars.tempty(b), kEpiWarps);  // one arrival per epilogue warp
       mbar_init(bars.ifull(b), 1);
-      mbar_init(bars.iempty(b), kIssuers + kEpiWarps);  // the MMA threads and each epilogue warp
+      // the MMA threads, each epilogue warp and (but for claimed chunks) inserter warp
+      mbar_init(bars.iempty(b), kIssuers + kEpiWarps + (kAsync && !Claim ? kListWarps : 0));
     }
     mbar_init(bars.afull(), 1);
     mbar_init(bars.aempty(), kIssuers);
     mbar_init(bars.drain(), kIssuers);
-    mbar_init(bars.lists_done(), kEpiWarps);
+    mbar_init(bars.lists_done(), kListWarps);
+    mbar_init(bars.warmed(), kEpiWarps);
+    mbar_init(bars.limits(), kListWarps);
+    mbar_init(bars.queued(), kEpiWarps);
     *abort_flag = 0u;
     chain_broken[0] = chain_broken[1] = 0u;
     fence_barrier_init();
+  }
+  if constexpr (kAsync) {
+    if (threadIdx.x < 16) st_shared_u32(sbase + L::kOffList + HandOver::kGiven + 4 * threadIdx.x, 0u);  // given, done
+    if (threadIdx.x == 0) {
+      *work_slot = acquire_slot(out);
+      if (*work_slot < 0) flag_timeout(abort_flag, dev_err);
+    }
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   tc_fence_before();
@@ -735,242 +756,107 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
     const int64_t j_end = min(*j_begin + work.split_len, n_ref);
     return stale_timeout ? 0 : (int)((j_end - *j_begin + kTileN - 1) / kTileN);
   };
+  // The tiles run twice at the start of this CTA's item i: none where the
+  // lists go on from the previous chunk or split.
+  auto warm_tiles = [&](int i, int64_t w, int ntiles) -> WarmUp {
+    if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false};
+    return warm_up<QT>(ntiles, out.K1);
+  };
 
-  if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------ producer
-      // an optional start gate; with nothing loaded the other roles' waits
-      // run out on the abort flag
-      bool go = true;
-      if (out.gate != nullptr && !stale_timeout && !wait_gate(out.gate, kWaitLimitNs, abort_flag)) {
-        flag_timeout(abort_flag, dev_err);
-        go = false;
-      }
-      prefetch_tmap(&tmap_q);
-      prefetch_tmap(&tmap_qe);
-      prefetch_tmap(&tmap_r);
-      prefetch_tmap(&tmap_re);
-      int it = 0;       // reference K-chunks issued
-      int a_loads = 0;  // query tiles issued
-      for (int i = 0; go; ++i) {
-        int64_t w;
-        if (persistent) {
-          const int slot = i & 1;
-          if (i >= 2 && !mbar_wait(bars.iempty(slot), (uint32_t)(((i >> 1) - 1) & 1), kWaitLimitNs, abort_flag)) {
-            flag_timeout(abort_flag, dev_err);
-            break;
-          }
-          w = *abort_flag ? work.n_items
-                          : (int64_t)atomicAdd(work.queue + (chunked ? blockIdx.x / work.group : 0u), 1u);
-          if (w > work.n_items) w = work.n_items;
-          item_slot[slot] = w;
-          mbar_arrive(bars.ifull(slot));
-        } else {
-          w = i == 0 ? (int64_t)blockIdx.x : work.n_items;
+  if (warp < kEpiWarp0) {
+    if constexpr (kWideLists<Epilogue, QT>) reg_dealloc<kRegsFirst>();
+    if (warp == 0) {
+      if (lane == 0) {
+        // ------------------------------------------------------------ producer
+        // an optional start gate; with nothing loaded the other roles' waits
+        // run out on the abort flag
+        bool go = true;
+        if (out.gate != nullptr && !stale_timeout && !wait_gate(out.gate, kWaitLimitNs, abort_flag)) {
+          flag_timeout(abort_flag, dev_err);
+          go = false;
         }
-        if (w >= work.n_items) break;
-        int64_t m0, j_begin;
-        const int ntiles = item_tiles(w, &m0, &j_begin);
-        // the query tiles: once the previous item's MMAs have read theirs (in
-        // the claimed-chunk form, once for the whole launch)
-        if (!chunked || a_loads == 0) {
-          if (a_loads > 0 && !mbar_wait(bars.aempty(), (uint32_t)((a_loads - 1) & 1), kWaitLimitNs, abort_flag)) {
-            flag_timeout(abort_flag, dev_err);
-            break;
-          }
-          mbar_arrive_expect_tx(bars.afull(), QT * (KC * kAChunkBytes + kAExtBytes));
-          for (int q = 0; q < QT; ++q) {
-            const uint32_t a = sbase + L::kOffA + q * L::kAQueryBytes;
-            const int32_t qrow = (int32_t)(m0 + q * kBM);
-            for (int kc = 0; kc < KC; ++kc) tma_load_2d(a + kc * kAChunkBytes, &tmap_q, kc * kBK, qrow, bars.afull());
-            tma_load_2d(a + KC * kAChunkBytes, &tmap_qe, 0, qrow, bars.afull());
-          }
-          ++a_loads;
-        }
-        bool ok = true;
-        for (int t = 0; ok && t < ntiles && !*abort_flag; ++t) {
-          const int32_t row = (int32_t)(j_begin + (int64_t)t * kTileN);
-          for (int kc = 0; kc < KC; ++kc, ++it) {
-            const int s = it % kStages;
-            const uint32_t round = (uint32_t)(it / kStages);
-            if (!mbar_wait(bars.empty(s), (round & 1u) ^ 1u, kWaitLimitNs, abort_flag)) {
+        prefetch_tmap(&tmap_q);
+        prefetch_tmap(&tmap_qe);
+        prefetch_tmap(&tmap_r);
+        prefetch_tmap(&tmap_re);
+        int it = 0;       // reference K-chunks issued
+        int a_loads = 0;  // query tiles issued
+        for (int i = 0; go; ++i) {
+          int64_t w;
+          if (persistent) {
+            const int slot = i & 1;
+            if (i >= 2 && !mbar_wait(bars.iempty(slot), (uint32_t)(((i >> 1) - 1) & 1), kWaitLimitNs, abort_flag)) {
               flag_timeout(abort_flag, dev_err);
-              ok = false;
               break;
             }
-            const uint32_t dst = sbase + L::kOffB + s * Sh::kStageBytes;
-            const bool last = kc == KC - 1;
-            mbar_arrive_expect_tx(bars.full(s), Sh::kBChunkBytes + (last ? Sh::kBExtBytes : 0u));
-            tma_load_2d(dst, &tmap_r, kc * kBK, row, bars.full(s));
-            if (last) tma_load_2d(dst + Sh::kBChunkBytes, &tmap_re, 0, row, bars.full(s));
+            w = *abort_flag ? work.n_items
+                            : (int64_t)atomicAdd(work.queue + (chunked ? blockIdx.x / work.group : 0u), 1u);
+            if (w > work.n_items) w = work.n_items;
+            item_slot[slot] = w;
+            mbar_arrive(bars.ifull(slot));
+          } else {
+            w = i == 0 ? (int64_t)blockIdx.x : work.n_items;
           }
-        }
-        if (!ok || *abort_flag) break;
-      }
-      // every load issued must land before the CTA may exit
-      const uint32_t never = 0;
-      if (a_loads > 0) mbar_wait(bars.afull(), (uint32_t)((a_loads - 1) & 1), kWaitLimitNs, &never);
-      for (int s = 0; s < kStages; ++s) {
-        const int issued = it / kStages + (s < it % kStages ? 1 : 0);
-        if (issued > 0) mbar_wait(bars.full(s), (uint32_t)((issued - 1) & 1), kWaitLimitNs, &never);
-      }
-    }
-  } else if (issuer) {
-    if (lane == 0) {
-      // --------------------------------------------------------- MMA issuers
-      const int q_first = kIssuers == QT ? (warp == 1 ? 0 : 1) : 0;  // this thread's query tiles
-      const int q_last = kIssuers == QT ? q_first + 1 : QT;
-      const long long clk0 = clock64();
-      const uint64_t ns0 = globaltimer_ns();
-      int it = 0;       // reference K-chunks consumed
-      int tg = 0;       // tiles over all items (accumulator use)
-      int64_t tiles_done = 0;
-      bool ok = true;
-      for (int i = 0; ok; ++i) {
-        int64_t w;
-        if (!consume_item(i, &w)) {
-          flag_timeout(abort_flag, dev_err);
-          break;
-        }
-        if (w >= work.n_items) break;
-        int64_t m0, j_begin;
-        const int ntiles = item_tiles(w, &m0, &j_begin);
-        if ((!chunked || i == 0) && !mbar_wait(bars.afull(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
-          flag_timeout(abort_flag, dev_err);
-          break;
-        }
-        tc_fence_after();
-        // no abort-flag read per tile here: shared-memory loads are slow on
-        // this thread while the MMAs stream their operands (the per-tile
-        // read cost 2% of the FP8 pass), and a role that gives up stops
-        // completing barriers, so the next wait below sees the flag
-        for (int t = 0; ok && t < ntiles; ++t, ++tg) {
-          const int b = tg & 1;
-          const uint32_t use = (uint32_t)(tg >> 1);
-          if (!mbar_wait(bars.tempty(b), (use & 1u) ^ 1u, kWaitLimitNs, abort_flag)) {
-            flag_timeout(abort_flag, dev_err);
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + b * kAccCols;
-          for (int kc = 0; kc < KC; ++kc, ++it) {
-            const int s = it % kStages;
-            const uint32_t round = (uint32_t)(it / kStages);
-            if (!mbar_wait(bars.full(s), round & 1u, kWaitLimitNs, abort_flag)) {
+          if (w >= work.n_items) break;
+          int64_t m0, j_begin;
+          const int ntiles = item_tiles(w, &m0, &j_begin);
+          // the query tiles: once the previous item's MMAs have read theirs (in
+          // the claimed-chunk form, once for the whole launch)
+          if (!chunked || a_loads == 0) {
+            if (a_loads > 0 && !mbar_wait(bars.aempty(), (uint32_t)((a_loads - 1) & 1), kWaitLimitNs, abort_flag)) {
               flag_timeout(abort_flag, dev_err);
-              ok = false;
               break;
             }
-            tc_fence_after();
-            // descriptors are built once per stage and advanced by adding the
-            // byte offset >> 4 to their start-address field (14 bits of
-            // addr >> 4; every shared address is below 256 KB, so the sum
-            // never carries out of the field): the MMA thread's issue loop is
-            // on the critical path of the N = 128 shape, which issues twice
-            // as many MMAs per step
-            const uint32_t b_base = sbase + L::kOffB + s * Sh::kStageBytes;
-            const uint64_t b_desc = sw128_kmajor_desc(b_base);
-            const uint64_t b_ext = sw32_kmajor_desc(b_base + Sh::kBChunkBytes);
-            const bool last = kc == KC - 1;  // the norms' K-extension rides with the last chunk
-#pragma unroll
+            mbar_arrive_expect_tx(bars.afull(), QT * (KC * kAChunkBytes + kAExtBytes));
             for (int q = 0; q < QT; ++q) {
-              if (q < q_first || q >= q_last) continue;
-              const uint32_t a_q = sbase + L::kOffA + q * L::kAQueryBytes;
-              const uint64_t a_desc = sw128_kmajor_desc(a_q) + (uint64_t)((kc * kAChunkBytes) >> 4);
-              const uint64_t a_ext = sw32_kmajor_desc(a_q + KC * kAChunkBytes);
-              const uint32_t d_q = d_tmem + q * kTileN;
-              if (Fmt::kExtFirst && last) mma_bf16(d_q, a_ext, b_ext, idesc_bf16_f32(kBM, kTileN), kc != 0 ? 1u : 0u);
-#pragma unroll
-              for (int kk = 0; kk < kMmaPerChunk; ++kk)  // K-steps of 32 bytes
-                Fmt::template mma<kTileN>(d_q, a_desc + (uint64_t)(2 * kk), b_desc + (uint64_t)(2 * kk),
-                                          (kc | kk) != 0 || (Fmt::kExtFirst && last) ? 1u : 0u);
-              if (!Fmt::kExtFirst && last) mma_bf16(d_q, a_ext, b_ext, idesc_bf16_f32(kBM, kTileN), 1u);
+              const uint32_t a = sbase + L::kOffA + q * L::kAQueryBytes;
+              const int32_t qrow = (int32_t)(m0 + q * kBM);
+              for (int kc = 0; kc < KC; ++kc) tma_load_2d(a + kc * kAChunkBytes, &tmap_q, kc * kBK, qrow, bars.afull());
+              tma_load_2d(a + KC * kAChunkBytes, &tmap_qe, 0, qrow, bars.afull());
             }
-            mma_commit(bars.empty(s));  // the producer may refill this stage
+            ++a_loads;
           }
-          if constexpr (!kStageSignalsTile) {
-            if (ok) mma_commit(bars.tfull(b));
+          bool ok = true;
+          const int warm = warm_tiles(i, w, ntiles).tiles;
+          for (int t = -warm; ok && t < ntiles && !*abort_flag; ++t) {
+            const int32_t row = (int32_t)(j_begin + (int64_t)(t < 0 ? t + warm : t) * kTileN);
+            for (int kc = 0; kc < KC; ++kc, ++it) {
+              const int s = it % kStages;
+              const uint32_t round = (uint32_t)(it / kStages);
+              if (!mbar_wait(bars.empty(s), (round & 1u) ^ 1u, kWaitLimitNs, abort_flag)) {
+                flag_timeout(abort_flag, dev_err);
+                ok = false;
+                break;
+              }
+              const uint32_t dst = sbase + L::kOffB + s * Sh::kStageBytes;
+              const bool last = kc == KC - 1;
+              mbar_arrive_expect_tx(bars.full(s), Sh::kBChunkBytes + (last ? Sh::kBExtBytes : 0u));
+              tma_load_2d(dst, &tmap_r, kc * kBK, row, bars.full(s));
+              if (last) tma_load_2d(dst + Sh::kBChunkBytes, &tmap_re, 0, row, bars.full(s));
+            }
           }
+          if (!ok || *abort_flag) break;
         }
-        tiles_done += ntiles;
-        if (!chunked) mma_commit(bars.aempty());  // the query tiles may be replaced once these MMAs are done
-        if (persistent) mbar_arrive(bars.iempty(i & 1));
+        // every load issued must land before the CTA may exit
+        const uint32_t never = 0;
+        if (a_loads > 0) mbar_wait(bars.afull(), (uint32_t)((a_loads - 1) & 1), kWaitLimitNs, &never);
+        for (int s = 0; s < kStages; ++s) {
+          const int issued = it / kStages + (s < it % kStages ? 1 : 0);
+          if (issued > 0) mbar_wait(bars.full(s), (uint32_t)((issued - 1) & 1), kWaitLimitNs, &never);
+        }
       }
-      // all MMAs issued by this thread must finish before TMEM is released
-      const uint32_t never = 0;
-      mma_commit(bars.drain());
-      mbar_wait(bars.drain(), 0, kWaitLimitNs, &never);
-      if (stats && warp == 1) {
-        atomicAdd(stats + 0, (unsigned long long)(clock64() - clk0));
-        atomicAdd(stats + 1, (unsigned long long)(globaltimer_ns() - ns0));
-        atomicAdd(stats + 2, (unsigned long long)tiles_done);
-        atomicAdd(stats + 3, 1ull);
-      }
-    }
-  } else {
-    // ------------------------------------------------------------- epilogue
-    const int quarter = warp & 3;          // this warp may read TMEM lanes [32*quarter, 32*quarter+32)
-    const int half = (warp - 2) >> 2;      // QT = 1: its column half of every tile; QT = 2: its query tile
-    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-    int tg = 0;
-    // the tiles of one work item into the lists of `e`; false if a wait ran out
-    auto scan_tiles = [&](auto& e, int ntiles, int64_t col_base) -> bool {
-      for (int t = 0; t < ntiles; ++t, ++tg) {
-        const int b = tg & 1;
-        bool done;
-        if constexpr (kStageSignalsTile) {
-          const int itl = tg * KC + KC - 1;  // the tile's last K-chunk
-          done = mbar_wait(bars.empty(itl % kStages), (uint32_t)(itl / kStages) & 1u, kWaitLimitNs, abort_flag);
-        } else {
-          done = mbar_wait(bars.tfull(b), (uint32_t)(tg >> 1) & 1u, kWaitLimitNs, abort_flag);
-        }
-        if (!done) {
-          flag_timeout(abort_flag, dev_err);
-          return false;
-        }
-        tc_fence_after();
-        // rounds of 64 columns; the accumulator goes back as soon as the last
-        // round is in registers
-        const uint32_t taddr = tmem_base + lane_addr + b * kAccCols + half * kEpiCols;
-        const int64_t col0 = col_base + (int64_t)t * kTileN;
-#pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-          uint32_t v0[32], v1[32], mn0, mn1;
-          tmem_ld_min_32x32b_x32(taddr + 64 * r, v0, mn0);
-          tmem_ld_min_32x32b_x32(taddr + 64 * r + 32, v1, mn1);
-          tmem_ld_wait(v0, mn0);
-          reg_fence(v1);
-          asm volatile("" : "+r"(mn1));
-          if (r == kRounds - 1) {
-            // every lane's loads are complete (waited above); one arrival
-            // per warp after a warp barrier (256 single-thread arrivals on
-            // one barrier, while the MMAs read their operands from shared
-            // memory, delayed the accumulator's return by ~100 cycles a step)
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bars.tempty(b));
-          }
-          e.group(v0, mn0, col0 + 64 * r);
-          e.group(v1, mn1, col0 + 64 * r + 32);
-        }
-        e.tile_end();
-      }
-      return true;
-    };
-    if constexpr (Claim) {
-      {
-        // claimed-chunk form: one query-tile group and one set of lists for
-        // the whole launch (list = this CTA's rank in the group's CTAs x the
-        // lists per CTA), written once every claimed chunk is scanned
-        const int rank = (int)(blockIdx.x % (unsigned)work.group);
-        const int64_t row =
-            (int64_t)(blockIdx.x / (unsigned)work.group) * (kBM * QT) + (QT == 2 ? half * kBM : 0) + quarter * 32 + lane;
-        const int64_t c_off = QT == 2 ? 0 : half * kEpiCols;
-        const int list = QT == 2 ? rank : rank * kEpiPerQuarter + half;
-        const bool active = row < m;
-        Epilogue epi(out, list, row, active, c_off, smem + L::kOffList, warp - 2);
-        for (int i = 0;; ++i) {
+    } else if (issuer) {
+      if (lane == 0) {
+        // --------------------------------------------------------- MMA issuers
+        const int q_first = kIssuers == QT ? (warp == 1 ? 0 : 1) : 0;  // this thread's query tiles
+        const int q_last = kIssuers == QT ? q_first + 1 : QT;
+        const long long clk0 = clock64();
+        const uint64_t ns0 = globaltimer_ns();
+        int it = 0;       // reference K-chunks consumed
+        int tg = 0;       // tiles over all items (accumulator use)
+        int64_t tiles_done = 0;
+        bool ok = true;
+        for (int i = 0; ok; ++i) {
           int64_t w;
           if (!consume_item(i, &w)) {
             flag_timeout(abort_flag, dev_err);
@@ -978,66 +864,334 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
           }
           if (w >= work.n_items) break;
           int64_t m0, j_begin;
-          const int ntiles = item_tiles(w, &m0, &j_begin);
-          if (!scan_tiles(epi, ntiles, j_begin + c_off)) break;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bars.iempty(i & 1));
+          int ntiles = item_tiles(w, &m0, &j_begin);
+          ntiles += warm_tiles(i, w, ntiles).tiles;
+          if ((!chunked || i == 0) && !mbar_wait(bars.afull(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
+            flag_timeout(abort_flag, dev_err);
+            break;
+          }
+          tc_fence_after();
+          // no abort-flag read per tile here: shared-memory loads are slow on
+          // this thread while the MMAs stream their operands (the per-tile
+          // read cost 2% of the FP8 pass), and a role that gives up stops
+          // completing barriers, so the next wait below sees the flag
+          for (int t = 0; ok && t < ntiles; ++t, ++tg) {
+            const int b = tg & 1;
+            const uint32_t use = (uint32_t)(tg >> 1);
+            if (!mbar_wait(bars.tempty(b), (use & 1u) ^ 1u, kWaitLimitNs, abort_flag)) {
+              flag_timeout(abort_flag, dev_err);
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + b * kAccCols;
+            for (int kc = 0; kc < KC; ++kc, ++it) {
+              const int s = it % kStages;
+              const uint32_t round = (uint32_t)(it / kStages);
+              if (!mbar_wait(bars.full(s), round & 1u, kWaitLimitNs, abort_flag)) {
+                flag_timeout(abort_flag, dev_err);
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              // descriptors are built once per stage and advanced by adding the
+              // byte offset >> 4 to their start-address field (14 bits of
+              // addr >> 4; every shared address is below 256 KB, so the sum
+              // never carries out of the field): the MMA thread's issue loop is
+              // on the critical path of the N = 128 shape, which issues twice
+              // as many MMAs per step
+              const uint32_t b_base = sbase + L::kOffB + s * Sh::kStageBytes;
+              const uint64_t b_desc = sw128_kmajor_desc(b_base);
+              const uint64_t b_ext = sw32_kmajor_desc(b_base + Sh::kBChunkBytes);
+              const bool last = kc == KC - 1;  // the norms' K-extension rides with the last chunk
+  #pragma unroll
+              for (int q = 0; q < QT; ++q) {
+                if (q < q_first || q >= q_last) continue;
+                const uint32_t a_q = sbase + L::kOffA + q * L::kAQueryBytes;
+                const uint64_t a_desc = sw128_kmajor_desc(a_q) + (uint64_t)((kc * kAChunkBytes) >> 4);
+                const uint64_t a_ext = sw32_kmajor_desc(a_q + KC * kAChunkBytes);
+                const uint32_t d_q = d_tmem + q * kTileN;
+                if (Fmt::kExtFirst && last) mma_bf16(d_q, a_ext, b_ext, idesc_bf16_f32(kBM, kTileN), kc != 0 ? 1u : 0u);
+  #pragma unroll
+                for (int kk = 0; kk < kMmaPerChunk; ++kk)  // K-steps of 32 bytes
+                  Fmt::template mma<kTileN>(d_q, a_desc + (uint64_t)(2 * kk), b_desc + (uint64_t)(2 * kk),
+                                            (kc | kk) != 0 || (Fmt::kExtFirst && last) ? 1u : 0u);
+                if (!Fmt::kExtFirst && last) mma_bf16(d_q, a_ext, b_ext, idesc_bf16_f32(kBM, kTileN), 1u);
+              }
+              mma_commit(bars.empty(s));  // the producer may refill this stage
+            }
+          }
+          tiles_done += ntiles;
+          if (!chunked) mma_commit(bars.aempty());  // the query tiles may be replaced once these MMAs are done
+          if (persistent) mbar_arrive(bars.iempty(i & 1));
         }
-        epi.finish();
+        // all MMAs issued by this thread must finish before TMEM is released
+        const uint32_t never = 0;
+        mma_commit(bars.drain());
+        mbar_wait(bars.drain(), 0, kWaitLimitNs, &never);
+        if (stats && warp == 1) {
+          atomicAdd(stats + 0, (unsigned long long)(clock64() - clk0));
+          atomicAdd(stats + 1, (unsigned long long)(globaltimer_ns() - ns0));
+          atomicAdd(stats + 2, (unsigned long long)tiles_done);
+          atomicAdd(stats + 3, 1ull);
+        }
       }
     }
-    for (int i = 0; !chunked; ++i) {
+  } else if (warp < kInsWarp0) {
+    // ------------------------------------------------------------- epilogue
+    const int quarter = warp & 3;               // this warp may read TMEM lanes [32*quarter, 32*quarter+32)
+    const int half = (warp - kEpiWarp0) >> 2;   // QT = 1: its column half of every tile; QT = 2: its query tile
+    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    int tg = 0;
+    const uint32_t taddr0 = tmem_base + lane_addr + half * kEpiCols;
+    // tile tg's MMAs are done (one answer for the warp: its lanes stay
+    // together when a wait runs out)
+    auto wait_tile = [&]() -> bool {
+      const int itl = tg * KC + KC - 1;  // the tile's last K-chunk
+      const bool done = __all_sync(
+          0xffffffffu,
+          mbar_wait(bars.empty(itl % kStages), (uint32_t)(itl / kStages) & 1u, kWaitLimitNs, abort_flag));
+      if (!done) flag_timeout(abort_flag, dev_err);
+      tc_fence_after();
+      return done;
+    };
+    // the accumulator goes back: every lane's loads are complete; one arrival
+    // per warp after a warp barrier (256 single-thread arrivals on one barrier,
+    // while the MMAs read their operands from shared memory, delayed the
+    // accumulator's return by ~100 cycles a step)
+    auto release_tile = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bars.tempty(tg & 1));
+    };
+    // the tiles of one work item into the lists of `e`; false if a wait ran out
+    auto scan_tiles = [&](auto& e, int ntiles, int64_t col_base) -> bool {
+      for (int t = 0; t < ntiles; ++t, ++tg) {
+        if (!wait_tile()) return false;
+        // rounds of 64 columns; the accumulator goes back as soon as the last
+        // round is in registers.  With inserter warps the rounds are one copy of
+        // the code (see merge_rows on the instruction cache).
+        const uint32_t taddr = taddr0 + (tg & 1) * kAccCols;
+        const int64_t col0 = col_base + (int64_t)t * kTileN;
+#pragma unroll (kAsync ? 1 : kRounds)
+        for (int r = 0; r < kRounds; ++r) {
+          uint32_t v0[32], v1[32], mn0, mn1;
+          tmem_ld_min_32x32b_x32(taddr + 64 * r, v0, mn0);
+          tmem_ld_min_32x32b_x32(taddr + 64 * r + 32, v1, mn1);
+          tmem_ld_wait(v0, mn0);
+          reg_fence(v1);
+          asm volatile("" : "+r"(mn1));
+          if (r == kRounds - 1) release_tile();
+          e.round(v0, mn0, v1, mn1, col0 + 64 * r);
+        }
+      }
+      return true;
+    };
+    // one work item after another (or claimed chunk after claimed chunk)
+    const int64_t c_off = QT == 2 ? 0 : half * kEpiCols;  // this warp's first column within a tile
+    const HandOver ho{sbase + L::kOffList};
+    const uint32_t t = (uint32_t)(half * kBM + quarter * 32 + lane);
+    Collector e;
+    if constexpr (kAsync) {
+      e.ho = ho;
+      e.w = (uint32_t)(warp - kEpiWarp0);
+      e.lane = (uint32_t)lane;
+      e.lim_at = ho.lim(QT == 2 ? t : t & 127u);
+      e.cap = (uint32_t)out.entries;
+      e.mine = out.work + max(*work_slot, 0) * tc_work_bytes(out.entries) + (int64_t)t * 2 * out.entries * kTcEntryBytes;
+      e.start = e.mine;
+      e.soft = (uint32_t)min(Epilogue::KMAX > 0 ? 8 : 32, out.entries - 8);
+      e.abort_flag = abort_flag;
+      e.dev_err = dev_err;
+    }
+    int i = 0;
+    for (;; ++i) {
       int64_t w;
-      if (!consume_item(i, &w)) {
+      if (!__all_sync(0xffffffffu, consume_item(i, &w))) {
         flag_timeout(abort_flag, dev_err);
         break;
       }
       if (w >= work.n_items) break;
       int64_t m0, j_begin;
       const int ntiles = item_tiles(w, &m0, &j_begin);
-      const int64_t y = w / work.T;
-      const int64_t row = m0 + (QT == 2 ? half * kBM : 0) + quarter * 32 + lane;
-      const int64_t c_off = QT == 2 ? 0 : half * kEpiCols;  // this warp's first column within a tile
-      const int list = QT == 2 ? (int)y : (int)y * kEpiPerQuarter + half;
-      const bool active = row < m;
-      Epilogue epi(out, list, row, active, j_begin + c_off, smem + L::kOffList, warp - 2);
-      // the previous split of these rows, if it has finished: start from its
-      // list.  Its flag says 2 when every earlier split of the rows was
-      // carried into it; a warp that cannot say the same of this item marks
-      // the item's slot (cleared by the thread that publishes the slot's
-      // previous item before that item's slot is released)
-      if (Epilogue::kSeeds && out.done != nullptr) {
-        const uint32_t prev = y > 0 && ntiles > 0 ? ld_acquire_gpu(out.done + (w - out.T)) : 0u;
-        if (prev != 0u)
-          epi.seed(out.lists + ((int64_t)(list - out.lists_per_split) * out.stride + (active ? row : 0)) * out.K1);
-        if (lane == 0 && y > 0 && prev != 2u) chain_broken[i & 1] = 1u;
-      }
-      const bool ok = scan_tiles(epi, ntiles, j_begin + c_off);
-      epi.finish();
-      if (Epilogue::kSeeds && out.done != nullptr) {
-        // this item's lists are complete once every epilogue warp has written
-        // its rows' lists; one thread then marks the item done: 2 if its
-        // lists hold every earlier split's keys (each split of the rows
-        // started from the one before), else 1 (if the wait runs out nothing
-        // is marked and a later split simply starts empty)
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars.lists_done());
-        if (warp == 2 && lane == 0 && ok &&
-            mbar_wait(bars.lists_done(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
-          // the item index again (from its slot, which the producer refills
-          // only after this warp's release below), not kept live across the tiles
-          const int64_t wd = persistent ? item_slot[i & 1] : (int64_t)blockIdx.x;
-          const uint32_t flag = chain_broken[i & 1] != 0u ? 1u : 2u;
-          chain_broken[i & 1] = 0u;
-          __threadfence();
-          st_release_gpu(out.done + wd, flag);
+      if constexpr (kAsync) {
+        if (!Claim || i == 0) {
+          const WarmUp wu = warm_tiles(i, w, ntiles);
+          int32_t most = wu.tiles > 0 ? INT32_MIN : INT32_MAX;
+          bool ok = true;
+          for (int u = 0; u < wu.tiles; ++u, ++tg) {
+            if (!(ok = wait_tile())) break;
+            const uint32_t taddr = taddr0 + (tg & 1) * kAccCols;
+            int32_t least = INT32_MAX;
+#pragma unroll 1
+            for (int c = 0; c < kEpiCols; c += 32) {
+              uint32_t v[32], mn;
+              tmem_ld_min_32x32b_x32(taddr + c, v, mn);
+              tmem_ld_wait(v, mn);
+              if (wu.fine) most = max(most, (int32_t)mn);
+              least = min(least, (int32_t)mn);
+            }
+            release_tile();
+            if (!wu.fine) most = max(most, least);
+          }
+          if (!ok) break;
+          st_shared_u32(ho.warm(t), (uint32_t)most);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bars.warmed());
+          if (!__all_sync(0xffffffffu, mbar_wait(bars.limits(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag))) {
+            flag_timeout(abort_flag, dev_err);
+            break;
+          }
+          e.read_limit();
         }
+        if (!scan_tiles(e, ntiles, j_begin + c_off)) break;
+        if (!Claim) {
+          if (!e.hand_over(true)) break;
+          if (lane == 0) mbar_arrive(bars.queued());
+        }
+      } else {
+        const int64_t row = m0 + (QT == 2 ? half * kBM : 0) + quarter * 32 + lane;
+        Epilogue epi(out, row, row < m, j_begin + c_off);
+        const bool ok = scan_tiles(epi, ntiles, j_begin + c_off);
+        epi.finish();
+        if (!ok) break;
       }
-      if (!ok) break;
       if (persistent) {
         __syncwarp();
         if (lane == 0) mbar_arrive(bars.iempty(i & 1));
+      }
+    }
+    if constexpr (kAsync && Claim) {
+      if (i == 0) {  // no chunk was left for this CTA
+        st_shared_u32(ho.warm(t), (uint32_t)INT32_MAX);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.warmed());
+      }
+      if (e.hand_over(true) && lane == 0) mbar_arrive(bars.queued());
+    }
+  } else {
+    if constexpr (kAsync) {
+      // ----------------------------------------------------------- inserters
+      if constexpr (kWideLists<Epilogue, QT>) reg_alloc<kRegsInserter>();
+      const uint32_t quarter = (uint32_t)(warp & 3);
+      Inserter<Epilogue::KMAX, QT> ins;
+      ins.ho = HandOver{sbase + L::kOffList};
+      ins.quarter = quarter;
+      ins.lane = (uint32_t)lane;
+      ins.K1 = out.K1;
+      ins.cap = out.entries;
+      ins.cand = out.work + max(*work_slot, 0) * tc_work_bytes(out.entries);
+      const bool share = out.bound_per_tile && out.row_thr != nullptr;
+      // one list per row and split (claimed chunks: per row and CTA of the group)
+      for (int i = 0; !Claim || i == 0; ++i) {
+        int64_t w = 0;
+        if (!Claim) {
+          if (!__all_sync(0xffffffffu, consume_item(i, &w))) {
+            flag_timeout(abort_flag, dev_err);
+            break;
+          }
+          if (w >= work.n_items) break;
+        }
+        int64_t m0, j_begin;
+        const int ntiles = item_tiles(w, &m0, &j_begin);
+        const int64_t y = Claim ? (int64_t)(blockIdx.x % (unsigned)work.group) : w / work.T;
+        // the previous split of these rows, if it has finished: start from its
+        // list.  Its flag says 2 when every earlier split of the rows was
+        // carried into it; a warp that cannot say the same of this item marks
+        // the item's slot (cleared by the thread that publishes the slot's
+        // previous item before that item's slot is released)
+        const bool chain = !Claim && out.done != nullptr;
+        const uint32_t prev = chain && y > 0 && ntiles > 0 ? ld_acquire_gpu(out.done + (w - out.T)) : 0u;
+        const bool carried = __all_sync(0xffffffffu, prev != 0u);
+        if (chain && y > 0 && !__all_sync(0xffffffffu, prev == 2u) && lane == 0) chain_broken[i & 1] = 1u;
+        bool ok = __all_sync(0xffffffffu, mbar_wait(bars.warmed(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag));
+        if (!ok) flag_timeout(abort_flag, dev_err);  // (the lists are written all the same, empty)
+#pragma unroll
+        for (int q = 0; q < QT; ++q) {
+          const int64_t row = m0 + q * kBM + quarter * 32 + lane;
+          const bool active = row < m;
+          const int64_t first = m0 + q * kBM + quarter * 32;
+          ins.list[q] = out.lists + (y * out.stride + first) * out.K1;
+          ins.seed[q] = carried ? ins.list[q] - out.stride * out.K1 : nullptr;
+          ins.listed[q] = 0u;
+          ins.kth[q] = INT32_MAX;
+          if constexpr (ins.kRegs) {
+            ins.L[q].init(out.K1);
+            if (carried && active) ins.L[q].seed(ins.seed[q] + lane * out.K1, out.K1);
+            ins.kth[q] = ins.L[q].worst();
+          } else if (carried && active) {
+            const uint64_t k = __ldcg(ins.seed[q] + lane * out.K1 + out.K1 - 1);
+            if (k != kEmptyKey) ins.kth[q] = dist_bits(key_dist(k));
+          }
+          ins.rthr[q] = active && out.row_thr ? out.row_thr + row : nullptr;
+          const uint32_t t = (uint32_t)(q * kBM) + quarter * 32 + (uint32_t)lane;
+          int32_t bound = (int32_t)ld_shared_u32(ins.ho.warm(t));
+          if (QT == 1) bound = max(bound, (int32_t)ld_shared_u32(ins.ho.warm(t + kBM)));
+          ins.shared[q] = ins.rthr[q] ? __ldcg(ins.rthr[q]) : kNoBound;
+          if (bound < ins.shared[q]) {
+            ins.shared[q] = bound;
+            if (share && ins.rthr[q]) atomicMin(ins.rthr[q], bound);
+          }
+          ins.lim[q] = active ? 0 : INT32_MIN;
+          ins.post_limit(q);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.limits());
+        const uint64_t t0 = globaltimer_ns();
+        uint32_t nap = 100;  // ns between polls: longer while nothing comes (polls every 100 ns cost the FP8 pass 5%)
+        for (uint32_t it = 0; ok; ++it) {
+          const bool last = __all_sync(0xffffffffu, mbar_test(bars.queued(), (uint32_t)(i & 1)));
+          bool took = false;
+          if constexpr (QT == 1) {  // one copy of the code
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) took |= ins.take(h, share);
+          } else {
+            took = ins.take(0, share);
+            took |= ins.take(1, share);
+          }
+          if (share) ins.read_bounds();
+          if (took) {
+            nap = 100;
+            continue;
+          }
+          if (last) break;
+          const bool over = (it & 255u) == 0 && globaltimer_ns() - t0 > kItemLimitNs;
+          if (__any_sync(0xffffffffu, *abort_flag != 0u || over)) {
+            flag_timeout(abort_flag, dev_err);
+            ok = false;
+            break;
+          }
+          __nanosleep(nap);
+          nap = min(2 * nap, 1600u);
+        }
+#pragma unroll
+        for (int q = 0; q < QT; ++q) {
+          const int64_t left = m - (m0 + q * kBM + quarter * 32);
+          ins.finish(q, (uint32_t)max(int64_t(0), min(left, int64_t(32))));
+          if (ins.rthr[q] && !out.bound_per_tile && ins.kth[q] < ins.shared[q]) atomicMin(ins.rthr[q], ins.kth[q]);
+        }
+        if (chain) {
+          // the item's lists are complete once every inserter warp has written
+          // its rows' lists; one thread then marks the item done: 2 if its
+          // lists hold every earlier split's keys (each split of the rows
+          // started from the one before), else 1 (if the wait runs out nothing
+          // is marked and a later split simply starts empty)
+          __threadfence();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bars.lists_done());
+          if (warp == kInsWarp0 && lane == 0 && ok &&
+              mbar_wait(bars.lists_done(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
+            const uint32_t flag = chain_broken[i & 1] != 0u ? 1u : 2u;
+            chain_broken[i & 1] = 0u;
+            __threadfence();
+            st_release_gpu(out.done + w, flag);
+          }
+        }
+        if (!ok) break;
+        if (persistent && !Claim) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bars.iempty(i & 1));
+        }
       }
     }
   }
@@ -1047,6 +1201,9 @@ __global__ void __launch_bounds__(threads_for(Epilogue::kWarpsPerQuarter, QT), 1
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
+  }
+  if constexpr (kAsync) {
+    if (threadIdx.x == 0) release_slot(out, *work_slot);
   }
 }
 
@@ -1144,7 +1301,6 @@ cudaError_t launch_scan(const CUtensorMap& tr, const CUtensorMap& tre, const voi
   ScanOut o = out;
   o.done = splits > 1 ? sched.done : nullptr;
   o.T = work.T;
-  o.lists_per_split = QT == 2 ? 1 : Epilogue::kWarpsPerQuarter;
   int64_t grid = work.queue ? std::min<int64_t>(work.n_items, sched.persistent_ctas) : work.n_items;
   if (sched.group > 0) {
     // the claimed-chunk form: `splits` is the CTAs per query-tile group (the
@@ -1157,17 +1313,25 @@ cudaError_t launch_scan(const CUtensorMap& tr, const CUtensorMap& tre, const voi
     grid = work.T * sched.group;
   }
   if (work.n_items > (int64_t)INT32_MAX || grid > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
+  if (Epilogue::kInserterWarps > 0) {
+    if (sched.work == nullptr || sched.work_slots < 1 || sched.entries < kTcMinEntries || (grid > sched.work_slots && sched.slot_used == nullptr))
+      return cudaErrorInvalidValue;
+    o.work = sched.work;
+    o.work_slots = sched.work_slots;
+    o.entries = sched.entries;
+    o.slot_used = grid > sched.work_slots ? sched.slot_used : nullptr;
+  }
   if constexpr (QT == 1 && Epilogue::kClaimsChunks) {
     if (work.group > 0) {
       tc_scan_kernel<Fmt, Epilogue, QT, true>
-          <<<(unsigned)grid, threads_for(Epilogue::kWarpsPerQuarter, QT), LayoutOf<Fmt, Epilogue, QT>::kSmemBytes,
+          <<<(unsigned)grid, kThreadsOf<Epilogue>, LayoutOf<Fmt, Epilogue, QT>::kSmemBytes,
              s>>>(tq, tqe, tr, tre, m, n_ref, work, o, dev_err, stats);
       return cudaGetLastError();
     }
   }
   if (work.group > 0) return cudaErrorInvalidValue;
   tc_scan_kernel<Fmt, Epilogue, QT, false>
-      <<<(unsigned)grid, threads_for(Epilogue::kWarpsPerQuarter, QT), LayoutOf<Fmt, Epilogue, QT>::kSmemBytes, s>>>(
+      <<<(unsigned)grid, kThreadsOf<Epilogue>, LayoutOf<Fmt, Epilogue, QT>::kSmemBytes, s>>>(
           tq, tqe, tr, tre, m, n_ref, work, o, dev_err, stats);
   return cudaGetLastError();
 }
@@ -1177,7 +1341,9 @@ cudaError_t prepare_kernel() {
   cudaFuncAttributes a;
   cudaError_t e = cudaFuncGetAttributes(&a, tc_scan_kernel<Fmt, Epilogue, QT, Claim>);
   if (e != cudaSuccess) return e;
-  if (a.numRegs > max_regs_for(Epilogue::kWarpsPerQuarter, QT)) return cudaErrorInvalidKernelImage;
+  if (a.numRegs > kMaxRegsOf<Epilogue>) return cudaErrorInvalidKernelImage;
+  // the register split counts on what the launch has
+  if (kWideLists<Epilogue, QT> && a.numRegs != kRegsLaunch) return cudaErrorInvalidKernelImage;
   return cudaFuncSetAttribute(tc_scan_kernel<Fmt, Epilogue, QT, Claim>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)LayoutOf<Fmt, Epilogue, QT>::kSmemBytes);
 }
@@ -1191,14 +1357,17 @@ cudaError_t prepare_one() {
   return e;
 }
 
-// One list kind's kernel for the tile shape the schedule asks for (two query
-// tiles per CTA only where the epilogue has two warps per lane quarter).
+// Lists of 33..64 keys run with one query tile per CTA only.
+template <class Epilogue>
+constexpr bool kTwoQueryTiles = Epilogue::KMAX <= kTcCoarseRegListMax;
+
+// One list kind's kernel for the tile shape the schedule asks for.
 template <class Fmt, class Epilogue>
 cudaError_t launch_shape(const TcTensorMaps& maps, bool sorted_copy, const void* qop, const __nv_bfloat16* qext,
                          int64_t m, int64_t m_pad, int64_t n_ref, int splits, int64_t split_len, const ScanOut& out,
                          uint32_t* dev_err, unsigned long long* stats, const TcSched& sched, cudaStream_t s) {
   constexpr bool coarse = Fmt::kChunks == 1;
-  if constexpr (Epilogue::kWarpsPerQuarter == 2) {
+  if constexpr (kTwoQueryTiles<Epilogue>) {
     if (sched.qt == 2) {
       const CUtensorMap& tr = coarse ? maps.f8_h : (sorted_copy ? maps.sref_h : maps.ref_h);
       const CUtensorMap& tre = coarse ? maps.f8_ext_h : (sorted_copy ? maps.sref_ext_h : maps.ref_ext_h);
@@ -1216,41 +1385,35 @@ cudaError_t launch_shape(const TcTensorMaps& maps, bool sorted_copy, const void*
 template <class Fmt, class Epilogue>
 cudaError_t prepare_both() {
   cudaError_t e = prepare_one<Fmt, Epilogue, 1>();
-  if constexpr (Epilogue::kWarpsPerQuarter == 2) {
+  if constexpr (kTwoQueryTiles<Epilogue>) {
     if (e == cudaSuccess) e = prepare_one<Fmt, Epilogue, 2>();
   }
   return e;
 }
 
-// The kNN scan with the list kind for K1 and the split length.
+// The kNN scan with the instantiation for K1.
 template <class Fmt>
 cudaError_t launch_lists(const TcTensorMaps& maps, bool sorted_copy, const void* qop, const __nv_bfloat16* qext,
                          int64_t m, int64_t m_pad, int64_t n_ref, int splits, int64_t split_len, int K1,
                          const ScanOut& out, uint32_t* dev_err, unsigned long long* stats, const TcSched& sched,
                          cudaStream_t s) {
-  switch (tc_list_kind(K1, split_len, Fmt::kChunks == 1)) {
-    case ListKind::Reg16:
+  switch (tc_list_max(K1)) {
+    case kTcRegListMax:
       return launch_shape<Fmt, KnnEpilogue<kTcRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits,
                                                            split_len, out, dev_err, stats, sched, s);
-    case ListKind::Reg24:
+    case kTcMidRegListMax:
       return launch_shape<Fmt, KnnEpilogue<kTcMidRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits,
                                                               split_len, out, dev_err, stats, sched, s);
-    case ListKind::Reg32:
+    case kTcCoarseRegListMax:
       return launch_shape<Fmt, KnnEpilogue<kTcCoarseRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref,
                                                                  splits, split_len, out, dev_err, stats, sched, s);
-    case ListKind::Smem64:
-      return launch_shape<Fmt, KnnSmemEpilogue<kTcWideRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref,
-                                                                   splits, split_len, out, dev_err, stats, sched, s);
-    case ListKind::Reg64:
-      if constexpr (Fmt::kChunks == 2)
-        return launch_shape<Fmt, KnnEpilogue<kTcWideRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref,
-                                                                 splits, split_len, out, dev_err, stats, sched, s);
-      return cudaErrorInvalidValue;
-    case ListKind::Heap:
-      break;
+    case kTcWideRegListMax:
+      return launch_shape<Fmt, KnnEpilogue<kTcWideRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits,
+                                                               split_len, out, dev_err, stats, sched, s);
+    default:
+      return launch_shape<Fmt, KnnEpilogue<0>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits, split_len, out,
+                                               dev_err, stats, sched, s);
   }
-  return launch_shape<Fmt, KnnEpilogue<0>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits, split_len, out,
-                                           dev_err, stats, sched, s);
 }
 
 }  // namespace
@@ -1260,13 +1423,12 @@ cudaError_t prepare_tc_kernels() {
   if (e == cudaSuccess) e = prepare_both<FmtBf16, KnnEpilogue<kTcMidRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnEpilogue<kTcMidRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtBf16, KnnEpilogue<kTcCoarseRegListMax>>();
-  if (e == cudaSuccess) e = prepare_both<FmtBf16, KnnSmemEpilogue<kTcWideRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtBf16, KnnEpilogue<kTcWideRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtBf16, KnnEpilogue<0>>();
   if (e == cudaSuccess) e = prepare_both<FmtBf16, NbnnEpilogue>();
   if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnEpilogue<kTcRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnEpilogue<kTcCoarseRegListMax>>();
-  if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnSmemEpilogue<kTcWideRegListMax>>();
+  if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnEpilogue<kTcWideRegListMax>>();
   if (e == cudaSuccess) e = prepare_both<FmtE4m3, KnnEpilogue<0>>();
   return e;
 }

@@ -16,42 +16,30 @@ constexpr int kTcRefTile = 256;
 // tiles, and concurrently running CTAs share them through L2.
 constexpr int kTcQueryTile = 128;
 static_assert(kQueryPad % kTcQueryTile == 0, "query padding must cover whole tiles");
-// Lists of the k+1 (or shortlist) nearest per query row: up to 16 entries a
-// 16-entry register list (the fewest registers), up to 24 a 24-entry one (a
-// narrower insertion network than 32), up to 32 a 32-entry one, up
-// to 64 a 64-entry list in shared memory with warp-cooperative inserts (in
-// registers for an exact scan of long splits), longer ones a heap in global
-// memory.
+// Lists of the k+1 (or shortlist) nearest per query row, by the longest list a
+// kernel instantiation takes; longer ones (up to LNBNN_MAX_K + 1) share one
+// instantiation.
 constexpr int kTcRegListMax = 16;
 constexpr int kTcMidRegListMax = 24;
 constexpr int kTcCoarseRegListMax = 32;
 constexpr int kTcWideRegListMax = 64;
-// Epilogue warps per TMEM lane quarter.  Each owns a column slice of every
-// tile and keeps its own top-K1 list per query row, so one reference split
-// yields this many sorted lists per row (merged afterwards).  Two, except for
-// the 64-entry register lists, which need one warp per quarter (all 256
-// columns of a tile) to have the registers.
-// With two query tiles per CTA (qt = 2) each epilogue warp takes all 128
-// columns of its own query tile's block, so a split yields one list per row.
-inline int tc_lists_per_split(int K1, int qt = 1) {
-  return qt == 2 || (K1 > kTcCoarseRegListMax && K1 <= kTcWideRegListMax) ? 1 : 2;
-}
+// Candidate entries (eight neighbouring columns, some below the row's limit) an
+// epilogue thread collects before they must be merged: the last eight places
+// are for the 64 columns it tests at a time.  One CTA has two such buffers for
+// each of its 256 epilogue threads.
+constexpr int kTcEntryBytes = 64;  // eight values, the first one's column; room for eight (column, value) pairs
+constexpr int kTcMinEntries = 10;
+__host__ __device__ constexpr int tc_entries(int K1) { return (K1 <= 64 ? 16 : 48) + 8; }
+__host__ __device__ constexpr int64_t tc_work_bytes(int entries) { return (int64_t)256 * 2 * entries * kTcEntryBytes; }
 
-// Longest reference split for which the exact scan keeps 33..64-entry lists
-// in shared memory rather than registers (shared-memory lists leave room for
-// a two-stage ring only; measured on the 256-class data at k = 50, shared
-// memory is faster while a split holds up to 5.76M references, registers at
-// 11.52M).
-constexpr int64_t kSmemListMaxRefs = int64_t(8) << 20;
-
-// Where a scan keeps its per-row lists of K1 keys.
-enum class ListKind { Reg16, Reg24, Reg32, Smem64, Reg64, Heap };
-inline ListKind tc_list_kind(int K1, int64_t split_len, bool coarse) {
-  if (K1 <= kTcRegListMax) return ListKind::Reg16;
-  if (K1 <= kTcMidRegListMax) return ListKind::Reg24;
-  if (K1 <= kTcCoarseRegListMax) return ListKind::Reg32;
-  if (K1 <= kTcWideRegListMax) return coarse || split_len <= kSmemListMaxRefs ? ListKind::Smem64 : ListKind::Reg64;
-  return ListKind::Heap;
+// The kernel instantiation for lists of K1 keys: the longest list it takes, 0
+// for the longest.
+inline int tc_list_max(int K1) {
+  return K1 <= kTcRegListMax         ? kTcRegListMax
+         : K1 <= kTcMidRegListMax    ? kTcMidRegListMax
+         : K1 <= kTcCoarseRegListMax ? kTcCoarseRegListMax
+         : K1 <= kTcWideRegListMax   ? kTcWideRegListMax
+                                     : 0;
 }
 
 // TMA descriptors over an index's BF16 reference operands (caller's row order
@@ -85,6 +73,13 @@ struct TcSched {
   // per CTA lists per query row.  kNN register lists and heaps only; never
   // with `done`.
   int group = 0;
+  // kNN: candidate buffers of the lists in progress, tc_work_bytes(entries)
+  // each: as many as the launch has CTAs, or else (with slot_used, that many
+  // words zeroed before the launch) one per SM, which the CTAs take in turn.
+  char* work = nullptr;
+  int64_t work_slots = 0;
+  int entries = 0;
+  uint32_t* slot_used = nullptr;
 };
 
 // Split-N schedule of one scan launch over T query-tile groups (qt 128-row
@@ -105,10 +100,13 @@ struct SplitModel {
 
 // Largest split count considered for T query-tile groups: at most four waves
 // of CTAs (so workspace sizes do not depend on the fitted model), at least
-// 4,096 references per split, at most max_splits.
+// 512 references per split, at most max_splits.  (A split of a few tiles is
+// bound by filling its lists: 2,000 queries against 5,000 references, k = 10,
+// took 173 us in all with one split and 104 us with seven.)
+constexpr int64_t kMinSplitRefs = 512;
 inline int64_t max_splits_for(int64_t T, int64_t n_ref, int sm_count, int64_t max_splits) {
   int64_t hi = (4 * (int64_t)sm_count + T - 1) / T;
-  hi = std::min<int64_t>(hi, std::max<int64_t>(1, n_ref / 4096));
+  hi = std::min<int64_t>(hi, std::max<int64_t>(1, n_ref / kMinSplitRefs));
   return std::max<int64_t>(1, std::min<int64_t>(hi, max_splits));
 }
 
@@ -147,10 +145,8 @@ bool make_tc_tensor_maps_e4m3(const uint8_t* ref_f8, const __nv_bfloat16* ref_f8
 
 // Exact top-K1 search on tensor cores.  qbf: BF16 -2q operand [m_pad, 128];
 // qext: its K-extension [m_pad, 16].  Split s scans reference rows
-// [s * split_len, min((s+1) * split_len, n_ref)) and writes L =
-// tc_lists_per_split(K1, sched.qt) sorted lists per query row i, list w at
-// lists[((s * L + w) * stride + i) * K1]; the K1 smallest keys of their union
-// are the split's answer.
+// [s * split_len, min((s+1) * split_len, n_ref)) and writes one sorted list per
+// query row i at lists[(s * stride + i) * K1].
 // row_thr (null, or [m_pad] int32 filled with the bytes 0x7F beforehand) is
 // the per-row bound the lists of a row share: each list may leave out columns
 // that cannot be among the row's K1 nearest over all lists, so only the union

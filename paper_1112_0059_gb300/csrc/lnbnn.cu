@@ -52,8 +52,8 @@ struct lnbnn_index {
   SplitModel split_model;  // split-N schedule (defaults, or fitted by lnbnn_autotune)
   lnbnn_schedule sched{0, 0, -1, -1};  // lnbnn_set_schedule: fixed choices (0 / -1: automatic)
   // large-batch forms per scan kind (exact, coarse, NBNN), chosen by lnbnn_autotune
-  int auto_qt[3] = {1, 2, 1};
-  int auto_persistent[3] = {0, 0, 0};
+  int auto_qt[3] = {1, 1, 1};
+  int auto_persistent[3] = {0, 1, 0};
   const uint32_t* gate = nullptr;  // lnbnn_set_start_gate: search kernels wait for *gate != 0
   // optional device-time profile (lnbnn_profile_enable)
   struct CallEvents {
@@ -69,6 +69,7 @@ struct lnbnn_workspace {
   const lnbnn_index* index = nullptr;
   void* base = nullptr;
   size_t bytes = 0;
+  size_t sized = 0;  // KnnPlan::sized of its largest call
 };
 
 namespace {
@@ -214,9 +215,9 @@ bool k_ok(const lnbnn_index* ix, int32_t k, int extra) {
 }
 
 // Most reference splits of one launch: two CTAs per SM for a single query
-// tile, within what the list merge takes (two lists per split).
+// tile, within what the list merge takes.
 int64_t max_splits(const lnbnn_index* ix) {
-  return std::min<int64_t>(2 * (int64_t)ix->sm_count, 32 * kMaxListsPerLane / 2);
+  return std::min<int64_t>(2 * (int64_t)ix->sm_count, 32 * kMaxListsPerLane);
 }
 
 // What a scan computes: kNN lists over the exact BF16 operand, kNN lists over
@@ -240,34 +241,25 @@ bool l2_splits_for(ScanKind k) { return k == ScanKind::Coarse; }
 // The large-batch form of a scan kind (query tiles per CTA, persistent grid)
 // for launches of at least a full wave of query tiles, unless lnbnn_autotune
 // measured another form faster on this index.  Defaults, measured on the
-// 256-class data (750k query rows): one query tile per CTA for the exact and
-// NBNN scans (exact 1,229 ms a classify call against 1,263 with two, whose
-// steps take fewer cycles, 1,305 against 1,341, at a lower SM clock); two
-// for the FP8 coarse pass (shortlist 24, lists carried across the 37
-// L2-sized splits: 860 against 899 ms); one CTA per work item (persistent
-// grids within 0.2%).
-// The exact scan with lists longer than 16 entries takes two query tiles
-// per CTA whatever the tuned k+1 = 11 form is: one list per row and split
-// instead of two column halves halves the list work (256-class data, 750k
-// query rows: k = 20 1,277 against 1,303 ms, k = 100 with heaps 2,225
-// against 3,571 ms).
-int auto_query_tiles(const lnbnn_index* ix, ScanKind k, int64_t T1, int K1) {
-  if (T1 < ix->sm_count) return 1;
-  if (k == ScanKind::Exact && K1 > kTcRegListMax) return 2;
-  return ix->auto_qt[(int)k];
+// 256-class data: one query tile per CTA for every scan (two halve the
+// reference bytes, but their N = 128 MMAs cost issue time: FP8 shortlist 24,
+// 102k query rows over the 37 L2-sized splits 112.6 against 111.0 ms; exact
+// k = 20 on the 101-class data 51.7 against 47.8 ms); one CTA per work item,
+// but a persistent grid for the FP8 coarse pass, whose items are short (116.2
+// against 111.0 ms).
+int auto_query_tiles(const lnbnn_index* ix, ScanKind k, int64_t T1) {
+  return T1 < ix->sm_count ? 1 : ix->auto_qt[(int)k];
 }
 bool auto_persistent(const lnbnn_index* ix, ScanKind k, int64_t T1) {
   return T1 >= ix->sm_count && ix->auto_persistent[(int)k] == 1;
 }
 
 // Splits for the exact scan of a launch of at least a full wave whose lists
-// are dearer than the 16-entry ones: with the splits run one after another
-// and their lists carried across, the later splits insert little, and the
-// shorter reference ranges stay in L2.  Measured on the 256-class data (300k
-// query rows): k = 20 (24-entry lists) 1 / 4 splits 556 / 527 ms; k = 100
-// (heaps) 1 / 2 / 4 / 8 splits 1,493 / 1,464 / 1,437 / 1,413 ms.  The
-// 64-entry lists keep one split (at shorter splits they move to shared
-// memory, 2,660 against 2,367 cycles per step at k = 50).
+// are longer than 16 keys: with the splits run one after another and their
+// lists carried across, the later splits insert little, and a last wave that
+// is not full costs a split of it only (256-class data, k = 20, 60k query rows
+// = 469 query tiles: 1 / 4 splits 123.4 / 102.2 ms; k = 100, 30k rows: 1 / 8
+// splits 78.5 / 71.6 ms).
 int long_list_splits(const lnbnn_index* ix, int K1) {
   int want = 1;
   if (K1 > kTcRegListMax && K1 <= kTcCoarseRegListMax) want = 4;
@@ -291,7 +283,6 @@ int64_t splits_bound(const lnbnn_index* ix, int64_t T, ScanKind k) {
 struct KnnPlan {
   int64_t m_pad;
   int splits;
-  int lists;  // sorted lists per query row the search writes (merged when > 1)
   int64_t split_len;
   int K1;
   int qt;               // 128-row query tiles per CTA
@@ -300,7 +291,9 @@ struct KnnPlan {
   bool seeded;          // each split's lists may start from the same rows' previous split's lists
   int group;            // > 0: the claimed-chunk form (`splits` = CTAs per query-tile group, split_len = chunk)
   int64_t items;        // work items of the launch (query-tile groups x splits)
-  size_t off_qnorm, off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, bytes;
+  int64_t work_slots;   // candidate buffers of lists in progress (one set per CTA)
+  size_t off_qnorm, off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_slots, off_work, bytes;
+  size_t sized;  // bytes of what grows with queries and list length (all but the candidate buffers)
   TcSched sched(char* ws, int sm_count) const {
     TcSched t;
     t.qt = qt;
@@ -309,14 +302,21 @@ struct KnnPlan {
     t.bound_per_tile = bound_per_tile;
     t.done = seeded ? reinterpret_cast<uint32_t*>(ws + off_done) : nullptr;
     t.group = group;
+    t.work = ws + off_work;
+    t.work_slots = work_slots;
+    t.entries = tc_entries(K1);
+    t.slot_used = reinterpret_cast<uint32_t*>(ws + off_slots);
     return t;
   }
   // Clears what a launch needs zeroed: the work counter of a persistent
-  // launch, the per-item flags of a seeded one.
+  // launch, the per-item flags of a seeded one, the work areas' marks of one
+  // with more CTAs than work areas.
   cudaError_t clear(char* ws, cudaStream_t s) const {
     cudaError_t e = cudaSuccess;
     if (persistent) e = cudaMemsetAsync(ws + off_queue, 0, sizeof(uint32_t) * (size_t)(group > 0 ? items / splits : 1), s);
     if (e == cudaSuccess && seeded) e = cudaMemsetAsync(ws + off_done, 0, sizeof(uint32_t) * (size_t)items, s);
+    if (e == cudaSuccess && items > work_slots && !persistent)
+      e = cudaMemsetAsync(ws + off_slots, 0, sizeof(uint32_t) * (size_t)work_slots, s);
     return e;
   }
   // The merge's view of a seeded launch: rows whose last split holds every
@@ -327,7 +327,6 @@ struct KnnPlan {
     c.done = reinterpret_cast<const uint32_t*>(ws + off_done);
     c.T = items / splits;
     c.rows_per_item = (int64_t)kTcQueryTile * qt;
-    c.lists_per_split = lists / splits;
     return c;
   }
 };
@@ -345,26 +344,21 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.K1 = K1;
   const int64_t T1 = p.m_pad / kTcQueryTile;
   const bool qt2_ok = kind == ScanKind::Nbnn || K1 <= kTcCoarseRegListMax || K1 > kTcWideRegListMax;
-  p.qt = qt2_ok && (o.query_tiles == 2 || (o.query_tiles == 0 && auto_query_tiles(ix, kind, T1, K1) == 2)) ? 2 : 1;
+  p.qt = qt2_ok && (o.query_tiles == 2 || (o.query_tiles == 0 && auto_query_tiles(ix, kind, T1) == 2)) ? 2 : 1;
   const int64_t T = (T1 + p.qt - 1) / p.qt;
   if (splits <= 0) splits = o.splits;
   // The claimed-chunk form for launches of fewer query-tile groups than SMs
-  // (automatic split count; register lists or heaps): on a class-sorted
+  // (automatic split count; lists of up to 32 keys or more than 64): on a class-sorted
   // index the few reference ranges that hold a query's own class carry most
   // of the list inserts, and with fixed splits the CTAs that draw them set
   // the launch's time.  Instead each of P / T CTAs per group keeps the
   // group's lists for the whole launch and claims short reference chunks, in
   // increasing order, from the group's counter: the near-class chunks are
   // shared by whichever CTAs are free.
-  // The coarse pass, whose shortlist inserts are dear, takes it while there
-  // are at least 8 CTAs per query tile (256-class data, shortlist 24, one
-  // image of 100 / 256 / 512 / 768 / 1,280 / 2,000 descriptors: 0.42-0.54 /
-  // 0.71-0.76 / 1.07-1.13 / 1.38-1.50 / 2.11-2.32 / 2.93-3.44 ms against
-  // 0.55-0.66 / 0.84-0.89 / 1.14-1.27 / 1.69-1.74 / 2.41-2.47 / 3.28-3.53
-  // with splits; 4,000: slower, 4 CTAs per tile leave SMs idle); the exact
-  // scan, whose inserts are few, for a lone query tile only (0.53 against
-  // 0.55 ms at 100 descriptors; 2 and 3 tiles were 7-30% slower, 4 to 10
-  // tiles 1-12% faster).
+  // The coarse pass takes it while there are at least 8 CTAs per query tile
+  // (256-class data, shortlist 24, 632 descriptors: 854 us a call against 908
+  // with splits; with fewer CTAs a tile the rest of the SMs idle); the exact
+  // scan for a lone query tile only (100 descriptors: 530 against 560 us).
   const bool claim_kind = kind != ScanKind::Nbnn && (K1 <= kTcCoarseRegListMax || K1 > kTcWideRegListMax) &&
                           (kind == ScanKind::Coarse ? T * 8 <= P : T == 1);
   const int64_t ref_tiles = (ix->n_ref + kTcRefTile - 1) / kTcRefTile;
@@ -398,12 +392,16 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.off_qnorm = c.take<int32_t>(p.m_pad);
   p.off_qbf = c.take<__nv_bfloat16>(p.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.m_pad * kExt);
-  p.lists = p.splits * tc_lists_per_split(K1, p.qt);
-  p.off_lists = c.take<uint64_t>(kind == ScanKind::Nbnn ? 0 : (size_t)p.lists * p.m_pad * K1);
-  p.off_merged = c.take<uint64_t>(kind == ScanKind::Nbnn ? 0 : (size_t)p.m_pad * K1);  // apart from the lists (rerank)
+  const bool knn = kind != ScanKind::Nbnn;
+  p.off_lists = c.take<uint64_t>(knn ? (size_t)p.splits * p.m_pad * K1 : 0);
+  p.off_merged = c.take<uint64_t>(knn ? (size_t)p.m_pad * K1 : 0);  // apart from the lists (rerank)
   p.off_rowthr = c.take<int32_t>(p.m_pad);                // the bound a row's lists share
   p.off_queue = c.take<uint32_t>((size_t)T);             // the work counter(s) of a persistent launch
   p.off_done = c.take<uint32_t>((size_t)p.items);        // per-item "lists written" flags
+  p.sized = c.off;
+  p.work_slots = knn ? std::min<int64_t>(p.items, P) : p.items;  // (none for NBNN, which keeps no lists)
+  p.off_slots = c.take<uint32_t>((size_t)P);
+  p.off_work = c.take<char>(knn ? (size_t)(p.work_slots * tc_work_bytes(tc_entries(K1))) : 0);
   p.bytes = c.off;
   return p;
 }
@@ -413,6 +411,7 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
 struct Scratch {
   lnbnn_index* ix;
   lnbnn_workspace* w;
+  lnbnn_status admit(int64_t m, int K1) const;
   lnbnn_status get(size_t need, char** out) {
     if (w) {
       if (need > w->bytes) return LNBNN_ERR_SCRATCH_LIMIT;
@@ -446,24 +445,40 @@ NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
   return p;
 }
 
-// Largest scratch any call with at most max_q queries and lists of K1 needs.
-// The lists grow with the split count, so the bound takes the largest count
-// the schedule may choose (for either tile shape), whatever model
-// lnbnn_autotune fits later.
-size_t scratch_bound(const lnbnn_index* ix, int64_t max_q, int K1) {
-  size_t b = 0;
-  for (int64_t m = kQueryPad; m < max_q + kQueryPad; m += kQueryPad) {
-    const int64_t mm = std::min(m, max_q);
-    const int64_t T1 = round_up(mm, kQueryPad) / kTcQueryTile;
-    for (ScanKind k : {ScanKind::Exact, ScanKind::Coarse, ScanKind::Nbnn}) {
-      const int64_t hi = std::max(splits_bound(ix, T1, k), splits_bound(ix, (T1 + 1) / 2, k));
-      if (k == ScanKind::Nbnn)
-        b = std::max(b, plan_nbnn(ix, mm, (int)hi).bytes);
-      else
-        b = std::max(b, plan_knn(ix, mm, K1, k, (int)hi).bytes);
+// Largest scratch any call with at most max_q queries and lists of K1 needs,
+// and its KnnPlan::sized.  The lists grow with the split count, so the bound
+// takes the largest count the schedule may choose (for either tile shape),
+// whatever model lnbnn_autotune fits later.
+struct ScratchBound {
+  size_t bytes = 0, sized = 0;
+};
+void add_bound(const lnbnn_index* ix, int64_t m, int K1, ScratchBound* b) {
+  const int64_t T1 = round_up(m, kQueryPad) / kTcQueryTile;
+  for (ScanKind k : {ScanKind::Exact, ScanKind::Coarse, ScanKind::Nbnn}) {
+    const int64_t hi = std::max(splits_bound(ix, T1, k), splits_bound(ix, (T1 + 1) / 2, k));
+    if (k == ScanKind::Nbnn) {
+      b->bytes = std::max(b->bytes, plan_nbnn(ix, m, (int)hi).bytes);
+    } else {
+      const KnnPlan p = plan_knn(ix, m, K1, k, (int)hi);
+      b->bytes = std::max(b->bytes, p.bytes);
+      b->sized = std::max(b->sized, p.sized);
     }
   }
+}
+ScratchBound scratch_bound(const lnbnn_index* ix, int64_t max_q, int K1) {
+  ScratchBound b;
+  for (int64_t m = kQueryPad; m < max_q + kQueryPad; m += kQueryPad) add_bound(ix, std::min(m, max_q), K1, &b);
   return b;
+}
+
+// Whether a kNN call of m queries with lists of K1 is within the workspace it
+// was given.  (Its bytes alone would let longer lists in: the candidate
+// buffers outweigh the lists of a small call.)
+lnbnn_status Scratch::admit(int64_t m, int K1) const {
+  if (!w || w->sized == 0) return LNBNN_OK;
+  ScratchBound b;
+  add_bound(ix, m, K1, &b);
+  return b.sized > w->sized ? LNBNN_ERR_SCRATCH_LIMIT : LNBNN_OK;
 }
 
 // Runs the exact search; *lists receives m sorted lists of K1 keys.
@@ -471,7 +486,8 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
                      const uint64_t** lists, CallProfile& prof, int force_splits = 0) {
   KnnPlan p = plan_knn(ix, m, K1, ScanKind::Exact, force_splits);
   char* ws = nullptr;
-  lnbnn_status st = scratch.get(p.bytes, &ws);
+  lnbnn_status st = scratch.admit(m, K1);
+  if (st == LNBNN_OK) st = scratch.get(p.bytes, &ws);
   if (st != LNBNN_OK) return st;
   int32_t* qnorm = reinterpret_cast<int32_t*>(ws + p.off_qnorm);
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qbf);
@@ -491,11 +507,11 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
                    ix->gate, sched, s));
   prof.launched(1, true);
   prof.mark(2);
-  if (p.lists > 1) {
-    CK(launch_merge_lists(part, p.lists, m, p.m_pad, K1, merged, s, p.chain(ws)));
+  if (p.splits > 1) {
+    CK(launch_merge_lists(part, p.splits, m, p.m_pad, K1, merged, s, p.chain(ws)));
     prof.launched(1);
   }
-  *lists = p.lists > 1 ? merged : part;
+  *lists = p.splits > 1 ? merged : part;
   return LNBNN_OK;
 }
 
@@ -505,7 +521,8 @@ lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, in
                          cudaStream_t s, const uint64_t** lists, CallProfile& prof) {
   KnnPlan p = plan_knn(ix, m, M1, ScanKind::Coarse);
   char* ws = nullptr;
-  lnbnn_status st = scratch.get(p.bytes, &ws);
+  lnbnn_status st = scratch.admit(m, M1);
+  if (st == LNBNN_OK) st = scratch.get(p.bytes, &ws);
   if (st != LNBNN_OK) return st;
   // the BF16 query operand's space holds the E4M3 bytes (half its size)
   uint8_t* qf8 = reinterpret_cast<uint8_t*>(ws + p.off_qbf);
@@ -527,8 +544,8 @@ lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, in
   prof.mark(2);
   // the shortlist is the merged lists (or the one list); the reranked lists
   // go to the other buffer
-  if (p.lists > 1) {
-    CK(launch_merge_lists(part, p.lists, m, p.m_pad, M1, merged, s, p.chain(ws)));
+  if (p.splits > 1) {
+    CK(launch_merge_lists(part, p.splits, m, p.m_pad, M1, merged, s, p.chain(ws)));
     CK(launch_rerank(merged, m, M1, q, ix->ref_u8, ix->n_ref, K1, part, s));
     prof.launched(2);
     *lists = part;
@@ -864,16 +881,10 @@ lnbnn_status lnbnn_plan_search(const lnbnn_index* index, int64_t n_queries, int3
   const KnnPlan p = plan_knn(index, n_queries, k1, fp8 ? ScanKind::Coarse : ScanKind::Exact);
   lnbnn_search_plan r{};
   r.splits = p.splits;
-  r.lists_per_row = p.lists;
+  r.lists_per_row = p.splits;
   r.split_len = p.split_len;
-  switch (tc_list_kind(k1, p.split_len, fp8 != 0)) {
-    case ListKind::Reg16: r.list_storage = 0; r.list_capacity = kTcRegListMax; break;
-    case ListKind::Reg24: r.list_storage = 0; r.list_capacity = kTcMidRegListMax; break;
-    case ListKind::Reg32: r.list_storage = 0; r.list_capacity = kTcCoarseRegListMax; break;
-    case ListKind::Smem64: r.list_storage = 1; r.list_capacity = kTcWideRegListMax; break;
-    case ListKind::Reg64: r.list_storage = 0; r.list_capacity = kTcWideRegListMax; break;
-    case ListKind::Heap: r.list_storage = 2; r.list_capacity = k1; break;
-  }
+  r.list_storage = tc_list_max(k1) > 0 ? 0 : 2;
+  r.list_capacity = tc_list_max(k1) > 0 ? tc_list_max(k1) : k1;
   r.tile_m = kTcQueryTile * p.qt;
   r.tile_n = kTcRefTile / p.qt;
   r.persistent = p.persistent ? 1 : 0;
@@ -1366,7 +1377,9 @@ lnbnn_status lnbnn_workspace_create(lnbnn_index* index, int64_t max_queries, int
   lnbnn_workspace* w = new (std::nothrow) lnbnn_workspace();
   if (!w) return LNBNN_ERR_OOM;
   w->index = index;
-  w->bytes = scratch_bound(index, max_queries, std::min<int>(max_k + 1, LNBNN_MAX_K + 1));
+  const ScratchBound bound = scratch_bound(index, max_queries, std::min<int>(max_k + 1, LNBNN_MAX_K + 1));
+  w->bytes = bound.bytes;
+  w->sized = bound.sized;
   cudaError_t e = lib_malloc(&w->base, w->bytes);
   if (e != cudaSuccess) {
     delete w;

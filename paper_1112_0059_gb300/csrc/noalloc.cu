@@ -116,11 +116,12 @@ extern "C" LNBNN_API lnbnn_status knn_search_noalloc(const uint8_t* ref, int64_t
   if (!on_device(ref, dev) || !on_device(queries, dev) || !on_device(idx, dev) || !on_device(dist, dev))
     return LNBNN_ERR_INVALID_ARG;
 
-  // The index path's split schedule with the default model, at most 32
-  // splits (which bounds the scratch the lists take).
+  // The index path's split schedule with the default model, at most 32 splits
+  // of at least 4,096 references (which bounds the scratch the lists take).
   const int64_t n_pad = round_up(n_ref, kRefPad);
   const int64_t m_pad = round_up(n_queries, kQueryPad);
-  int64_t splits = choose_splits_model(SplitModel{}, m_pad / kTcQueryTile, n_ref, sm_count, 32);
+  int64_t splits = choose_splits_model(SplitModel{}, m_pad / kTcQueryTile, n_ref, sm_count,
+                                       std::min<int64_t>(32, std::max<int64_t>(1, n_ref / 4096)));
   const int64_t split_len = round_up((n_ref + splits - 1) / splits, kTcRefTile);
   splits = (n_ref + split_len - 1) / split_len;
 
@@ -128,42 +129,56 @@ extern "C" LNBNN_API lnbnn_status knn_search_noalloc(const uint8_t* ref, int64_t
   const size_t o_err = L.take<uint32_t>(1);
   const size_t o_rbf = L.take<__nv_bfloat16>((size_t)n_pad * kDim);
   const size_t o_rext = L.take<__nv_bfloat16>((size_t)n_pad * kExt);
-  const size_t o_rn = L.take<float>((size_t)n_pad);
-  const size_t o_qn = L.take<int32_t>((size_t)m_pad);
   const size_t o_qbf = L.take<__nv_bfloat16>((size_t)m_pad * kDim);
   const size_t o_qext = L.take<__nv_bfloat16>((size_t)m_pad * kExt);
-  const int64_t n_lists = splits * tc_lists_per_split(k);
-  const size_t o_lists = L.take<uint64_t>((size_t)n_lists * m_pad * k);
-  const size_t o_merged = n_lists > 1 ? L.take<uint64_t>((size_t)m_pad * k) : o_lists;
+  const size_t o_lists = L.take<uint64_t>((size_t)splits * m_pad * k);
+  const size_t o_merged = splits > 1 ? L.take<uint64_t>((size_t)m_pad * k) : o_lists;
   const size_t o_rowthr = L.take<int32_t>((size_t)m_pad);  // the bound the lists of a row share
+  const size_t o_queue = L.take<uint32_t>(1);
+  // candidate buffers of the lists in progress: one set per CTA, as many CTAs as the rest
+  // of the scratch has room for (those take the work items from a queue)
+  const size_t o_work = L.take<char>((size_t)tc_work_bytes(kTcMinEntries));
   if (L.off > (size_t)LNBNN_NOALLOC_SCRATCH_BYTES) return LNBNN_ERR_SCRATCH_LIMIT;
+  const int64_t items = (m_pad / kTcQueryTile) * splits;
+  TcSched sched;
+  auto areas = [&](int entries) {
+    const int64_t room = (int64_t)((size_t)LNBNN_NOALLOC_SCRATCH_BYTES - o_work) / tc_work_bytes(entries);
+    return std::min<int64_t>(std::min<int64_t>(items, sm_count), room);
+  };
+  sched.entries = tc_entries(k);
+  while (sched.entries > kTcMinEntries && areas(sched.entries) < areas(kTcMinEntries)) sched.entries -= 2;
+  sched.work_slots = areas(sched.entries);
 
   char* b = static_cast<char*>(base);
   uint32_t* err = reinterpret_cast<uint32_t*>(b + o_err);
   __nv_bfloat16* ref_bf = reinterpret_cast<__nv_bfloat16*>(b + o_rbf);
   __nv_bfloat16* ref_ext = reinterpret_cast<__nv_bfloat16*>(b + o_rext);
-  float* rnorm = reinterpret_cast<float*>(b + o_rn);
-  int32_t* qnorm = reinterpret_cast<int32_t*>(b + o_qn);
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(b + o_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(b + o_qext);
   uint64_t* lists = reinterpret_cast<uint64_t*>(b + o_lists);
   uint64_t* merged = reinterpret_cast<uint64_t*>(b + o_merged);
   int32_t* row_thr = reinterpret_cast<int32_t*>(b + o_rowthr);
+  sched.work = b + o_work;
+  if (items > sched.work_slots) {
+    sched.persistent_ctas = (int)sched.work_slots;
+    sched.queue = reinterpret_cast<uint32_t*>(b + o_queue);
+  }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
   TcTensorMaps maps;
   if (!make_tc_tensor_maps(ref_bf, ref_bf, ref_ext, ref_ext, n_pad, &maps)) return LNBNN_ERR_CUDA;
   // The array keeps the previous call's contents: the error word must start at
-  // zero and the rows' shared bounds above every distance; every other buffer
-  // is fully written before it is read.
+  // zero, the work counter too, and the rows' shared bounds above every
+  // distance; every other buffer is written before it is read.
   cudaError_t e = cudaMemsetAsync(err, 0, sizeof(uint32_t), s);
+  if (e == cudaSuccess && sched.queue) e = cudaMemsetAsync(sched.queue, 0, sizeof(uint32_t), s);
   if (e == cudaSuccess && splits > 1) e = cudaMemsetAsync(row_thr, 0x7F, sizeof(int32_t) * (size_t)m_pad, s);
-  if (e == cudaSuccess) e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, rnorm, ref_ext, s);
-  if (e == cudaSuccess) e = launch_prep_query(queries, n_queries, m_pad, kDim, 0, qnorm, qbf, qext, s);
+  if (e == cudaSuccess) e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, nullptr, ref_ext, s);
+  if (e == cudaSuccess) e = launch_prep_query(queries, n_queries, m_pad, kDim, 0, nullptr, qbf, qext, s);
   if (e == cudaSuccess)
     e = launch_knn_tc(maps, false, qbf, qext, n_queries, m_pad, n_ref, (int)splits, split_len, k, lists, m_pad,
-                      splits > 1 ? row_thr : nullptr, err, nullptr, nullptr, TcSched{}, s);
-  if (e == cudaSuccess && n_lists > 1) e = launch_merge_lists(lists, (int)n_lists, n_queries, m_pad, k, merged, s);
+                      splits > 1 ? row_thr : nullptr, err, nullptr, nullptr, sched, s);
+  if (e == cudaSuccess && splits > 1) e = launch_merge_lists(lists, (int)splits, n_queries, m_pad, k, merged, s);
   if (e == cudaSuccess) e = launch_extract_knn(merged, n_queries, k, k, idx, dist, s);
   uint32_t herr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);

@@ -89,7 +89,7 @@ __global__ void prep_ref_kernel(const uint8_t* __restrict__ ref, int64_t n_ref, 
     ly = (int32_t)ref[row * row_bytes + kDim + 1] - 128;
   }
   const int32_t norm = real ? ss + loc_w * (lx * lx + ly * ly) : (int32_t)kPadNorm;
-  rnorm[row] = (float)norm;
+  if (rnorm) rnorm[row] = (float)norm;
   // base-256 digits: d2 <= 56 for real rows, 512 for padding rows
   const float v[kExt] = {(float)(norm & 255), (float)((norm >> 8) & 255), (float)(norm >> 16), 1.0f, 256.0f,
                          65536.0f, (float)lx, (float)lx, (float)ly, (float)ly, 0, 0, 0, 0, 0, 0};
@@ -130,7 +130,7 @@ __global__ void prep_query_kernel(const uint8_t* __restrict__ q, int64_t m, int6
     ly = (int32_t)q[row * row_bytes + kDim + 1] - 128;
   }
   const int32_t norm = ss + loc_w * (lx * lx + ly * ly);
-  if (real) qnorm[row] = norm;
+  if (real && qnorm) qnorm[row] = norm;
   if (!qext) return;
   int32_t hx, lox, hy, loy;
   split256(loc_w * lx, &hx, &lox);

@@ -18,14 +18,13 @@ constexpr int kMergeWarps = 4;
 constexpr int kThreadMergeLists = 8;
 
 // The first list of row i to merge: all of them, or only the last split's
-// when that split's work item says its lists hold every earlier split's keys
+// when that split's work item says its list holds every earlier split's keys
 // (the scan's done flag 2).  Work item x + y T covers query rows
 // [x rows_per_item, (x + 1) rows_per_item) of split y.
 __device__ __forceinline__ int first_list(const MergeChain& c, int64_t i, int n_lists) {
   if (c.done == nullptr) return 0;
-  const int splits = n_lists / c.lists_per_split;
-  const int64_t w = i / c.rows_per_item + (int64_t)(splits - 1) * c.T;
-  return c.done[w] == 2u ? n_lists - c.lists_per_split : 0;
+  const int64_t w = i / c.rows_per_item + (int64_t)(n_lists - 1) * c.T;
+  return c.done[w] == 2u ? n_lists - 1 : 0;
 }
 
 __global__ void merge_lists_thread_kernel(const uint64_t* __restrict__ lists, int n_lists, int64_t m, int64_t stride,
@@ -258,9 +257,7 @@ cudaError_t launch_merge_lists(const uint64_t* lists, int splits, int64_t m, int
                                cudaStream_t s, const MergeChain& chain) {
   if (m == 0) return cudaSuccess;
   if (splits < 1 || splits > 32 * kMaxListsPerLane) return cudaErrorInvalidValue;
-  if (chain.done != nullptr &&
-      (chain.lists_per_split < 1 || splits % chain.lists_per_split != 0 || chain.T < 1 || chain.rows_per_item < 1))
-    return cudaErrorInvalidValue;
+  if (chain.done != nullptr && (chain.T < 1 || chain.rows_per_item < 1)) return cudaErrorInvalidValue;
   if (splits <= kThreadMergeLists) {
     merge_lists_thread_kernel<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(lists, splits, m, stride, K1, chain, out);
     return cudaGetLastError();

@@ -49,6 +49,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Whether the phase with the given parity has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Wait until the phase with the given parity has completed, for at most
 // `limit_ns` nanoseconds, giving up early once *abort_flag is set by another
 // role of the CTA.  Returns false on expiry or abort (the caller then winds
@@ -61,6 +72,65 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 255u) == 0 && (*abort_flag || globaltimer_ns() - t0 > limit_ns)) return false;
   }
+}
+
+// ------------------------------------------------------------ shared memory
+
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t ld_shared_acquire(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_shared_release(uint32_t addr, uint32_t v) {
+  asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// If least < lim: v[0..8) and col to the n-th 64-byte entry at `base`, and one
+// more entry.
+__device__ __forceinline__ void push_octet_if_less(const char* base, uint32_t& n, int32_t least, int32_t lim,
+                                                   const uint32_t* v, uint32_t col) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a;\n\tsetp.lt.s32 p, %1, %2;\n\tmad.wide.u32 a, %0, 64, %3;\n\t"
+      "@p st.global.v4.b32 [a], {%4, %5, %6, %7};\n\t@p st.global.v4.b32 [a+16], {%8, %9, %10, %11};\n\t"
+      "@p st.global.b32 [a+32], %12;\n\t@p add.u32 %0, %0, 1;\n\t}"
+      : "+r"(n)
+      : "r"(least), "r"(lim), "l"(base), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
+        "r"(v[7]), "r"(col)
+      : "memory");
+}
+
+// If x < lim: the pair (y, x) to [at], and step `at` past it.
+__device__ __forceinline__ void push_global_if_less(uint64_t*& at, int32_t x, int32_t lim, uint32_t y) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %1, %2;\n\t@p st.global.v2.b32 [%0], {%3, %1};\n\t"
+      "@p add.u64 %0, %0, 8;\n\t}"
+      : "+l"(at)
+      : "r"(x), "r"(lim), "r"(y)
+      : "memory");
+}
+
+// --------------------------------------------------------------- registers
+
+// A whole warpgroup gives up registers down to N a thread, or waits until it
+// has N.  What is taken must have been given up by others of the launch.
+template <int N>
+__device__ __forceinline__ void reg_dealloc() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_alloc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
 // ------------------------------------------------- gpu-scope flag accesses
