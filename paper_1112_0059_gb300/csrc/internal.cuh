@@ -100,7 +100,7 @@ cudaError_t launch_extract_knn(const uint64_t* lists, int64_t m, int K1, int k, 
 cudaError_t launch_lnbnn_score(const uint64_t* lists, int64_t m, int K1, int k, const int32_t* labels, int64_t n_ref,
                                const int64_t* offsets, int64_t n_img, int32_t C, int64_t* totals,
                                uint32_t* dev_err, cudaStream_t s);
-// Alg. 1 sum: totals[img][c] = sum of mins[row][c] over the image's rows.
+// Alg. 1 sum: totals[img][c] += sum of mins[row][c] over the image's rows.
 cudaError_t launch_nbnn_sum(const int32_t* mins, int64_t m, int32_t C, const int64_t* offsets, int64_t n_img,
                             int64_t* totals, cudaStream_t s);
 // Offsets validation (0 = o[0] <= ... <= o[n_img] = m); flags kDevErrOffsets.
@@ -118,19 +118,15 @@ cudaError_t launch_prep_query_e4m3(const uint8_t* q, int64_t m, int64_t m_pad, u
 // among the rows of its shortlist [m, M1] (kEmptyKey entries are no row).
 cudaError_t launch_rerank(const uint64_t* shortlist, int64_t m, int M1, const uint8_t* q, const uint8_t* ref,
                           int64_t n_ref, int K1, uint64_t* out, cudaStream_t s);
-// NBNN as a sum of log-odds increments (logodds.cu).  Per descriptor row of the
-// [m, C] class-minimum table, the statistics of its posterior (32 bytes a row);
-// then per image and class the sum of the increments (all, or only those > 0)
-// in row order, and per image the number of increments added (counts may be
-// null; it is added to, so the caller zeroes it).
-constexpr int kLogoddsRowStatBytes = 32;
-cudaError_t launch_logodds_rowstat(const int32_t* mins, int64_t m, int32_t C, double beta, void* rowstat,
-                                   cudaStream_t s);
-cudaError_t launch_logodds_sum(const int32_t* mins, const void* rowstat, int64_t m, int32_t C, double beta,
-                               bool positive_only, const int64_t* offsets, int64_t n_img, double* totals,
-                               int64_t* counts, cudaStream_t s);
-// argmax over classes per image, lowest class on ties.
-cudaError_t launch_argmax_f64(const double* totals, int64_t n_img, int32_t C, int32_t* classes, cudaStream_t s);
+// NBNN as a sum of log-odds increments (logodds.cu): from the [m, C] table of
+// class minima (which it overwrites), per image and class the sum of the
+// increments (all, or only those > 0), per image the number of increments
+// added (counts may be null) and the class of the largest sum, the lowest on
+// ties.  totals and counts are zeroed by the caller.  prepare_logodds sets the
+// kernel's shared-memory size on the current device (once, as prepare_tc_kernels).
+cudaError_t prepare_logodds();
+cudaError_t launch_logodds(int32_t* mins, int64_t m, int32_t C, double beta, bool positive_only, const int64_t* offsets,
+                           int64_t n_img, double* totals, int64_t* counts, int32_t* classes, cudaStream_t s);
 // argmin over classes per image, lowest class on ties.
 cudaError_t launch_argmin(const int64_t* totals, int64_t n_img, int32_t C, int32_t* classes, cudaStream_t s);
 

@@ -426,7 +426,7 @@ struct Scratch {
 
 struct NbnnPlan {
   KnnPlan k;
-  size_t off_qnorm, off_qbf, off_qext, off_mins, off_rowstat, off_queue, bytes;
+  size_t off_qnorm, off_qbf, off_qext, off_mins, off_queue, bytes;
 };
 
 NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
@@ -437,7 +437,6 @@ NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
   p.off_qbf = c.take<__nv_bfloat16>(p.k.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.k.m_pad * kExt);
   p.off_mins = c.take<int32_t>((size_t)p.k.m_pad * ix->n_classes);
-  p.off_rowstat = c.take<char>((size_t)p.k.m_pad * kLogoddsRowStatBytes);  // log-odds rule only
   p.off_queue = c.take<uint32_t>(1);
   p.k.off_queue = p.off_queue;
   p.k.seeded = false;
@@ -693,6 +692,7 @@ static lnbnn_status create_index(const uint8_t* ref, const int32_t* labels, int6
   if (!make_tc_tensor_maps(ix->ref_bf, ix->sref_bf, ix->ref_ext, ix->sref_ext, ix->n_pad, &ix->tc))
     return fail(LNBNN_ERR_CUDA);
   CKF(prepare_tc_kernels());
+  CKF(prepare_logodds());
   CKF(cudaStreamSynchronize(s));
   cudaFree(counts);
   cudaFree(bad);
@@ -1240,11 +1240,9 @@ static lnbnn_status do_lnbnn_classify(lnbnn_index* index, lnbnn_workspace* w, co
 
 // The [m_pad, C] table of class minima NN_C(d), one row per query row, filled
 // by the tensor-core scan of the class-sorted references (Alg. 1's inner
-// loop).  Sets *mins and, when rowstat is given, the row-statistics buffer of
-// the same workspace.
+// loop).
 static lnbnn_status scan_class_minima(lnbnn_index* index, lnbnn_workspace* w, const uint8_t* queries,
-                                      int64_t n_queries, cudaStream_t s, CallProfile& prof, int32_t** mins,
-                                      void** rowstat) {
+                                      int64_t n_queries, cudaStream_t s, CallProfile& prof, int32_t** mins) {
   const NbnnPlan np = plan_nbnn(index, n_queries);
   const KnnPlan& p = np.k;
   Scratch scratch{index, w};
@@ -1255,7 +1253,6 @@ static lnbnn_status scan_class_minima(lnbnn_index* index, lnbnn_workspace* w, co
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qext);
   *mins = reinterpret_cast<int32_t*>(ws + np.off_mins);
-  if (rowstat) *rowstat = ws + np.off_rowstat;
   CK(launch_prep_query(queries, n_queries, p.m_pad, index->row_bytes, index->loc_w, qnorm, qbf, qext, s));
   CK(cudaMemsetAsync(*mins, 0x7F, sizeof(int32_t) * (size_t)p.m_pad * index->n_classes, s));  // > any distance
   const TcSched sched = p.sched(ws, index->sm_count);
@@ -1289,7 +1286,7 @@ static lnbnn_status do_nbnn_classify(lnbnn_index* index, lnbnn_workspace* w, con
     prof.mark(2);
   } else {
     int32_t* mins = nullptr;
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins, nullptr);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins);
     if (st != LNBNN_OK) return st;
     CK(launch_nbnn_sum(mins, n_queries, C, offsets, n_images, totals, s));
     prof.launched(1);
@@ -1316,20 +1313,16 @@ static lnbnn_status do_nbnn_logodds_classify(lnbnn_index* index, lnbnn_workspace
   if (n_increments) CK(cudaMemsetAsync(n_increments, 0, sizeof(int64_t) * (size_t)n_images, s));
   CK(launch_check_offsets(offsets, n_images, n_queries, index->dev_err, s));
   prof.launched(1);
+  int32_t* mins = nullptr;
   if (n_queries == 0) {
     prof.mark(1);
     prof.mark(2);
   } else {
-    int32_t* mins = nullptr;
-    void* rowstat = nullptr;
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins, &rowstat);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins);
     if (st != LNBNN_OK) return st;
-    CK(launch_logodds_rowstat(mins, n_queries, C, beta, rowstat, s));
-    CK(launch_logodds_sum(mins, rowstat, n_queries, C, beta, positive_only, offsets, n_images, totals,
-                          n_increments, s));
-    prof.launched(2);
+    prof.launched(1);
   }
-  CK(launch_argmax_f64(totals, n_images, C, classes, s));
+  CK(launch_logodds(mins, n_queries, C, beta, positive_only, offsets, n_images, totals, n_increments, classes, s));
   prof.launched(1);
   return LNBNN_OK;
 }

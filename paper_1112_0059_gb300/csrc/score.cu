@@ -1,5 +1,7 @@
 // Split merge, knn_search output, the Local NBNN class update (Alg. 2), the
 // offsets check and the per-image argmin (Alg. 1 and Alg. 2, last line).
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace lnbnn {
@@ -140,76 +142,111 @@ __device__ __forceinline__ int64_t image_of(const int64_t* __restrict__ offsets,
 // (distance, row): dist_B = distance of the (k+1)-th; every class found among
 // the first k is updated once with dist_C - dist_B, where dist_C is the
 // distance of its first (hence nearest) occurrence in the sorted list.
-// Thread per row; the adds are aggregated per warp: at each neighbour rank
-// the lanes that update the same (image, class) are grouped, and one of them
-// adds the group's sum (int64 addition, exact in any order).
-constexpr int kScoreThreads = 128;
-__global__ void __launch_bounds__(kScoreThreads)
+//
+// A warp per row: lane a holds neighbours a, a + 32, ..., so the labels of a
+// row are gathered at once, and __match_any_sync finds the first of each class
+// (a thread per row gathered and compared k^2 / 2 of them one after another:
+// k = 100, 15k rows 1.78 ms).  A block takes consecutive rows; a stretch of at
+// least kTableRows of one image is summed in shared memory first (int32: the
+// block's rows times the largest distance stay below 2^31), the rest goes
+// straight to the totals.
+constexpr int kScoreWarps = 8;
+constexpr int kScoreMaxRows = 128;    // rows of a block: 128 x 14,565,600 < 2^31
+constexpr int kTableRows = 8;
+constexpr int kTableClasses = 8192;   // classes up to which the sums fit (32 KB)
+template <int G>  // ceil(k / 32) neighbours per lane, or more
+__global__ void __launch_bounds__(32 * kScoreWarps)
     lnbnn_score_kernel(const uint64_t* __restrict__ lists, int64_t m, int K1, int k,
                        const int32_t* __restrict__ labels, int64_t n_ref, const int64_t* __restrict__ offsets,
-                       int64_t n_img, int32_t C, int64_t* __restrict__ totals, uint32_t* __restrict__ dev_err) {
-  __shared__ int64_t part[kScoreThreads];
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int64_t* wpart = part + (threadIdx.x & ~31);
-  bool ok = i < m;
-  int64_t img = 0;
-  if (ok) {
-    img = image_of(offsets, n_img, i);
-    if (i < offsets[img] || i >= offsets[img + 1]) {  // only with invalid offsets
-      atomicOr(dev_err, kDevErrOffsets);
-      ok = false;
-    }
-  }
-  const uint64_t* L = lists + (ok ? i : 0) * K1;
-  // A complete list holds k+1 real rows.  Only a search that gave up (a
-  // timeout, reported by lnbnn_sync) leaves empty keys: skip such a row
-  // rather than gather labels[] at an empty key's row.
-  if (ok)
-    for (int a = 0; a <= k; ++a)
-      if ((int64_t)key_row(L[a]) >= n_ref) ok = false;
-  const int64_t dist_B = ok ? (int64_t)key_dist(L[k]) : 0;
+                       int64_t n_img, int32_t C, int rows, bool table, int64_t* __restrict__ totals,
+                       uint32_t* __restrict__ dev_err) {
+  extern __shared__ int32_t sums[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long* t = reinterpret_cast<unsigned long long*>(totals);
-  for (int a = 0; a < k; ++a) {  // every lane of the warp takes every step
-    long long slot = -1;          // img * C + class of this lane's update, or none
-    int64_t delta = 0;
-    if (ok) {
-      const uint64_t ka = L[a];
-      const int32_t c = labels[key_row(ka)];
-      bool seen = false;
-      for (int b = 0; b < a && !seen; ++b) seen = labels[key_row(L[b])] == c;
-      if (!seen) {
-        delta = (int64_t)key_dist(ka) - dist_B;  // <= 0
-        if (delta != 0) slot = img * C + c;
+  const int64_t row1 = min(m, ((int64_t)blockIdx.x + 1) * rows);
+  for (int64_t r = (int64_t)blockIdx.x * rows; r < row1;) {  // stretches of one image (the same for the block)
+    const int64_t img = image_of(offsets, n_img, r);
+    const int64_t end = min(offsets[img + 1], row1);
+    if (r < offsets[img] || r >= end) {  // only with invalid offsets
+      if (threadIdx.x == 0) atomicOr(dev_err, kDevErrOffsets);
+      ++r;
+      continue;
+    }
+    const bool summed = table && end - r >= kTableRows;
+    if (summed) {
+      for (int32_t c = threadIdx.x; c < C; c += 32 * kScoreWarps) sums[c] = 0;
+      __syncthreads();
+    }
+    for (int64_t i = r + warp; i < end; i += kScoreWarps) {
+      const uint64_t* L = lists + i * K1;
+      const uint64_t last = L[k];
+      uint64_t key[G];
+      int32_t lab[G];
+      // A complete list holds k+1 real rows.  Only a search that gave up (a
+      // timeout, reported by lnbnn_sync) leaves empty keys: skip such a row
+      // rather than gather labels[] at an empty key's row.
+      bool ok = (int64_t)key_row(last) < n_ref;
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int a = 32 * g + lane;
+        key[g] = a < k ? L[a] : last;
+        ok = ok && (int64_t)key_row(key[g]) < n_ref;
+      }
+      if (!__all_sync(0xffffffffu, ok)) continue;
+#pragma unroll
+      for (int g = 0; g < G; ++g) lab[g] = 32 * g + lane < k ? labels[key_row(key[g])] : -1 - lane;
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        bool first = __ffs(__match_any_sync(0xffffffffu, lab[g])) - 1 == lane && lab[g] >= 0;
+#pragma unroll
+        for (int h = 0; h < g; ++h)
+#pragma unroll 8
+          for (int j = 0; j < 32; ++j) {
+            const int32_t other = __shfl_sync(0xffffffffu, lab[h], j);  // (every lane takes part)
+            first = first && other != lab[g];
+          }
+        const int32_t delta = (int32_t)key_dist(key[g]) - (int32_t)key_dist(last);  // <= 0
+        if (first && delta != 0) {
+          if (summed)
+            atomicAdd(sums + lab[g], delta);
+          else
+            atomicAdd(t + img * C + lab[g], (unsigned long long)(int64_t)delta);
+        }
       }
     }
-    const unsigned act = __ballot_sync(0xffffffffu, slot >= 0);
-    if (slot >= 0) {
-      const unsigned grp = __match_any_sync(act, (unsigned long long)slot);
-      wpart[lane] = delta;
-      __syncwarp(act);
-      if (lane == __ffs(grp) - 1) {
-        int64_t sum = 0;
-        for (unsigned g = grp; g; g &= g - 1) sum += wpart[__ffs(g) - 1];
-        atomicAdd(t + slot, (unsigned long long)sum);
-      }
-      __syncwarp(act);  // the leaders have read the slots before the next step writes them
+    if (summed) {
+      __syncthreads();
+      for (int32_t c = threadIdx.x; c < C; c += 32 * kScoreWarps)
+        if (sums[c] != 0) atomicAdd(t + img * C + c, (unsigned long long)(int64_t)sums[c]);
+      __syncthreads();
     }
+    r = end;
   }
 }
 
-// Alg. 1's sum for image img and class c: totals[img][c] = sum over the image's
-// descriptor rows of mins[row][c] (= NN_c of that descriptor).  Rows outside
-// [0, m) are skipped (they only arise from invalid offsets, flagged elsewhere).
+// Alg. 1's sums: totals[img][c] += the sum over the image's descriptor rows of
+// mins[row][c] (= NN_c of that descriptor).  A block takes 32 rows and 128
+// classes, whatever the images (a block per image left most SMs idle: 20
+// images, 162 us); integer addition is exact in any order.
+constexpr int kSumRows = 32;
 __global__ void nbnn_sum_kernel(const int32_t* __restrict__ mins, int64_t m, int32_t C,
-                                const int64_t* __restrict__ offsets, int64_t* __restrict__ totals) {
-  const int64_t img = blockIdx.x;
+                                const int64_t* __restrict__ offsets, int64_t n_img, int64_t* __restrict__ totals) {
   const int32_t c = blockIdx.y * blockDim.x + threadIdx.x;
   if (c >= C) return;
-  const int64_t r0 = max(offsets[img], (int64_t)0), r1 = min(offsets[img + 1], m);
-  int64_t acc = 0;
-  for (int64_t r = r0; r < r1; ++r) acc += mins[r * C + c];
-  totals[img * C + c] = acc;
+  const int64_t row1 = min(m, ((int64_t)blockIdx.x + 1) * kSumRows);
+  for (int64_t r = (int64_t)blockIdx.x * kSumRows; r < row1;) {
+    const int64_t img = image_of(offsets, n_img, r);
+    const int64_t end = min(offsets[img + 1], row1);
+    if (r < offsets[img] || r >= end) {  // only with invalid offsets, flagged elsewhere
+      ++r;
+      continue;
+    }
+    int64_t acc = 0;
+#pragma unroll 8
+    for (int64_t i = r; i < end; ++i) acc += mins[i * C + c];
+    atomicAdd(reinterpret_cast<unsigned long long*>(totals) + img * C + c, (unsigned long long)acc);
+    r = end;
+  }
 }
 
 __global__ void check_offsets_kernel(const int64_t* __restrict__ offsets, int64_t n_img, int64_t m,
@@ -279,16 +316,32 @@ cudaError_t launch_lnbnn_score(const uint64_t* lists, int64_t m, int K1, int k, 
                                const int64_t* offsets, int64_t n_img, int32_t C, int64_t* totals, uint32_t* dev_err,
                                cudaStream_t s) {
   if (m == 0 || n_img == 0) return cudaSuccess;
-  lnbnn_score_kernel<<<(unsigned)((m + kScoreThreads - 1) / kScoreThreads), kScoreThreads, 0, s>>>(
-      lists, m, K1, k, labels, n_ref, offsets, n_img, C, totals, dev_err);
+  // a row per warp while the rows do not fill the chip that way, then more (the
+  // table is written to the totals once per block)
+  const int rows = (int)std::min<int64_t>(kScoreMaxRows, kScoreWarps * std::max<int64_t>(1, m / 8192));
+  const bool table = C <= kTableClasses;
+  const unsigned blocks = (unsigned)((m + rows - 1) / rows);
+  const size_t smem = table ? sizeof(int32_t) * (size_t)C : 0;
+  auto launch = [&](auto kernel) {
+    kernel<<<blocks, 32 * kScoreWarps, smem, s>>>(lists, m, K1, k, labels, n_ref, offsets, n_img, C, rows, table, totals,
+                                                  dev_err);
+  };
+  if (k <= 32)
+    launch(lnbnn_score_kernel<1>);
+  else if (k <= 64)
+    launch(lnbnn_score_kernel<2>);
+  else if (k <= 128)
+    launch(lnbnn_score_kernel<4>);
+  else
+    launch(lnbnn_score_kernel<8>);
   return cudaGetLastError();
 }
 
 cudaError_t launch_nbnn_sum(const int32_t* mins, int64_t m, int32_t C, const int64_t* offsets, int64_t n_img,
                             int64_t* totals, cudaStream_t s) {
-  if (n_img == 0) return cudaSuccess;
-  dim3 grid((unsigned)n_img, (unsigned)((C + 127) / 128));
-  nbnn_sum_kernel<<<grid, 128, 0, s>>>(mins, m, C, offsets, totals);
+  if (n_img == 0 || m == 0) return cudaSuccess;
+  dim3 grid((unsigned)((m + kSumRows - 1) / kSumRows), (unsigned)((C + 127) / 128));
+  nbnn_sum_kernel<<<grid, 128, 0, s>>>(mins, m, C, offsets, n_img, totals);
   return cudaGetLastError();
 }
 
