@@ -15,6 +15,7 @@
 // (distance, row) keys, the same keys the exact search produces.
 #include <cuda_fp8.h>
 
+#include "begin.cuh"
 #include "internal.cuh"
 
 namespace lnbnn {
@@ -47,7 +48,12 @@ __device__ __forceinline__ uint4 ext_head(float a, float b, float c, float d, fl
 // all zero for queries.
 template <bool kQuery>
 __global__ void prep_e4m3_kernel(const uint8_t* __restrict__ x, int64_t n, int64_t n_pad, uint8_t* __restrict__ f8,
-                                 __nv_bfloat16* __restrict__ ext) {
+                                 __nv_bfloat16* __restrict__ ext, const __grid_constant__ Begin begin,
+                                 unsigned prep_blocks) {
+  if (blockIdx.x >= prep_blocks) {
+    begin_part(begin, blockIdx.x - prep_blocks, gridDim.x - prep_blocks);
+    return;
+  }
   const int sub = threadIdx.x % kThreadsPerRow;
   const int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.x / kThreadsPerRow;
   if (row >= n_pad) return;
@@ -157,15 +163,17 @@ cudaError_t launch_prep_ref_e4m3(const uint8_t* ref, int64_t n_ref, int64_t n_pa
                                  __nv_bfloat16* ref_ext, cudaStream_t s) {
   if (n_pad == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((n_pad + kRowsPerBlock - 1) / kRowsPerBlock);
-  prep_e4m3_kernel<false><<<blocks, kThreadsPerRow * kRowsPerBlock, 0, s>>>(ref, n_ref, n_pad, ref_f8, ref_ext);
+  prep_e4m3_kernel<false><<<blocks, kThreadsPerRow * kRowsPerBlock, 0, s>>>(ref, n_ref, n_pad, ref_f8, ref_ext, Begin{},
+                                                                          blocks);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prep_query_e4m3(const uint8_t* q, int64_t m, int64_t m_pad, uint8_t* qf8, __nv_bfloat16* qext,
-                                   cudaStream_t s) {
-  if (m_pad == 0) return cudaSuccess;
+                                   const Begin& begin, cudaStream_t s) {
+  static_assert(kThreadsPerRow * kRowsPerBlock == kBeginThreads, "one block size for both parts");
+  if (m_pad == 0) return launch_begin(begin, s);
   const unsigned blocks = (unsigned)((m_pad + kRowsPerBlock - 1) / kRowsPerBlock);
-  prep_e4m3_kernel<true><<<blocks, kThreadsPerRow * kRowsPerBlock, 0, s>>>(q, m, m_pad, qf8, qext);
+  prep_e4m3_kernel<true><<<blocks + begin_blocks(begin), kBeginThreads, 0, s>>>(q, m, m_pad, qf8, qext, begin, blocks);
   return cudaGetLastError();
 }
 

@@ -291,8 +291,9 @@ struct KnnPlan {
   bool seeded;          // each split's lists may start from the same rows' previous split's lists
   int group;            // > 0: the claimed-chunk form (`splits` = CTAs per query-tile group, split_len = chunk)
   int64_t items;        // work items of the launch (query-tile groups x splits)
+  bool bounded;         // several splits of a row share its bound
   int64_t work_slots;   // candidate buffers of lists in progress (one set per CTA)
-  size_t off_qnorm, off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_slots, off_work, bytes;
+  size_t off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_slots, off_work, bytes;
   size_t sized;  // bytes of what grows with queries and list length (all but the candidate buffers)
   TcSched sched(char* ws, int sm_count) const {
     TcSched t;
@@ -308,16 +309,14 @@ struct KnnPlan {
     t.slot_used = reinterpret_cast<uint32_t*>(ws + off_slots);
     return t;
   }
-  // Clears what a launch needs zeroed: the work counter of a persistent
-  // launch, the per-item flags of a seeded one, the work areas' marks of one
-  // with more CTAs than work areas.
-  cudaError_t clear(char* ws, cudaStream_t s) const {
-    cudaError_t e = cudaSuccess;
-    if (persistent) e = cudaMemsetAsync(ws + off_queue, 0, sizeof(uint32_t) * (size_t)(group > 0 ? items / splits : 1), s);
-    if (e == cudaSuccess && seeded) e = cudaMemsetAsync(ws + off_done, 0, sizeof(uint32_t) * (size_t)items, s);
-    if (e == cudaSuccess && items > work_slots && !persistent)
-      e = cudaMemsetAsync(ws + off_slots, 0, sizeof(uint32_t) * (size_t)work_slots, s);
-    return e;
+  // What a launch needs set before it: the work counters of a persistent one,
+  // the per-item flags of a seeded one, the candidate buffers' marks of one
+  // with more CTAs than buffers, the rows' shared bounds.
+  void begin(char* ws, Begin* b) const {
+    if (persistent) b->fill(ws + off_queue, sizeof(uint32_t) * (size_t)(group > 0 ? items / splits : 1), 0u);
+    if (seeded) b->fill(ws + off_done, sizeof(uint32_t) * (size_t)items, 0u);
+    if (items > work_slots && !persistent) b->fill(ws + off_slots, sizeof(uint32_t) * (size_t)work_slots, 0u);
+    if (bounded) b->fill(ws + off_rowthr, sizeof(int32_t) * (size_t)m_pad, 0x7F7F7F7Fu);
   }
   // The merge's view of a seeded launch: rows whose last split holds every
   // split's keys merge only that split's lists.
@@ -389,10 +388,10 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.items = T * p.splits;
   p.seeded = kind != ScanKind::Nbnn && p.splits > 1 && !p.bound_per_tile;
   Carve c;
-  p.off_qnorm = c.take<int32_t>(p.m_pad);
   p.off_qbf = c.take<__nv_bfloat16>(p.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.m_pad * kExt);
   const bool knn = kind != ScanKind::Nbnn;
+  p.bounded = knn && p.splits > 1;
   p.off_lists = c.take<uint64_t>(knn ? (size_t)p.splits * p.m_pad * K1 : 0);
   p.off_merged = c.take<uint64_t>(knn ? (size_t)p.m_pad * K1 : 0);  // apart from the lists (rerank)
   p.off_rowthr = c.take<int32_t>(p.m_pad);                // the bound a row's lists share
@@ -426,14 +425,13 @@ struct Scratch {
 
 struct NbnnPlan {
   KnnPlan k;
-  size_t off_qnorm, off_qbf, off_qext, off_mins, off_queue, bytes;
+  size_t off_qbf, off_qext, off_mins, off_queue, bytes;
 };
 
 NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
   NbnnPlan p{};
   p.k = plan_knn(ix, m, 1, ScanKind::Nbnn, splits);
   Carve c;
-  p.off_qnorm = c.take<int32_t>(p.k.m_pad);
   p.off_qbf = c.take<__nv_bfloat16>(p.k.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.k.m_pad * kExt);
   p.off_mins = c.take<int32_t>((size_t)p.k.m_pad * ix->n_classes);
@@ -482,27 +480,25 @@ lnbnn_status Scratch::admit(int64_t m, int K1) const {
 
 // Runs the exact search; *lists receives m sorted lists of K1 keys.
 lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, cudaStream_t s,
-                     const uint64_t** lists, CallProfile& prof, int force_splits = 0) {
+                     const uint64_t** lists, CallProfile& prof, Begin begin = Begin{}, int force_splits = 0) {
   KnnPlan p = plan_knn(ix, m, K1, ScanKind::Exact, force_splits);
   char* ws = nullptr;
   lnbnn_status st = scratch.admit(m, K1);
   if (st == LNBNN_OK) st = scratch.get(p.bytes, &ws);
   if (st != LNBNN_OK) return st;
-  int32_t* qnorm = reinterpret_cast<int32_t*>(ws + p.off_qnorm);
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qext);
   uint64_t* part = reinterpret_cast<uint64_t*>(ws + p.off_lists);
   uint64_t* merged = reinterpret_cast<uint64_t*>(ws + p.off_merged);
   int32_t* row_thr = reinterpret_cast<int32_t*>(ws + p.off_rowthr);
   Range range("lnbnn: exact k+1 search");
-  CK(launch_prep_query(q, m, p.m_pad, ix->row_bytes, ix->loc_w, qnorm, qbf, qext, s));
-  CK(cudaMemsetAsync(row_thr, 0x7F, sizeof(int32_t) * (size_t)p.m_pad, s));
+  p.begin(ws, &begin);
+  CK(launch_prep_query(q, m, p.m_pad, ix->row_bytes, ix->loc_w, qbf, qext, begin, s));
   const TcSched sched = p.sched(ws, ix->sm_count);
-  CK(p.clear(ws, s));
   prof.launched(1);
   prof.mark(1);
   CK(launch_knn_tc(ix->tc, /*sorted_copy=*/false, qbf, qext, m, p.m_pad, ix->n_ref, p.splits, p.split_len, K1, part,
-                   p.m_pad, p.splits > 1 ? row_thr : nullptr, ix->dev_err, ix->prof_on ? ix->prof_stats : nullptr,
+                   p.m_pad, p.bounded ? row_thr : nullptr, ix->dev_err, ix->prof_on ? ix->prof_stats : nullptr,
                    ix->gate, sched, s));
   prof.launched(1, true);
   prof.mark(2);
@@ -517,7 +513,7 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
 // The FP8 shortlist search: coarse pass keeping the M1 smallest coarse keys,
 // merge, exact rerank; *lists receives m sorted lists of K1 exact keys.
 lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, int M1,
-                         cudaStream_t s, const uint64_t** lists, CallProfile& prof) {
+                         cudaStream_t s, const uint64_t** lists, CallProfile& prof, Begin begin = Begin{}) {
   KnnPlan p = plan_knn(ix, m, M1, ScanKind::Coarse);
   char* ws = nullptr;
   lnbnn_status st = scratch.admit(m, M1);
@@ -530,14 +526,13 @@ lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, in
   uint64_t* merged = reinterpret_cast<uint64_t*>(ws + p.off_merged);
   int32_t* row_thr = reinterpret_cast<int32_t*>(ws + p.off_rowthr);
   Range range("lnbnn: FP8 shortlist search");
-  CK(launch_prep_query_e4m3(q, m, p.m_pad, qf8, qext, s));
-  CK(cudaMemsetAsync(row_thr, 0x7F, sizeof(int32_t) * (size_t)p.m_pad, s));
+  p.begin(ws, &begin);
+  CK(launch_prep_query_e4m3(q, m, p.m_pad, qf8, qext, begin, s));
   const TcSched sched = p.sched(ws, ix->sm_count);
-  CK(p.clear(ws, s));
   prof.launched(1);
   prof.mark(1);
   CK(launch_coarse_tc(ix->tc, qf8, qext, m, p.m_pad, ix->n_ref, p.splits, p.split_len, M1, part, p.m_pad,
-                      p.splits > 1 ? row_thr : nullptr, ix->dev_err, ix->prof_on ? ix->prof_stats : nullptr,
+                      p.bounded ? row_thr : nullptr, ix->dev_err, ix->prof_on ? ix->prof_stats : nullptr,
                       ix->gate, sched, s));
   prof.launched(1, true);
   prof.mark(2);
@@ -1013,7 +1008,7 @@ lnbnn_status lnbnn_autotune(lnbnn_index* index, void* stream, lnbnn_tuning* out)
       Scratch scratch{index, &w};
       CallProfile prof(index, s);
       const uint64_t* lists = nullptr;
-      return run_knn(index, scratch, q, r.T * kTcQueryTile, r.K1, s, &lists, prof, (int)r.splits);
+      return run_knn(index, scratch, q, r.T * kTcQueryTile, r.K1, s, &lists, prof, Begin{}, (int)r.splits);
     }, &r.ms);
     if (st != LNBNN_OK) {
       cleanup();
@@ -1217,19 +1212,24 @@ static lnbnn_status do_lnbnn_classify(lnbnn_index* index, lnbnn_workspace* w, co
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallProfile prof(index, s);
   const int32_t C = index->n_classes;
-  CK(cudaMemsetAsync(totals, 0, sizeof(int64_t) * (size_t)n_images * C, s));
-  CK(launch_check_offsets(offsets, n_images, n_queries, index->dev_err, s));
-  prof.launched(1);
+  Begin begin;
+  begin.fill(totals, sizeof(int64_t) * (size_t)n_images * C, 0u);
+  begin.offsets = offsets;
+  begin.n_img = n_images;
+  begin.m = n_queries;
+  begin.dev_err = index->dev_err;
   if (n_queries > 0) {
     Scratch scratch{index, w};
     const uint64_t* lists = nullptr;
-    lnbnn_status st = shortlist ? run_knn_fp8(index, scratch, queries, n_queries, k + 1, M1, s, &lists, prof)
-                                : run_knn(index, scratch, queries, n_queries, k + 1, s, &lists, prof);
+    lnbnn_status st = shortlist ? run_knn_fp8(index, scratch, queries, n_queries, k + 1, M1, s, &lists, prof, begin)
+                                : run_knn(index, scratch, queries, n_queries, k + 1, s, &lists, prof, begin);
     if (st != LNBNN_OK) return st;
     CK(launch_lnbnn_score(lists, n_queries, k + 1, k, index->labels, index->n_ref, offsets, n_images, C, totals,
                           index->dev_err, s));
     prof.launched(1);
   } else {
+    CK(launch_begin(begin, s));
+    prof.launched(1);
     prof.mark(1);
     prof.mark(2);
   }
@@ -1242,21 +1242,21 @@ static lnbnn_status do_lnbnn_classify(lnbnn_index* index, lnbnn_workspace* w, co
 // by the tensor-core scan of the class-sorted references (Alg. 1's inner
 // loop).
 static lnbnn_status scan_class_minima(lnbnn_index* index, lnbnn_workspace* w, const uint8_t* queries,
-                                      int64_t n_queries, cudaStream_t s, CallProfile& prof, int32_t** mins) {
+                                      int64_t n_queries, Begin begin, cudaStream_t s, CallProfile& prof,
+                                      int32_t** mins) {
   const NbnnPlan np = plan_nbnn(index, n_queries);
   const KnnPlan& p = np.k;
   Scratch scratch{index, w};
   char* ws = nullptr;
   lnbnn_status st = scratch.get(np.bytes, &ws);
   if (st != LNBNN_OK) return st;
-  int32_t* qnorm = reinterpret_cast<int32_t*>(ws + np.off_qnorm);
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qext);
   *mins = reinterpret_cast<int32_t*>(ws + np.off_mins);
-  CK(launch_prep_query(queries, n_queries, p.m_pad, index->row_bytes, index->loc_w, qnorm, qbf, qext, s));
-  CK(cudaMemsetAsync(*mins, 0x7F, sizeof(int32_t) * (size_t)p.m_pad * index->n_classes, s));  // > any distance
+  begin.fill(*mins, sizeof(int32_t) * (size_t)p.m_pad * index->n_classes, 0x7F7F7F7Fu);  // > any distance
+  p.begin(ws, &begin);
+  CK(launch_prep_query(queries, n_queries, p.m_pad, index->row_bytes, index->loc_w, qbf, qext, begin, s));
   const TcSched sched = p.sched(ws, index->sm_count);
-  CK(p.clear(ws, s));
   prof.launched(1);
   prof.mark(1);
   CK(launch_nbnn_tc(index->tc, qbf, qext, n_queries, p.m_pad, index->n_ref, p.splits, p.split_len, *mins,
@@ -1278,15 +1278,20 @@ static lnbnn_status do_nbnn_classify(lnbnn_index* index, lnbnn_workspace* w, con
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallProfile prof(index, s);
   const int32_t C = index->n_classes;
-  CK(cudaMemsetAsync(totals, 0, sizeof(int64_t) * (size_t)n_images * C, s));
-  CK(launch_check_offsets(offsets, n_images, n_queries, index->dev_err, s));
-  prof.launched(1);
+  Begin begin;
+  begin.fill(totals, sizeof(int64_t) * (size_t)n_images * C, 0u);
+  begin.offsets = offsets;
+  begin.n_img = n_images;
+  begin.m = n_queries;
+  begin.dev_err = index->dev_err;
   if (n_queries == 0) {
+    CK(launch_begin(begin, s));
+    prof.launched(1);
     prof.mark(1);
     prof.mark(2);
   } else {
     int32_t* mins = nullptr;
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins);
     if (st != LNBNN_OK) return st;
     CK(launch_nbnn_sum(mins, n_queries, C, offsets, n_images, totals, s));
     prof.launched(1);
@@ -1309,16 +1314,21 @@ static lnbnn_status do_nbnn_logodds_classify(lnbnn_index* index, lnbnn_workspace
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallProfile prof(index, s);
   const int32_t C = index->n_classes;
-  CK(cudaMemsetAsync(totals, 0, sizeof(double) * (size_t)n_images * C, s));
-  if (n_increments) CK(cudaMemsetAsync(n_increments, 0, sizeof(int64_t) * (size_t)n_images, s));
-  CK(launch_check_offsets(offsets, n_images, n_queries, index->dev_err, s));
-  prof.launched(1);
+  Begin begin;
+  begin.fill(totals, sizeof(double) * (size_t)n_images * C, 0u);
+  if (n_increments) begin.fill(n_increments, sizeof(int64_t) * (size_t)n_images, 0u);
+  begin.offsets = offsets;
+  begin.n_img = n_images;
+  begin.m = n_queries;
+  begin.dev_err = index->dev_err;
   int32_t* mins = nullptr;
   if (n_queries == 0) {
+    CK(launch_begin(begin, s));
+    prof.launched(1);
     prof.mark(1);
     prof.mark(2);
   } else {
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, s, prof, &mins);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins);
     if (st != LNBNN_OK) return st;
     prof.launched(1);
   }

@@ -170,11 +170,12 @@ extern "C" LNBNN_API lnbnn_status knn_search_noalloc(const uint8_t* ref, int64_t
   // The array keeps the previous call's contents: the error word must start at
   // zero, the work counter too, and the rows' shared bounds above every
   // distance; every other buffer is written before it is read.
-  cudaError_t e = cudaMemsetAsync(err, 0, sizeof(uint32_t), s);
-  if (e == cudaSuccess && sched.queue) e = cudaMemsetAsync(sched.queue, 0, sizeof(uint32_t), s);
-  if (e == cudaSuccess && splits > 1) e = cudaMemsetAsync(row_thr, 0x7F, sizeof(int32_t) * (size_t)m_pad, s);
-  if (e == cudaSuccess) e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, nullptr, ref_ext, s);
-  if (e == cudaSuccess) e = launch_prep_query(queries, n_queries, m_pad, kDim, 0, nullptr, qbf, qext, s);
+  Begin begin;
+  begin.fill(err, sizeof(uint32_t), 0u);
+  if (sched.queue) begin.fill(sched.queue, sizeof(uint32_t), 0u);
+  if (splits > 1) begin.fill(row_thr, sizeof(int32_t) * (size_t)m_pad, 0x7F7F7F7Fu);
+  cudaError_t e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, nullptr, ref_ext, s);
+  if (e == cudaSuccess) e = launch_prep_query(queries, n_queries, m_pad, kDim, 0, qbf, qext, begin, s);
   if (e == cudaSuccess)
     e = launch_knn_tc(maps, false, qbf, qext, n_queries, m_pad, n_ref, (int)splits, split_len, k, lists, m_pad,
                       splits > 1 ? row_thr : nullptr, err, nullptr, nullptr, sched, s);

@@ -21,6 +21,7 @@
 // and w x_q' = 256 hx + lx (0 <= lx < 256, |hx| <= 24), so that the
 // location columns add -2 w (x_q' x_r' + y_q' y_r').  Every value is exact in
 // BF16.  Rows without a location (128 bytes) have zeros there.
+#include "begin.cuh"
 #include "internal.cuh"
 
 namespace lnbnn {
@@ -103,8 +104,12 @@ __device__ __forceinline__ void split256(int32_t v, int32_t* h, int32_t* l) {
 }
 
 __global__ void prep_query_kernel(const uint8_t* __restrict__ q, int64_t m, int64_t m_pad, int row_bytes, int loc_w,
-                                  int32_t* __restrict__ qnorm, __nv_bfloat16* __restrict__ qbf,
-                                  __nv_bfloat16* __restrict__ qext) {
+                                  __nv_bfloat16* __restrict__ qbf, __nv_bfloat16* __restrict__ qext,
+                                  const __grid_constant__ Begin begin, unsigned prep_blocks) {
+  if (blockIdx.x >= prep_blocks) {
+    begin_part(begin, blockIdx.x - prep_blocks, gridDim.x - prep_blocks);
+    return;
+  }
   const int sub = threadIdx.x % kThreadsPerRow;
   const int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.x / kThreadsPerRow;
   if (row >= m_pad) return;
@@ -120,7 +125,7 @@ __global__ void prep_query_kernel(const uint8_t* __restrict__ q, int64_t m, int6
     ss += x0 * x0 + x1 * x1;
     o[t] = pack_bf16x2(-2.0f * (float)x0, -2.0f * (float)x1);
   }
-  if (qbf) *reinterpret_cast<uint4*>(qbf + row * kDim + sub * 8) = out;
+  *reinterpret_cast<uint4*>(qbf + row * kDim + sub * 8) = out;
 #pragma unroll
   for (int off = kThreadsPerRow / 2; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
   if (sub != 0) return;
@@ -130,8 +135,6 @@ __global__ void prep_query_kernel(const uint8_t* __restrict__ q, int64_t m, int6
     ly = (int32_t)q[row * row_bytes + kDim + 1] - 128;
   }
   const int32_t norm = ss + loc_w * (lx * lx + ly * ly);
-  if (real && qnorm) qnorm[row] = norm;
-  if (!qext) return;
   int32_t hx, lox, hy, loy;
   split256(loc_w * lx, &hx, &lox);
   split256(loc_w * ly, &hy, &loy);
@@ -179,7 +182,18 @@ __global__ void fill_float_kernel(float* __restrict__ dst, int64_t n, float v) {
     dst[j] = v;
 }
 
+__global__ void begin_kernel(const __grid_constant__ Begin begin) { begin_part(begin, blockIdx.x, gridDim.x); }
+
+static_assert(kRowsPerBlock * kThreadsPerRow == kBeginThreads, "one block size for both parts");
+
 }  // namespace
+
+cudaError_t launch_begin(const Begin& begin, cudaStream_t s) {
+  const unsigned blocks = begin_blocks(begin);
+  if (blocks == 0) return cudaSuccess;
+  begin_kernel<<<blocks, kBeginThreads, 0, s>>>(begin);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_fill_float(float* dst, int64_t n, float v, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
@@ -198,13 +212,13 @@ cudaError_t launch_prep_ref(const uint8_t* ref, int64_t n_ref, int64_t n_pad, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_prep_query(const uint8_t* q, int64_t m, int64_t m_pad, int row_bytes, int loc_w, int32_t* qnorm,
-                              __nv_bfloat16* qbf, __nv_bfloat16* qext, cudaStream_t s) {
-  if (m_pad == 0) return cudaSuccess;
+cudaError_t launch_prep_query(const uint8_t* q, int64_t m, int64_t m_pad, int row_bytes, int loc_w, __nv_bfloat16* qbf,
+                              __nv_bfloat16* qext, const Begin& begin, cudaStream_t s) {
+  if (m_pad == 0) return launch_begin(begin, s);
   if (!row_layout_ok(row_bytes, loc_w)) return cudaErrorInvalidValue;
-  const int64_t blocks = (m_pad + kRowsPerBlock - 1) / kRowsPerBlock;
-  prep_query_kernel<<<(unsigned)blocks, kRowsPerBlock * kThreadsPerRow, 0, s>>>(q, m, m_pad, row_bytes, loc_w, qnorm,
-                                                                                 qbf, qext);
+  const unsigned blocks = (unsigned)((m_pad + kRowsPerBlock - 1) / kRowsPerBlock);
+  prep_query_kernel<<<blocks + begin_blocks(begin), kBeginThreads, 0, s>>>(q, m, m_pad, row_bytes, loc_w, qbf, qext,
+                                                                           begin, blocks);
   return cudaGetLastError();
 }
 

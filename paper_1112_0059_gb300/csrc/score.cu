@@ -1,5 +1,5 @@
-// Split merge, knn_search output, the Local NBNN class update (Alg. 2), the
-// offsets check and the per-image argmin (Alg. 1 and Alg. 2, last line).
+// Split merge, knn_search output, the Local NBNN class update (Alg. 2) and the
+// per-image argmin (Alg. 1 and Alg. 2, last line).
 #include <algorithm>
 
 #include "internal.cuh"
@@ -249,17 +249,6 @@ __global__ void nbnn_sum_kernel(const int32_t* __restrict__ mins, int64_t m, int
   }
 }
 
-__global__ void check_offsets_kernel(const int64_t* __restrict__ offsets, int64_t n_img, int64_t m,
-                                     uint32_t* __restrict__ dev_err) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > n_img) return;
-  bool bad = false;
-  if (i == 0) bad = offsets[0] != 0;
-  if (i == n_img) bad = bad || offsets[n_img] != m;
-  if (i < n_img) bad = bad || offsets[i + 1] < offsets[i];
-  if (bad) atomicOr(dev_err, kDevErrOffsets);
-}
-
 // One warp per image; lanes scan classes lane, lane+32, ...; ties -> lowest class.
 __global__ void argmin_kernel(const int64_t* __restrict__ totals, int64_t n_img, int32_t C,
                               int32_t* __restrict__ classes) {
@@ -342,12 +331,6 @@ cudaError_t launch_nbnn_sum(const int32_t* mins, int64_t m, int32_t C, const int
   if (n_img == 0 || m == 0) return cudaSuccess;
   dim3 grid((unsigned)((m + kSumRows - 1) / kSumRows), (unsigned)((C + 127) / 128));
   nbnn_sum_kernel<<<grid, 128, 0, s>>>(mins, m, C, offsets, n_img, totals);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_check_offsets(const int64_t* offsets, int64_t n_img, int64_t m, uint32_t* dev_err,
-                                 cudaStream_t s) {
-  check_offsets_kernel<<<(unsigned)((n_img + 1 + 255) / 256), 256, 0, s>>>(offsets, n_img, m, dev_err);
   return cudaGetLastError();
 }
 

@@ -67,3 +67,27 @@ def test_logodds_class_counts(lnbnn, C):
     tol = 33 * 8 * np.finfo(np.float64).eps * (beta * dmax + np.log(C)) * 16
     assert np.abs(lt.cpu().numpy() - ot).max() <= tol
     assert np.array_equal(ln.cpu().numpy(), np.diff(off) * C)
+
+
+@pytest.mark.parametrize("n_img", [1, 255, 4095, 4096, 9000])
+def test_totals_cleared_and_offsets_checked(lnbnn, n_img):
+    """Whatever the totals held before a call, and an image whose offset is out
+    of order in any part of the check."""
+    C = 7
+    sizes = [1] * 40 + [0] * (n_img - 40) if n_img > 1 else [40]
+    ref, labels, q, off = case(n_img, C, 400, sizes)
+    want = oracle.local_nbnn(ref, labels, C, q, off, 3)[0]
+    with lnbnn.Index(dev(ref), dev(labels), C) as ix:
+        buf = torch.full((n_img * C + 1,), -5, dtype=torch.int64, device="cuda")
+        cls = torch.empty(n_img, dtype=torch.int32, device="cuda")
+        t = buf[1:].view(n_img, C)  # 8-byte aligned only
+        for qq, oo in ((q, off), (q[:0], off * 0)):
+            t.fill_(-5)
+            ix.lnbnn_classify(dev(qq), dev(oo), 3, out=(t, cls))
+            ix.sync()
+            assert np.array_equal(t.cpu().numpy(), want if len(qq) else want * 0) and int(buf[0]) == -5
+        bad = off.copy()
+        bad[n_img - 1 if n_img > 1 else 1] = 41
+        ix.lnbnn_classify(dev(q), dev(bad), 3)
+        with pytest.raises(lnbnn.LnbnnError):
+            ix.sync()
