@@ -17,6 +17,7 @@
 
 #include "begin.cuh"
 #include "internal.cuh"
+#include "sqdist.cuh"
 
 namespace lnbnn {
 namespace {
@@ -95,26 +96,6 @@ __global__ void prep_e4m3_kernel(const uint8_t* __restrict__ x, int64_t n, int64
 
 constexpr int kRerankWarps = 8;
 constexpr int kMaxPerLane = (LNBNN_MAX_K + 1 + 31) / 32;  // shortlist entries per lane, at most
-
-// ||q - r||^2 over one 128-byte row, 16 bytes at a time.
-__device__ __forceinline__ uint32_t sqdist_u8(const uint4 (&q)[8], const uint8_t* __restrict__ r) {
-  uint32_t acc = 0;
-  const uint4* rv = reinterpret_cast<const uint4*>(r);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint4 b = __ldg(rv + i);
-    uint32_t d;
-    d = __vabsdiffu4(q[i].x, b.x);
-    acc = __dp4a(d, d, acc);
-    d = __vabsdiffu4(q[i].y, b.y);
-    acc = __dp4a(d, d, acc);
-    d = __vabsdiffu4(q[i].z, b.z);
-    acc = __dp4a(d, d, acc);
-    d = __vabsdiffu4(q[i].w, b.w);
-    acc = __dp4a(d, d, acc);
-  }
-  return acc;
-}
 
 __global__ void __launch_bounds__(32 * kRerankWarps)
     rerank_kernel(const uint64_t* __restrict__ shortlist, int64_t m, int M1, const uint8_t* __restrict__ q,

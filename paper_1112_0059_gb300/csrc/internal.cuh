@@ -119,6 +119,34 @@ cudaError_t launch_extract_knn(const uint64_t* lists, int64_t m, int K1, int k, 
 cudaError_t launch_lnbnn_score(const uint64_t* lists, int64_t m, int K1, int k, const int32_t* labels, int64_t n_ref,
                                const int64_t* offsets, int64_t n_img, int32_t C, int64_t* totals,
                                uint32_t* dev_err, cudaStream_t s);
+// After the scan, for lists of at most 32 keys: merge, rerank (rerank != null:
+// the shortlists' exact distances, K1 kept) and either the Alg. 2 update
+// (score != null) or the first k neighbours (idx, dist) in one launch.  The
+// update also takes the argmin where the totals are few and there is a counter
+// (one word, zero before the launch): *argmin_done says whether it does.
+struct RowLists {
+  const uint64_t* lists;  // list l of row i at lists + (l * stride + i) * K
+  int n_lists, K;
+  int64_t stride, m, n_ref;
+  MergeChain chain;
+};
+struct RowRerank {
+  const uint8_t* q;
+  const uint8_t* ref;
+  int K1;
+};
+struct RowScore {
+  const int32_t* labels;
+  const int64_t* offsets;
+  int64_t n_img;
+  int32_t C;
+  int64_t* totals;
+  uint32_t* dev_err;
+  int32_t* classes;
+  uint32_t* counter;
+};
+cudaError_t launch_row_end(const RowLists& in, const RowRerank* rerank, const RowScore* score, int32_t k, int32_t* idx,
+                           int32_t* dist, cudaStream_t s, bool* argmin_done);
 // Alg. 1 sum: totals[img][c] += sum of mins[row][c] over the image's rows.
 cudaError_t launch_nbnn_sum(const int32_t* mins, int64_t m, int32_t C, const int64_t* offsets, int64_t n_img,
                             int64_t* totals, cudaStream_t s);

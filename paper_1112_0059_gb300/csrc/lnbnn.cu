@@ -291,9 +291,10 @@ struct KnnPlan {
   bool seeded;          // each split's lists may start from the same rows' previous split's lists
   int group;            // > 0: the claimed-chunk form (`splits` = CTAs per query-tile group, split_len = chunk)
   int64_t items;        // work items of the launch (query-tile groups x splits)
+  bool lists_kept;      // a kNN scan
   bool bounded;         // several splits of a row share its bound
   int64_t work_slots;   // candidate buffers of lists in progress (one set per CTA)
-  size_t off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_slots, off_work, bytes;
+  size_t off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_count, off_slots, off_work, bytes;
   size_t sized;  // bytes of what grows with queries and list length (all but the candidate buffers)
   TcSched sched(char* ws, int sm_count) const {
     TcSched t;
@@ -316,6 +317,7 @@ struct KnnPlan {
     if (persistent) b->fill(ws + off_queue, sizeof(uint32_t) * (size_t)(group > 0 ? items / splits : 1), 0u);
     if (seeded) b->fill(ws + off_done, sizeof(uint32_t) * (size_t)items, 0u);
     if (items > work_slots && !persistent) b->fill(ws + off_slots, sizeof(uint32_t) * (size_t)work_slots, 0u);
+    if (lists_kept) b->fill(ws + off_count, sizeof(uint32_t), 0u);
     if (bounded) b->fill(ws + off_rowthr, sizeof(int32_t) * (size_t)m_pad, 0x7F7F7F7Fu);
   }
   // The merge's view of a seeded launch: rows whose last split holds every
@@ -391,12 +393,14 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.off_qbf = c.take<__nv_bfloat16>(p.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.m_pad * kExt);
   const bool knn = kind != ScanKind::Nbnn;
+  p.lists_kept = knn;
   p.bounded = knn && p.splits > 1;
   p.off_lists = c.take<uint64_t>(knn ? (size_t)p.splits * p.m_pad * K1 : 0);
   p.off_merged = c.take<uint64_t>(knn ? (size_t)p.m_pad * K1 : 0);  // apart from the lists (rerank)
   p.off_rowthr = c.take<int32_t>(p.m_pad);                // the bound a row's lists share
   p.off_queue = c.take<uint32_t>((size_t)T);             // the work counter(s) of a persistent launch
   p.off_done = c.take<uint32_t>((size_t)p.items);        // per-item "lists written" flags
+  p.off_count = c.take<uint32_t>(1);                      // blocks done (launch_row_end)
   p.sized = c.off;
   p.work_slots = knn ? std::min<int64_t>(p.items, P) : p.items;  // (none for NBNN, which keeps no lists)
   p.off_slots = c.take<uint32_t>((size_t)P);
@@ -478,9 +482,18 @@ lnbnn_status Scratch::admit(int64_t m, int K1) const {
   return b.sized > w->sized ? LNBNN_ERR_SCRATCH_LIMIT : LNBNN_OK;
 }
 
-// Runs the exact search; *lists receives m sorted lists of K1 keys.
-lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, cudaStream_t s,
-                     const uint64_t** lists, CallProfile& prof, Begin begin = Begin{}, int force_splits = 0) {
+// What a scan leaves: its plan, the call's scratch and the lists it wrote.
+struct Found {
+  KnnPlan p;
+  char* ws = nullptr;
+  uint64_t* part = nullptr;    // [splits][m_pad][K]
+  uint64_t* merged = nullptr;  // room for [m_pad][K]
+  int64_t m = 0;
+};
+
+// Runs the exact scan.
+lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, cudaStream_t s, Found* out,
+                     CallProfile& prof, Begin begin = Begin{}, int force_splits = 0) {
   KnnPlan p = plan_knn(ix, m, K1, ScanKind::Exact, force_splits);
   char* ws = nullptr;
   lnbnn_status st = scratch.admit(m, K1);
@@ -489,7 +502,6 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qext);
   uint64_t* part = reinterpret_cast<uint64_t*>(ws + p.off_lists);
-  uint64_t* merged = reinterpret_cast<uint64_t*>(ws + p.off_merged);
   int32_t* row_thr = reinterpret_cast<int32_t*>(ws + p.off_rowthr);
   Range range("lnbnn: exact k+1 search");
   p.begin(ws, &begin);
@@ -502,18 +514,13 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
                    ix->gate, sched, s));
   prof.launched(1, true);
   prof.mark(2);
-  if (p.splits > 1) {
-    CK(launch_merge_lists(part, p.splits, m, p.m_pad, K1, merged, s, p.chain(ws)));
-    prof.launched(1);
-  }
-  *lists = p.splits > 1 ? merged : part;
+  *out = Found{p, ws, part, reinterpret_cast<uint64_t*>(ws + p.off_merged), m};
   return LNBNN_OK;
 }
 
-// The FP8 shortlist search: coarse pass keeping the M1 smallest coarse keys,
-// merge, exact rerank; *lists receives m sorted lists of K1 exact keys.
-lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, int M1,
-                         cudaStream_t s, const uint64_t** lists, CallProfile& prof, Begin begin = Begin{}) {
+// The FP8 shortlist search's coarse pass, keeping the M1 smallest coarse keys.
+lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int M1, cudaStream_t s,
+                         Found* out, CallProfile& prof, Begin begin = Begin{}) {
   KnnPlan p = plan_knn(ix, m, M1, ScanKind::Coarse);
   char* ws = nullptr;
   lnbnn_status st = scratch.admit(m, M1);
@@ -523,7 +530,6 @@ lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, in
   uint8_t* qf8 = reinterpret_cast<uint8_t*>(ws + p.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qext);
   uint64_t* part = reinterpret_cast<uint64_t*>(ws + p.off_lists);
-  uint64_t* merged = reinterpret_cast<uint64_t*>(ws + p.off_merged);
   int32_t* row_thr = reinterpret_cast<int32_t*>(ws + p.off_rowthr);
   Range range("lnbnn: FP8 shortlist search");
   p.begin(ws, &begin);
@@ -536,18 +542,41 @@ lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, in
                       ix->gate, sched, s));
   prof.launched(1, true);
   prof.mark(2);
-  // the shortlist is the merged lists (or the one list); the reranked lists
-  // go to the other buffer
-  if (p.splits > 1) {
-    CK(launch_merge_lists(part, p.splits, m, p.m_pad, M1, merged, s, p.chain(ws)));
-    CK(launch_rerank(merged, m, M1, q, ix->ref_u8, ix->n_ref, K1, part, s));
-    prof.launched(2);
-    *lists = part;
-  } else {
-    CK(launch_rerank(part, m, M1, q, ix->ref_u8, ix->n_ref, K1, merged, s));
+  *out = Found{p, ws, part, reinterpret_cast<uint64_t*>(ws + p.off_merged), m};
+  return LNBNN_OK;
+}
+
+// Merge, rerank and the update or the neighbours of a scan's lists: one launch
+// for lists of at most 32 keys, separate steps for longer ones.  K1 exact keys
+// per row are needed (the list length itself without a rerank).
+lnbnn_status finish_rows(lnbnn_index* ix, const Found& f, const uint8_t* rerank_q, int K1, const RowScore* score,
+                         int32_t k, int32_t* idx, int32_t* dist, cudaStream_t s, CallProfile& prof, bool* argmin_done) {
+  const int K = f.p.K1;
+  if (K <= 32) {
+    const RowLists in{f.part, f.p.splits, K, f.p.m_pad, f.m, ix->n_ref, f.p.chain(f.ws)};
+    const RowRerank rr{rerank_q, ix->ref_u8, K1};
+    CK(launch_row_end(in, rerank_q ? &rr : nullptr, score, k, idx, dist, s, argmin_done));
     prof.launched(1);
-    *lists = merged;
+    return LNBNN_OK;
   }
+  const uint64_t* lists = f.part;
+  if (f.p.splits > 1) {
+    CK(launch_merge_lists(f.part, f.p.splits, f.m, f.p.m_pad, K, f.merged, s, f.p.chain(f.ws)));
+    prof.launched(1);
+    lists = f.merged;
+  }
+  if (rerank_q) {  // the reranked lists go to the other buffer
+    uint64_t* to = f.p.splits > 1 ? f.part : f.merged;
+    CK(launch_rerank(lists, f.m, K, rerank_q, ix->ref_u8, ix->n_ref, K1, to, s));
+    prof.launched(1);
+    lists = to;
+  }
+  if (score)
+    CK(launch_lnbnn_score(lists, f.m, K1, k, score->labels, ix->n_ref, score->offsets, score->n_img, score->C,
+                          score->totals, score->dev_err, s));
+  else
+    CK(launch_extract_knn(lists, f.m, K1, k, idx, dist, s));
+  prof.launched(1);
   return LNBNN_OK;
 }
 
@@ -1007,8 +1036,11 @@ lnbnn_status lnbnn_autotune(lnbnn_index* index, void* stream, lnbnn_tuning* out)
     st = time_call([&]() {
       Scratch scratch{index, &w};
       CallProfile prof(index, s);
-      const uint64_t* lists = nullptr;
-      return run_knn(index, scratch, q, r.T * kTcQueryTile, r.K1, s, &lists, prof, Begin{}, (int)r.splits);
+      Found found;
+      const lnbnn_status rs = run_knn(index, scratch, q, r.T * kTcQueryTile, r.K1, s, &found, prof, Begin{}, (int)r.splits);
+      if (rs == LNBNN_OK && found.p.splits > 1)
+        CK(launch_merge_lists(found.part, found.p.splits, found.m, found.p.m_pad, r.K1, found.merged, s));
+      return rs;
     }, &r.ms);
     if (st != LNBNN_OK) {
       cleanup();
@@ -1021,10 +1053,9 @@ lnbnn_status lnbnn_autotune(lnbnn_index* index, void* stream, lnbnn_tuning* out)
     st = time_call([&]() {
       Scratch scratch{index, &w};
       CallProfile prof(index, s);
-      const uint64_t* lists = nullptr;
-      return f.kind == ScanKind::Coarse
-                 ? run_knn_fp8(index, scratch, q, t_big * kTcQueryTile, 11, 32, s, &lists, prof)
-                 : run_knn(index, scratch, q, t_big * kTcQueryTile, 11, s, &lists, prof);
+      Found found;
+      return f.kind == ScanKind::Coarse ? run_knn_fp8(index, scratch, q, t_big * kTcQueryTile, 32, s, &found, prof)
+                                        : run_knn(index, scratch, q, t_big * kTcQueryTile, 11, s, &found, prof);
     }, &f.ms);
     if (st != LNBNN_OK) {
       cleanup();
@@ -1166,12 +1197,10 @@ static lnbnn_status do_knn_search(lnbnn_index* index, lnbnn_workspace* w, const 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallProfile prof(index, s);
   Scratch scratch{index, w};
-  const uint64_t* lists = nullptr;
-  lnbnn_status st = run_knn(index, scratch, queries, n_queries, k, s, &lists, prof);
+  Found found;
+  lnbnn_status st = run_knn(index, scratch, queries, n_queries, k, s, &found, prof);
   if (st != LNBNN_OK) return st;
-  CK(launch_extract_knn(lists, n_queries, k, k, idx, dist, s));
-  prof.launched(1);
-  return LNBNN_OK;
+  return finish_rows(index, found, nullptr, k, nullptr, k, idx, dist, s, prof, nullptr);
 }
 
 static lnbnn_status do_knn_search_fp8(lnbnn_index* index, lnbnn_workspace* w, const uint8_t* queries,
@@ -1187,12 +1216,10 @@ static lnbnn_status do_knn_search_fp8(lnbnn_index* index, lnbnn_workspace* w, co
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallProfile prof(index, s);
   Scratch scratch{index, w};
-  const uint64_t* lists = nullptr;
-  lnbnn_status st = run_knn_fp8(index, scratch, queries, n_queries, k, M1, s, &lists, prof);
+  Found found;
+  lnbnn_status st = run_knn_fp8(index, scratch, queries, n_queries, M1, s, &found, prof);
   if (st != LNBNN_OK) return st;
-  CK(launch_extract_knn(lists, n_queries, k, k, idx, dist, s));
-  prof.launched(1);
-  return LNBNN_OK;
+  return finish_rows(index, found, queries, k, nullptr, k, idx, dist, s, prof, nullptr);
 }
 
 // shortlist = 0: exact search; otherwise the FP8 shortlist search.
@@ -1218,21 +1245,25 @@ static lnbnn_status do_lnbnn_classify(lnbnn_index* index, lnbnn_workspace* w, co
   begin.n_img = n_images;
   begin.m = n_queries;
   begin.dev_err = index->dev_err;
+  bool argmin_done = false;
   if (n_queries > 0) {
     Scratch scratch{index, w};
-    const uint64_t* lists = nullptr;
-    lnbnn_status st = shortlist ? run_knn_fp8(index, scratch, queries, n_queries, k + 1, M1, s, &lists, prof, begin)
-                                : run_knn(index, scratch, queries, n_queries, k + 1, s, &lists, prof, begin);
+    Found found;
+    lnbnn_status st = shortlist ? run_knn_fp8(index, scratch, queries, n_queries, M1, s, &found, prof, begin)
+                                : run_knn(index, scratch, queries, n_queries, k + 1, s, &found, prof, begin);
     if (st != LNBNN_OK) return st;
-    CK(launch_lnbnn_score(lists, n_queries, k + 1, k, index->labels, index->n_ref, offsets, n_images, C, totals,
-                          index->dev_err, s));
-    prof.launched(1);
+    const RowScore score{index->labels, offsets, n_images, C, totals, index->dev_err, classes,
+                         reinterpret_cast<uint32_t*>(found.ws + found.p.off_count)};
+    st = finish_rows(index, found, shortlist ? queries : nullptr, k + 1, &score, k, nullptr, nullptr, s, prof,
+                     &argmin_done);
+    if (st != LNBNN_OK) return st;
   } else {
     CK(launch_begin(begin, s));
     prof.launched(1);
     prof.mark(1);
     prof.mark(2);
   }
+  if (argmin_done) return LNBNN_OK;
   CK(launch_argmin(totals, n_images, C, classes, s));
   prof.launched(1);
   return LNBNN_OK;
