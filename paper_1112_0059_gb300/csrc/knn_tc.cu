@@ -265,7 +265,7 @@ __device__ __forceinline__ void release_slot(const ScanOut& out, int32_t s) {
 // list ends with, since keys are compared by (distance, row) and a column at
 // the limit passes.  Measured, whole calls before and after (one GB300):
 // 101-class data, 200k rows, k = 50 121.6 / 64.2 ms; 256-class data, 15k rows,
-// k = 100 95.0 / 37.5 ms, FP8 shortlist 128 84.5 / 28.0 ms, shortlist 24 on
+// k = 100 95.0 / 32.9 ms, FP8 shortlist 128 84.5 / 27.2 ms, shortlist 24 on
 // one image of 632 rows 1.31 / 0.90 ms.
 //
 // The lists of a row in other reference splits share a bound with it:
@@ -428,9 +428,9 @@ struct Inserter {
       const uint32_t rows = __ballot_sync(0xffffffffu, keys > 0);
       const uint64_t* packed = reinterpret_cast<const uint64_t*>(from);
       if (K1 <= 128) {
-        kth[q] = merge_rows<4, 2>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
+        kth[q] = merge_rows<4>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
       } else {
-        kth[q] = merge_rows<8, 1>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
+        kth[q] = merge_rows<8>(packed, stride / 2, keys, list[q], seed[q], rows, listed[q], K1, kth[q]);
       }
       listed[q] |= rows;
     }
@@ -1000,7 +1000,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
       e.cap = (uint32_t)out.entries;
       e.mine = out.work + max(*work_slot, 0) * tc_work_bytes(out.entries) + (int64_t)t * 2 * out.entries * kTcEntryBytes;
       e.start = e.mine;
-      e.soft = (uint32_t)min(Epilogue::KMAX > 0 ? 8 : 32, out.entries - 8);
+      e.soft = (uint32_t)min(8, out.entries - 8);
       e.abort_flag = abort_flag;
       e.dev_err = dev_err;
     }

@@ -93,154 +93,137 @@ struct RegList {
 template <>
 struct RegList<0> {};
 
-// A bitonic stage between elements `stride` >= 32 apart: registers of one lane.
-template <int S, int R, typename Key>
-__device__ __forceinline__ void between_registers(Key (&k)[R][S], int size, int stride) {
-#pragma unroll
-  for (int d = S / 2; d > 0; d >>= 1) {
-    if (stride == 32 * d) {
-#pragma unroll
-      for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-          if ((s & d) == 0) {
-            const bool up = ((32 * s) & size) == 0;
-            const Key a = k[i][s], b = k[i][s | d];
-            const bool keep = (a < b) == up;
-            k[i][s] = keep ? a : b;
-            k[i][s | d] = keep ? b : a;
-          }
-    }
-  }
-}
-
 // Candidate entries: eight neighbouring columns' distance bits, then the first
 // one's column (row of the references).
 constexpr int kEntryWords = 16;
 
 // Merges the rows of the mask `rows` (row r < 32; its counters and result are
 // lane r's): n candidates at cand + r * cand_stride, (row, distance bits)
-// pairs in increasing row order, into the K1 smallest (distance, row) keys, ascending,
-// at list + r * K1.  The list holds keys already where `listed` has the row;
+// pairs, into the K1 <= 32 S smallest (distance, row) keys, ascending, at
+// list + r * K1.  The list holds keys already where `listed` has the row;
 // otherwise it starts from seed + r * K1 if there is a seed, or empty.
 // Returns the bits of the lane's row's K1-th distance (INT32_MAX: not full),
 // `kth` for rows not merged.
 //
-// R rows at a time: the candidates are sorted bitonically, N = 32 S at a time,
-// and the smaller half of list and candidates merged; lane l holds elements l,
-// l + 32, ...  The sort runs on 32-bit keys (a distance is below 2^24, so it
-// has room for the candidate's place), a shuffle and a minimum or maximum per
-// key and stage; candidates must therefore come in increasing row order among
-// equal distances.  Only the merge compares 64-bit (distance, row) keys: the
-// list may hold rows from other columns.  A stage waits on its shuffle, so R
-// rows share it.  The stages run in rolled loops and the function is not
-// inlined: straight-line code past what the instruction cache holds (about
-// 10 KB for all roles of the scan kernel) runs at a third of the speed (6
-// cycles an instruction against 2 measured on one warp).
-template <int S, int R>
+// One row after another, by counting: lane l holds the list's keys l, l + 32,
+// ... and candidate l of (up to) 32.  Each candidate in turn is shown to every
+// lane, which counts it for those of its keys that it sorts before; a key's new
+// place is its old one plus its count, a candidate's the number of list keys
+// (summed over the lanes by one reduction) and candidates before it.  A row has
+// ten or so candidates when its warp's buffers come, so this is less than a
+// bitonic sort and merge of 32 S keys, which took 3,900 cycles a row whatever
+// their number: 256-class data, 15k rows, k = 100 35.7 / 32.9 ms, FP8 shortlist
+// 128 28.4 / 27.2 ms.  Of about 2,600 cycles a row, 900 wait for the row's keys
+// (from L2; the next row's are loaded meanwhile, but the operands stream at the
+// same time and shared memory leaves L1 28 KB), 1,300 show the candidates (a
+// shuffle waits its turn behind the MMAs' operand reads, so four are shown at a
+// time: one at a time 34.9 ms, eight 33.3) and 440 store.  Straight-line code
+// past what the instruction cache holds (about 10 KB for all roles of the scan
+// kernel) runs at a third of the speed (6 cycles an instruction against 2
+// measured on one warp), so the function is rolled and not inlined.
+template <int S>
 __device__ __noinline__ int32_t merge_rows(const uint64_t* cand, int cand_stride, int n_cand, uint64_t* list,
                                            const uint64_t* seed, uint32_t rows, uint32_t listed, int K1, int32_t kth) {
-  constexpr int N = 32 * S;
+  constexpr int W = (S + 3) / 4;  // words of four 8-bit counts
+  constexpr int U = 4;            // candidates shown at a time
   const int lane = threadIdx.x & 31;
-  while (rows != 0u) {
-    int row[R], n[R], most = 0;
-    uint64_t l[R][S];
+  uint64_t l[S], next_l[S], c = 0, next_c = 0;
+  int row = -1, n = 0, next_n = 0;
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      row[i] = __ffs(rows) - 1;  // -1: fewer than R rows are left
+  for (int s = 0; s < S; ++s) l[s] = next_l[s] = kEmptyKey;
+#pragma unroll 1
+  do {
+    const int next = __ffs(rows) - 1;  // -1: no row is left
+    if (next >= 0) {
       rows &= rows - 1;
-      n[i] = row[i] < 0 ? 0 : __shfl_sync(0xffffffffu, n_cand, row[i] & 31);
-      most = max(most, n[i]);
-      const uint64_t* src = row[i] < 0                       ? nullptr
-                            : ((listed >> row[i]) & 1u) != 0 ? list + row[i] * K1
-                            : seed != nullptr                ? seed + row[i] * K1
-                                                             : nullptr;
+      next_n = __shfl_sync(0xffffffffu, n_cand, next);
+      const uint64_t* src = ((listed >> next) & 1u) != 0 ? list + next * K1 : seed != nullptr ? seed + next * K1 : nullptr;
 #pragma unroll
       for (int s = 0; s < S; ++s)
-        l[i][s] = src != nullptr && lane + 32 * s < K1 ? ld_global_u64(src + lane + 32 * s) : kEmptyKey;
+        next_l[s] = src != nullptr && lane + 32 * s < K1 ? ld_global_u64(src + lane + 32 * s) : kEmptyKey;
+      next_c = lane < next_n ? ld_global_u64(cand + (int64_t)next * cand_stride + lane) : 0;
     }
+    if (row >= 0) {
+      uint64_t* to = list + row * K1;
+      bool all = ((listed >> row) & 1u) == 0;  // nothing is written yet
 #pragma unroll 1
-    for (int off = 0; off < most; off += N) {
-      uint32_t c[R][S];
-#pragma unroll
-      for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int e = lane + 32 * s;
-          c[i][s] = 0xFFFFFFFFu;
-          if (off + e < n[i]) {
-            const uint32_t d = bits_dist((uint32_t)(ld_global_u64(cand + (int64_t)row[i] * cand_stride + off + e) >> 32));
-            if (d < kDistLimit) c[i][s] = (d << 8) | (uint32_t)e;  // (a padding row's distance is above it)
-          }
+      for (int off = 0;;) {
+        uint64_t key = kEmptyKey;
+        if (off + lane < n) {
+          const uint32_t d = bits_dist((uint32_t)(c >> 32));
+          if (d < kDistLimit) key = make_key(d, (uint32_t)c);  // (a padding row's distance is above it)
         }
-      // the first power of two that holds them all is sorted; the rest of c is
-      // empty, above all, and stays where it is
-      int span = 32;
-      while (span < N && span < most - off) span <<= 1;
-#pragma unroll 1
-      for (int size = 2; size <= span; size <<= 1) {
-#pragma unroll 1
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-          if (S > 1 && stride >= 32) {
-            between_registers<S, R>(c, size, stride);
-          } else {
+        const int shown = min(n - off, 32);
+        uint32_t count[W], above = 0;
+        int rank = 0;
 #pragma unroll
-            for (int s = 0; s < S; ++s) {
-              if (s > 0 && 32 * s >= span) break;
-              const bool low = ((lane & stride) == 0) == (((lane + 32 * s) & size) == 0);
+        for (int w = 0; w < W; ++w) count[w] = 0;
+#pragma unroll 1
+        for (int j = 0; j < shown; j += U) {
+          uint64_t x[U];
+          uint32_t one[U][W], g[U];
 #pragma unroll
-              for (int i = 0; i < R; ++i) {
-                const uint32_t o = __shfl_xor_sync(0xffffffffu, c[i][s], stride);
-                c[i][s] = low ? min(c[i][s], o) : max(c[i][s], o);
-              }
+          for (int u = 0; u < U; ++u) x[u] = __shfl_sync(0xffffffffu, key, j + u);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            rank += x[u] < key;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+              one[u][w] = 0;
+#pragma unroll
+              for (int s = 4 * w; s < min(S, 4 * w + 4); ++s)
+                if (x[u] < l[s]) one[u][w] += 1u << (8 * (s & 3));
+              count[w] += one[u][w];
             }
           }
-        }
-      }
-      // both ascending: element e of the list against element N - 1 - e of the
-      // candidates leaves the N smallest, as a bitonic sequence
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        uint64_t k[S];
+          for (int u = 0; u < U; ++u) {
+            g[u] = 0;  // list keys that x sorts before
+#pragma unroll
+            for (int w = 0; w < W; ++w) g[u] = __dp4a(__reduce_add_sync(0xffffffffu, one[u][w]), 0x01010101u, g[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (lane == j + u) above = g[u];
+        }
+        // a place for every key: nothing moves before the first candidate's
+        uint32_t last = 0;
+        bool at_end = false;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
-          const uint32_t o = __shfl_xor_sync(0xffffffffu, c[i][S - 1 - s], 31);
-          k[s] = kEmptyKey;
-          if (o != 0xFFFFFFFFu)
-            k[s] = make_key(o >> 8, (uint32_t)ld_global_u64(cand + (int64_t)row[i] * cand_stride + off + (o & 255u)));
+          const int by = (int)((count[s / 4] >> (8 * (s & 3))) & 255u), at = lane + 32 * s + by;
+          if (at < K1 && (all || by > 0)) to[at] = l[s];
+          if (at == K1 - 1) {
+            at_end = true;
+            last = (uint32_t)(l[s] >> 32);
+          }
         }
-#pragma unroll
-        for (int s = 0; s < S; ++s) l[i][s] = min(l[i][s], k[s]);
-      }
-#pragma unroll 1
-      for (int stride = N >> 1; stride > 0; stride >>= 1) {
-        if (S > 1 && stride >= 32) {
-          between_registers<S, R>(l, 2 * N, stride);
-        } else {
-          const bool low = (lane & stride) == 0;
-#pragma unroll
-          for (int s = 0; s < S; ++s)
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-              const uint64_t o = __shfl_xor_sync(0xffffffffu, l[i][s], stride);
-              l[i][s] = (l[i][s] < o) == low ? l[i][s] : o;
-            }
+        const int at = 32 * S - (int)above + rank;
+        if (key != kEmptyKey && at < K1) {
+          to[at] = key;
+          if (at == K1 - 1) {
+            at_end = true;
+            last = (uint32_t)(key >> 32);
+          }
         }
+        const uint32_t holder = __ballot_sync(0xffffffffu, at_end);
+        const uint32_t d = __shfl_sync(0xffffffffu, last, __ffs(holder) - 1);
+        if (lane == row) kth = d == 0xFFFFFFFFu ? INT32_MAX : dist_bits(d);
+        off += 32;
+        if (off >= n) break;
+        __syncwarp();
+        all = false;
+#pragma unroll
+        for (int s = 0; s < S; ++s) l[s] = lane + 32 * s < K1 ? ld_global_u64(to + lane + 32 * s) : kEmptyKey;
+        if (off + lane < n) c = ld_global_u64(cand + (int64_t)row * cand_stride + off + lane);
       }
     }
+    row = next;
+    n = next_n;
+    c = next_c;
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      if (row[i] < 0) continue;
-      uint64_t last = kEmptyKey;
-#pragma unroll
-      for (int s = 0; s < S; ++s) {
-        if (lane + 32 * s < K1) list[row[i] * K1 + lane + 32 * s] = l[i][s];
-        if ((K1 - 1) >> 5 == s) last = l[i][s];
-      }
-      const uint32_t d = __shfl_sync(0xffffffffu, (uint32_t)(last >> 32), (K1 - 1) & 31);
-      if (lane == row[i]) kth = d == 0xFFFFFFFFu ? INT32_MAX : dist_bits(d);
-    }
-  }
+    for (int s = 0; s < S; ++s) l[s] = next_l[s];
+  } while (row >= 0);
   __syncwarp();
   return kth;
 }
