@@ -264,9 +264,9 @@ __device__ __forceinline__ void release_slot(const ScanOut& out, int32_t s) {
 // read late: that changes which columns are appended, never which K1 keys the
 // list ends with, since keys are compared by (distance, row) and a column at
 // the limit passes.  Measured, whole calls before and after (one GB300):
-// 101-class data, 200k rows, k = 50 121.6 / 64.2 ms; 256-class data, 15k rows,
-// k = 100 95.0 / 32.9 ms, FP8 shortlist 128 84.5 / 27.2 ms, shortlist 24 on
-// one image of 632 rows 1.31 / 0.90 ms.
+// 101-class data, 200k rows, k = 50 121.6 / 60.5 ms; 256-class data, 15k rows,
+// k = 100 95.0 / 32.5 ms, FP8 shortlist 128 84.5 / 26.2 ms, shortlist 24 on
+// one image of 632 rows 1.31 / 0.83 ms (all steps together).
 //
 // The lists of a row in other reference splits share a bound with it:
 // row_thr[row] holds the bit pattern of a distance at or below which some list
@@ -280,24 +280,45 @@ __device__ __forceinline__ void release_slot(const ScanOut& out, int32_t s) {
 // of the row never are, so the merged result does not.
 //
 // Warm-up: a list that starts empty would copy every column until its first
-// merge.  So the first `warm_tiles` tiles of an item are run twice, first for
-// a limit alone: their columns fall into at least K1 groups (the row's columns
-// of one tile and column half, or of 32 columns where the item is short), each
-// group's least value is the distance of another column, and the largest of
-// them therefore bounds the K1-th smallest distance.
+// merge.  So the first tiles of an item are run twice, first for a limit alone:
+// the columns fall into groups of 32, each group's least value is the distance
+// of another column, and so the K1-th smallest of these minima bounds the K1-th
+// smallest distance.  A thread keeps the least ceil(K1 / 2) minima of its column
+// half sorted (QT = 2: K1), and the larger of the two halves' last ones is the
+// limit ("ranked").  Lists too long for that take the largest minimum of
+// exactly as many groups, of a tile's column half where the item is long
+// enough.
 constexpr int32_t kNoBound = 0x7F7F7F7F;  // row_thr's initial value: above every distance
 
 struct WarmUp {
-  int tiles;  // tiles run twice
-  bool fine;  // groups of 32 columns
+  int tiles;     // tiles run twice
+  bool fine;     // groups of 32 columns
+  bool ranked;   // the limit is the K1-th (per column half) smallest of the minima
 };
-template <int QT>
+// How many minima a thread can keep sorted, for the ranked limit.
+template <int KMAX, int QT>
+constexpr int kRankedMax = KMAX > 0 ? KMAX * QT / 2 : QT == 1 ? 64 : 0;
+template <int KMAX, int QT, bool Claim>
 __device__ __forceinline__ WarmUp warm_up(int ntiles, int K1) {
   constexpr int kHalves = QT == 2 ? 1 : 2;  // column halves of a row per tile
   const int wide = (K1 + kHalves - 1) / kHalves, fine = (K1 + 4 * kHalves - 1) / (4 * kHalves);
-  if (ntiles >= 2 * wide) return {wide, false};
-  if (ntiles >= fine) return {fine, true};
-  return {0, false};
+  if (ntiles < fine) return {0, false, false};
+  if (wide <= kRankedMax<KMAX, QT>) {
+    // A tile more costs a step; twice as many save K1 ln 2 candidates a row,
+    // which cost more the longer the list.  Whole calls (one GB300), against
+    // the largest minimum of ceil(K1 / 2) tiles: 2,000 queries x 5,000 rows
+    // 81 / 68 us; FP8 shortlist 24, one image of 632 rows, K1 / 4, K1 / 2, K1
+    // and 2 K1 tiles 802, 780, 777 and 786 us (before: 802); 3-NN with
+    // locations 855 / 830 us; k = 50, 200k rows x 1.5 million, K1 / 4, K1, 4 K1
+    // and 8 K1 tiles of 5,918 63.4, 61.7, 61.7 and 56.3 ms (63.8), one image
+    // against 11.5 million (items of 1,500 tiles) 102, 204 and 375 tiles 1.38,
+    // 1.48 and 1.59 ms (1.50); k = 100, 15k rows, items of 9,000 tiles, 2 K1,
+    // 4 K1 and 8 K1 tiles 32.3, 31.8 and 32.5 ms (32.9), FP8 shortlist 128
+    // 26.5, 26.8 and 27.7 ms (27.2).
+    const int want = K1 <= 32 ? K1 : (K1 <= 64 ? 8 : 3) * K1;
+    return {max(fine, min(want, ntiles / (Claim || K1 <= 32 ? 4 : 16))), true, true};
+  }
+  return ntiles >= 2 * wide ? WarmUp{wide, false, false} : WarmUp{fine, true, false};
 }
 
 // Shared memory of the hand-over between epilogue and inserter warps.
@@ -759,8 +780,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   // The tiles run twice at the start of this CTA's item i: none where the
   // lists go on from the previous chunk or split.
   auto warm_tiles = [&](int i, int64_t w, int ntiles) -> WarmUp {
-    if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false};
-    return warm_up<QT>(ntiles, out.K1);
+    if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false, false};
+    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1);
   };
 
   if (warp < kEpiWarp0) {
@@ -1017,6 +1038,11 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
       if constexpr (kAsync) {
         if (!Claim || i == 0) {
           const WarmUp wu = warm_tiles(i, w, ntiles);
+          // ranked: the least minima, sorted, behind slots that nothing displaces
+          constexpr int kRanked = kRankedMax<Epilogue::KMAX, QT>;
+          int32_t ranked[kRanked > 0 ? kRanked : 1];
+#pragma unroll
+          for (int j = 0; j < kRanked; ++j) ranked[j] = j < kRanked - (out.K1 * QT + 1) / 2 ? INT32_MIN : INT32_MAX;
           int32_t most = wu.tiles > 0 ? INT32_MIN : INT32_MAX;
           bool ok = true;
           for (int u = 0; u < wu.tiles; ++u, ++tg) {
@@ -1028,12 +1054,19 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
               uint32_t v[32], mn;
               tmem_ld_min_32x32b_x32(taddr + c, v, mn);
               tmem_ld_wait(v, mn);
-              if (wu.fine) most = max(most, (int32_t)mn);
-              least = min(least, (int32_t)mn);
+              if (kRanked > 0 && wu.ranked) {
+#pragma unroll
+                for (int j = kRanked - 1; j > 0; --j) ranked[j] = max(ranked[j - 1], min(ranked[j], (int32_t)mn));
+                ranked[0] = min(ranked[0], (int32_t)mn);
+              } else {
+                if (wu.fine) most = max(most, (int32_t)mn);
+                least = min(least, (int32_t)mn);
+              }
             }
             release_tile();
             if (!wu.fine) most = max(most, least);
           }
+          if (kRanked > 0 && wu.ranked) most = ranked[kRanked - 1];
           if (!ok) break;
           st_shared_u32(ho.warm(t), (uint32_t)most);
           __syncwarp();

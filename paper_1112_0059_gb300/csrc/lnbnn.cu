@@ -372,7 +372,9 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   if (p.group > 0) {
     const int64_t tiles = ref_tiles;
     const int64_t chunk_tiles = std::max<int64_t>(4, (tiles + 8 * (int64_t)p.group - 1) / (8 * (int64_t)p.group));
-    p.split_len = chunk_tiles * kTcRefTile;  // about eight chunks per CTA
+    // about eight chunks per CTA (sixteen: shortlist 24, 632 descriptors 780 / 799 us,
+    // 100 descriptors 328 / 348 us)
+    p.split_len = chunk_tiles * kTcRefTile;
     p.splits = p.group;
     p.persistent = true;
     p.bound_per_tile = true;
