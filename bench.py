@@ -680,7 +680,7 @@ def run_sections(sections, index, ref, labels, k, m) -> dict:
 
 
 def list_kind(K1: int) -> int:
-    """Register-list size the search kernel uses for lists of K1 (0: heap)."""
+    """Register-list size the search kernel uses for lists of K1 (0: lists in global memory)."""
     return 16 if K1 <= 16 else 24 if K1 <= 24 else 32 if K1 <= 32 else 64 if K1 <= 64 else 0
 
 

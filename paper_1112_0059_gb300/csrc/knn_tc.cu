@@ -308,8 +308,8 @@ __device__ __forceinline__ WarmUp warm_up(int ntiles, int K1) {
     // which cost more the longer the list.  Whole calls (one GB300), against
     // the largest minimum of ceil(K1 / 2) tiles: 2,000 queries x 5,000 rows
     // 81 / 68 us; FP8 shortlist 24, one image of 632 rows, K1 / 4, K1 / 2, K1
-    // and 2 K1 tiles 802, 780, 777 and 786 us (before: 802); 3-NN with
-    // locations 855 / 830 us; k = 50, 200k rows x 1.5 million, K1 / 4, K1, 4 K1
+    // and 2 K1 tiles 802, 780, 777 and 786 us (before: 802); 20-NN of 3,001 rows
+    // with locations 855 / 830 us; k = 50, 200k rows x 1.5 million, K1 / 4, K1, 4 K1
     // and 8 K1 tiles of 5,918 63.4, 61.7, 61.7 and 56.3 ms (63.8), one image
     // against 11.5 million (items of 1,500 tiles) 102, 204 and 375 tiles 1.38,
     // 1.48 and 1.59 ms (1.50); k = 100, 15k rows, items of 9,000 tiles, 2 K1,

@@ -270,8 +270,8 @@ __global__ void __launch_bounds__(32 * kScoreWarps)
 // once, the next ones as the list advances.  As kernels of their own (merge,
 // rerank, update, argmin) each waited for a launch and for the lists from
 // memory again: whole calls took, before and after, 2,000 queries against 5,000
-// rows 85 / 76 us, 64 images against 1.5 million rows 1,414 / 1,388 us, 1,000
-// queries against 11.5 million 508 / 502 us.
+// rows 85 / 76 us, 5 images of 400 to 1,601 from host memory against 1.5 million
+// rows 1,414 / 1,388 us, one image of 100 against 11.5 million 508 / 502 us.
 //
 // kScore: the last block of the launch (a counter zeroed before it) also takes
 // the argmin of every image when the totals are few.
