@@ -314,8 +314,12 @@ __device__ __forceinline__ WarmUp warm_up(int ntiles, int K1) {
     // against 11.5 million (items of 1,500 tiles) 102, 204 and 375 tiles 1.38,
     // 1.48 and 1.59 ms (1.50); k = 100, 15k rows, items of 9,000 tiles, 2 K1,
     // 4 K1 and 8 K1 tiles 32.3, 31.8 and 32.5 ms (32.9), FP8 shortlist 128
-    // 26.5, 26.8 and 27.7 ms (27.2).
-    const int want = K1 <= 32 ? K1 : (K1 <= 64 ? 8 : 3) * K1;
+    // 26.5, 26.8 and 27.7 ms (27.2).  At least 16 tiles, and hand-overs from two
+    // entries on for lists of less than 8 keys: 37,271 queries x 27,412 rows
+    // (items of 107 tiles), k = 1, 2, 5 and 10 476, 503, 546 and 598 us with K1
+    // tiles, 451, 488, 542 and 584 us with at least 8, 397, 449, 499 and 573 us
+    // with at least 16.
+    const int want = K1 <= 32 ? max(K1, 16) : (K1 <= 64 ? 8 : 3) * K1;
     return {max(fine, min(want, ntiles / (Claim || K1 <= 32 ? 4 : 16))), true, true};
   }
   return ntiles >= 2 * wide ? WarmUp{wide, false, false} : WarmUp{fine, true, false};
@@ -1021,7 +1025,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
       e.cap = (uint32_t)out.entries;
       e.mine = out.work + max(*work_slot, 0) * tc_work_bytes(out.entries) + (int64_t)t * 2 * out.entries * kTcEntryBytes;
       e.start = e.mine;
-      e.soft = (uint32_t)min(8, out.entries - 8);
+      e.soft = (uint32_t)min(out.K1 < 8 ? 2 : 8, out.entries - 8);
       e.abort_flag = abort_flag;
       e.dev_err = dev_err;
     }
