@@ -360,13 +360,14 @@ struct Collector {
   int32_t lim = INT32_MIN;  // a column enters below it (bit pattern)
   __device__ __forceinline__ void read_limit() { lim = (int32_t)ld_shared_u32(lim_at); }
   // Hands the warp's buffers over and goes on with the other ones, once the
-  // hand-over before has been merged (without `wait`: only if it has).
-  // False when the CTA gives up.
+  // hand-over before has been merged (without `wait`: only if it has): a vote,
+  // since each lane loads the inserter's word for itself and full-mask
+  // operations follow.  False when the CTA gives up.
   __device__ __forceinline__ bool hand_over(bool wait) {
-    if (ld_shared_acquire(ho.done(w)) != given) {
+    if (!__all_sync(0xffffffffu, ld_shared_acquire(ho.done(w)) == given)) {
       if (!wait) return true;
       const uint64_t t0 = globaltimer_ns();
-      for (uint32_t it = 1; ld_shared_acquire(ho.done(w)) != given; ++it) {
+      for (uint32_t it = 1; !__all_sync(0xffffffffu, ld_shared_acquire(ho.done(w)) == given); ++it) {
         if ((it & 63u) == 0 && __any_sync(0xffffffffu, *abort_flag != 0u || globaltimer_ns() - t0 > kWaitLimitNs)) {
           flag_timeout(abort_flag, dev_err);
           n = 0;  // (the candidates are lost: the call reports the timeout)
@@ -440,7 +441,8 @@ struct Inserter {
     const uint32_t w = (uint32_t)h * 4 + quarter;
     const int q = QT == 2 ? h : 0;
     const uint32_t done = h == 0 ? done0 : done1;
-    if (ld_shared_acquire(ho.given(w)) == done) return false;
+    // one answer for the warp, whose lanes each load the word the epilogue changes
+    if (!__all_sync(0xffffffffu, ld_shared_acquire(ho.given(w)) != done)) return false;
     const int n = (int)ld_shared_u32(ho.count(w * 32 + lane));
     uint32_t* from =
         reinterpret_cast<uint32_t*>(cand) + ((int64_t)w * 64 + (done & 1u)) * cap * kEntryWords;
