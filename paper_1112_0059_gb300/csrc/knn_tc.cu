@@ -121,7 +121,7 @@ struct Layout {
   // drain; item full, item empty per item slot; lists written; warm-up done,
   // the rows' limits posted, the columns of an item all queued
   static constexpr int kNumBars = 2 * Stages + 2 + 3 + 2 + 2 + 1 + 3;
-  // TMEM address, abort flag, 2 item slots, 2 "an earlier split was not carried" words, work slot
+  // TMEM address, abort flag, "a timeout was reported before" flag, 2 item slots, 2 "an earlier split was not carried" words, work slot
   static constexpr uint32_t kOffMisc = kOffBar + 8 * kNumBars;
   static constexpr uint32_t kOffList = (kOffMisc + 48 + 1023) / 1024 * 1024;
   static constexpr uint32_t kSmemBytes = kOffList + ListBytes + 1024;  // + alignment slack
@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   const Bars<kStages> bars{sbase + L::kOffBar};
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kOffMisc);
   volatile uint32_t* abort_flag = tmem_slot + 1;
+  volatile uint32_t* stale_slot = tmem_slot + 2;
   volatile int64_t* item_slot = reinterpret_cast<volatile int64_t*>(smem + L::kOffMisc + 16);
   volatile uint32_t* chain_broken = reinterpret_cast<volatile uint32_t*>(smem + L::kOffMisc + 32);
   volatile int32_t* work_slot = reinterpret_cast<volatile int32_t*>(smem + L::kOffMisc + 40);
@@ -722,11 +723,10 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   constexpr int kIssuers = QT;
   constexpr int kSecondIssuerWarp = 2;
   const bool issuer = warp == 1 || (kIssuers == 2 && warp == kSecondIssuerWarp);
-  // A timeout reported earlier and not yet collected by lnbnn_sync: scan no
-  // tiles (every item's lists are still written, empty).
-  const bool stale_timeout = (*reinterpret_cast<volatile uint32_t*>(dev_err) & kDevErrTimeout) != 0;
-
   if (threadIdx.x == 0) {
+    // read by one thread: another CTA may report a timeout meanwhile, and the
+    // roles (and lanes) of this one have to agree on what they scan
+    const uint32_t reported = *reinterpret_cast<volatile uint32_t*>(dev_err);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(bars.full(s), 1);
       mbar_init(bars.empty(s), kIssuers);  // the MMA completions that free the stage
@@ -745,6 +745,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
     mbar_init(bars.limits(), kListWarps);
     mbar_init(bars.queued(), kEpiWarps);
     *abort_flag = 0u;
+    *stale_slot = reported & kDevErrTimeout;
     chain_broken[0] = chain_broken[1] = 0u;
     fence_barrier_init();
   }
@@ -781,7 +782,9 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
     *m0 = x * (int64_t)(kBM * QT);
     *j_begin = y * work.split_len;
     const int64_t j_end = min(*j_begin + work.split_len, n_ref);
-    return stale_timeout ? 0 : (int)((j_end - *j_begin + kTileN - 1) / kTileN);
+    // a timeout reported earlier and not yet collected by lnbnn_sync: scan no
+    // tiles (every item's lists are still written, empty)
+    return *stale_slot != 0u ? 0 : (int)((j_end - *j_begin + kTileN - 1) / kTileN);
   };
   // The tiles run twice at the start of this CTA's item i: none where the
   // lists go on from the previous chunk or split.
@@ -798,7 +801,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         // an optional start gate; with nothing loaded the other roles' waits
         // run out on the abort flag
         bool go = true;
-        if (out.gate != nullptr && !stale_timeout && !wait_gate(out.gate, kWaitLimitNs, abort_flag)) {
+        if (out.gate != nullptr && *stale_slot == 0u && !wait_gate(out.gate, kWaitLimitNs, abort_flag)) {
           flag_timeout(abort_flag, dev_err);
           go = false;
         }

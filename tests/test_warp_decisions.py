@@ -20,3 +20,11 @@ def test_hand_over_words_are_read_under_a_vote():
     for at in loads:
         before = re.split(r"[;{}]", text[:at])[-1]
         assert re.search(r"__(all|any)_sync\(0xffffffffu,\s*$", before), text[at - 80:at + 60]
+
+
+def test_error_word_is_read_by_one_thread():
+    text = _source("knn_tc.cu")
+    reads = [m.start() for m in re.finditer(r"volatile uint32_t\*>\(dev_err\)", text)]
+    assert len(reads) == 1
+    opened = text[:reads[0]].rindex("if (threadIdx.x == 0) {")
+    assert "}" not in text[opened:reads[0]]  # inside that branch; the CTA reads what it stored after the barrier
