@@ -174,12 +174,16 @@ LNBNN_API lnbnn_status nbnn_classify(lnbnn_index *index, const uint8_t *queries,
 
 /*
  * Workspaces: the device scratch of one call (query operand copies, the
- * per-row neighbour lists, the NBNN minima table), sized once for at most
+ * per-row neighbour lists, the NBNN minima table, the candidate buffers of a
+ * scan: 0.8 MB, or 1.8 MB for max_k above 63, for each CTA that runs at a time,
+ * up to 120 or 280 MB on 152 SMs), sized once for at most
  * max_queries query descriptors and neighbourhoods up to max_k.  A call given a
  * workspace allocates nothing, so it may be captured into a CUDA graph, and
  * calls with distinct workspaces may run concurrently on different streams
  * (the index itself is only read).  A workspace belongs to the index it was
- * created for.  A call larger than its workspace returns SCRATCH_LIMIT.
+ * created for.  It holds every call of that size, whatever the schedule was
+ * when it was made; a call larger than its workspace, whose lists and operand
+ * copies do not fit, returns SCRATCH_LIMIT.
  * The profile (lnbnn_profile_*) is not for captured calls.
  */
 typedef struct lnbnn_workspace lnbnn_workspace;

@@ -32,6 +32,20 @@ constexpr int kTcMinEntries = 10;
 __host__ __device__ constexpr int tc_entries(int K1) { return (K1 <= 64 ? 16 : 48) + 8; }
 __host__ __device__ constexpr int64_t tc_work_bytes(int entries) { return (int64_t)256 * 2 * entries * kTcEntryBytes; }
 
+// Candidate buffers for up to `ctas` CTAs at a time in `bytes` of scratch:
+// entries per epilogue thread, fewer where the buffers of all CTAs would not
+// fit, and for how many CTAs (0: not even one's).
+struct TcWork {
+  int entries;
+  int64_t slots;
+};
+inline TcWork tc_fit_work(int K1, int64_t ctas, int64_t bytes) {
+  TcWork f;
+  f.entries = (int)std::min<int64_t>(tc_entries(K1), std::max<int64_t>(kTcMinEntries, bytes / ctas / tc_work_bytes(1)));
+  f.slots = std::min<int64_t>(ctas, bytes / tc_work_bytes(f.entries));
+  return f;
+}
+
 // The kernel instantiation for lists of K1 keys: the longest list it takes, 0
 // for the longest.
 inline int tc_list_max(int K1) {

@@ -69,7 +69,8 @@ struct lnbnn_workspace {
   const lnbnn_index* index = nullptr;
   void* base = nullptr;
   size_t bytes = 0;
-  size_t sized = 0;  // KnnPlan::sized of its largest call
+  size_t room = 0;  // of it, what grows with queries and list length (not the candidate buffers)
+  int64_t keys = 0;  // list keys of its largest call: padded queries x list length
 };
 
 namespace {
@@ -294,19 +295,20 @@ struct KnnPlan {
   bool lists_kept;      // a kNN scan
   bool bounded;         // several splits of a row share its bound
   int64_t work_slots;   // candidate buffers of lists in progress (one set per CTA)
+  int entries;          // of each
   size_t off_qbf, off_qext, off_lists, off_merged, off_rowthr, off_queue, off_done, off_count, off_slots, off_work, bytes;
   size_t sized;  // bytes of what grows with queries and list length (all but the candidate buffers)
   TcSched sched(char* ws, int sm_count) const {
     TcSched t;
     t.qt = qt;
-    t.persistent_ctas = persistent ? sm_count : 0;
+    t.persistent_ctas = !persistent ? 0 : group > 0 ? sm_count : (int)std::min<int64_t>(sm_count, work_slots);
     t.queue = reinterpret_cast<uint32_t*>(ws + off_queue);
     t.bound_per_tile = bound_per_tile;
     t.done = seeded ? reinterpret_cast<uint32_t*>(ws + off_done) : nullptr;
     t.group = group;
     t.work = ws + off_work;
     t.work_slots = work_slots;
-    t.entries = tc_entries(K1);
+    t.entries = entries;
     t.slot_used = reinterpret_cast<uint32_t*>(ws + off_slots);
     return t;
   }
@@ -319,6 +321,20 @@ struct KnnPlan {
     if (items > work_slots && !persistent) b->fill(ws + off_slots, sizeof(uint32_t) * (size_t)work_slots, 0u);
     if (lists_kept) b->fill(ws + off_count, sizeof(uint32_t), 0u);
     if (bounded) b->fill(ws + off_rowthr, sizeof(int32_t) * (size_t)m_pad, 0x7F7F7F7Fu);
+  }
+  // Makes do with `have` bytes where the candidate buffers do not fit: fewer
+  // entries each, then fewer buffers, whose CTAs take the items from the
+  // queue (not in the claimed-chunk form).  False if that is not enough.
+  bool fit(size_t have) {
+    if (bytes <= have) return true;
+    if (!lists_kept || off_work >= have) return false;
+    const TcWork f = tc_fit_work(K1, work_slots, (int64_t)(have - off_work));
+    if (f.slots < 1 || (group > 0 && f.slots < work_slots)) return false;
+    if (f.slots < work_slots) persistent = true;
+    entries = f.entries;
+    work_slots = f.slots;
+    bytes = off_work + (size_t)(work_slots * tc_work_bytes(entries));
+    return true;
   }
   // The merge's view of a seeded launch: rows whose last split holds every
   // split's keys merge only that split's lists.
@@ -337,9 +353,9 @@ struct KnnPlan {
 // fixed choices (lnbnn_set_schedule) or else the rules and split model above.
 // splits > 0 fixes the split count (an upper bound after rounding the split
 // length to whole tiles).
-KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int splits = 0) {
+KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int splits, const lnbnn_schedule& o,
+                 bool may_claim = true) {
   KnnPlan p{};
-  const lnbnn_schedule& o = ix->sched;
   const int P = ix->sm_count;
   p.m_pad = round_up(m, kQueryPad);
   p.K1 = K1;
@@ -363,7 +379,7 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   const bool claim_kind = kind != ScanKind::Nbnn && (K1 <= kTcCoarseRegListMax || K1 > kTcWideRegListMax) &&
                           (kind == ScanKind::Coarse ? T * 8 <= P : T == 1);
   const int64_t ref_tiles = (ix->n_ref + kTcRefTile - 1) / kTcRefTile;
-  p.group = splits <= 0 && T < P && p.qt == 1 && claim_kind && o.persistent != 0 && o.bound_per_tile != 0
+  p.group = may_claim && splits <= 0 && T < P && p.qt == 1 && claim_kind && o.persistent != 0 && o.bound_per_tile != 0
                 // chunks of >= 4 tiles each, and no more lists than the split
                 // form may write (workspaces are sized for that)
                 ? (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(P / T, ref_tiles / 4),
@@ -406,9 +422,13 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.sized = c.off;
   p.work_slots = knn ? std::min<int64_t>(p.items, P) : p.items;  // (none for NBNN, which keeps no lists)
   p.off_slots = c.take<uint32_t>((size_t)P);
-  p.off_work = c.take<char>(knn ? (size_t)(p.work_slots * tc_work_bytes(tc_entries(K1))) : 0);
+  p.entries = tc_entries(K1);
+  p.off_work = c.take<char>(knn ? (size_t)(p.work_slots * tc_work_bytes(p.entries)) : 0);
   p.bytes = c.off;
   return p;
+}
+KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int splits = 0) {
+  return plan_knn(ix, m, K1, kind, splits, ix->sched);
 }
 
 // Device scratch of one call: the caller's workspace (fixed size, nothing is
@@ -416,7 +436,7 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
 struct Scratch {
   lnbnn_index* ix;
   lnbnn_workspace* w;
-  lnbnn_status admit(int64_t m, int K1) const;
+  lnbnn_status plan(int64_t m, int K1, ScanKind kind, int splits, KnnPlan* p) const;
   lnbnn_status get(size_t need, char** out) {
     if (w) {
       if (need > w->bytes) return LNBNN_ERR_SCRATCH_LIMIT;
@@ -448,40 +468,50 @@ NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
   return p;
 }
 
-// Largest scratch any call with at most max_q queries and lists of K1 needs,
-// and its KnnPlan::sized.  The lists grow with the split count, so the bound
-// takes the largest count the schedule may choose (for either tile shape),
-// whatever model lnbnn_autotune fits later.
+// The scratch of a workspace for at most max_q queries and lists of K1: the
+// largest any such call needs.  The lists grow with the split count and the
+// per-item words with the query tiles, so the bound takes the largest count
+// the schedule may choose (for either tile shape) over tiles of 128 queries,
+// whatever is fixed or fitted when the workspace is made or used.
 struct ScratchBound {
-  size_t bytes = 0, sized = 0;
+  size_t bytes = 0, room = 0;
 };
-void add_bound(const lnbnn_index* ix, int64_t m, int K1, ScratchBound* b) {
-  const int64_t T1 = round_up(m, kQueryPad) / kTcQueryTile;
-  for (ScanKind k : {ScanKind::Exact, ScanKind::Coarse, ScanKind::Nbnn}) {
-    const int64_t hi = std::max(splits_bound(ix, T1, k), splits_bound(ix, (T1 + 1) / 2, k));
-    if (k == ScanKind::Nbnn) {
-      b->bytes = std::max(b->bytes, plan_nbnn(ix, m, (int)hi).bytes);
-    } else {
-      const KnnPlan p = plan_knn(ix, m, K1, k, (int)hi);
-      b->bytes = std::max(b->bytes, p.bytes);
-      b->sized = std::max(b->sized, p.sized);
+ScratchBound scratch_bound(const lnbnn_index* ix, int64_t max_q, int K1) {
+  const lnbnn_schedule one{0, 1, 0, -1};
+  size_t room = 0, work = 0;
+  for (int64_t m = kQueryPad; m < max_q + kQueryPad; m += kQueryPad) {
+    const int64_t mm = std::min(m, max_q), T1 = round_up(mm, kQueryPad) / kTcQueryTile;
+    for (ScanKind k : {ScanKind::Exact, ScanKind::Coarse, ScanKind::Nbnn}) {
+      const int hi = (int)std::max(splits_bound(ix, T1, k), splits_bound(ix, (T1 + 1) / 2, k));
+      if (k == ScanKind::Nbnn) {
+        room = std::max(room, plan_nbnn(ix, mm, hi).bytes);
+      } else {
+        const KnnPlan p = plan_knn(ix, mm, K1, k, hi, one);
+        room = std::max(room, p.sized);
+        work = std::max(work, p.bytes - p.sized);
+      }
     }
   }
-}
-ScratchBound scratch_bound(const lnbnn_index* ix, int64_t max_q, int K1) {
-  ScratchBound b;
-  for (int64_t m = kQueryPad; m < max_q + kQueryPad; m += kQueryPad) add_bound(ix, std::min(m, max_q), K1, &b);
-  return b;
+  return {room + 256 + work, room};  // (+ the alignment of what follows)
 }
 
-// Whether a kNN call of m queries with lists of K1 is within the workspace it
-// was given.  (Its bytes alone would let longer lists in: the candidate
-// buffers outweigh the lists of a small call.)
-lnbnn_status Scratch::admit(int64_t m, int K1) const {
-  if (!w || w->sized == 0) return LNBNN_OK;
-  ScratchBound b;
-  add_bound(ix, m, K1, &b);
-  return b.sized > w->sized ? LNBNN_ERR_SCRATCH_LIMIT : LNBNN_OK;
+// The plan of a kNN call, within the workspace if there is one: what it needs
+// besides candidate buffers has to fit what the workspace was sized for, and
+// the buffers make do with the rest.  A call that asks for no more list keys
+// than the workspace was made for (longer lists of fewer queries, or shorter
+// ones of more) takes fewer splits if the automatic count does not fit.
+lnbnn_status Scratch::plan(int64_t m, int K1, ScanKind kind, int splits, KnnPlan* p) const {
+  *p = plan_knn(ix, m, K1, kind, splits);
+  if (!w) return LNBNN_OK;
+  auto fits = [&]() { return p->sized <= w->room && p->fit(w->bytes); };
+  if (fits()) return LNBNN_OK;
+  if (splits > 0 || ix->sched.splits > 0 || p->m_pad * K1 > w->keys) return LNBNN_ERR_SCRATCH_LIMIT;
+  *p = plan_knn(ix, m, K1, kind, 0, ix->sched, /*may_claim=*/false);
+  while (!fits()) {
+    if (p->splits == 1) return LNBNN_ERR_SCRATCH_LIMIT;
+    *p = plan_knn(ix, m, K1, kind, p->splits - 1);
+  }
+  return LNBNN_OK;
 }
 
 // What a scan leaves: its plan, the call's scratch and the lists it wrote.
@@ -496,9 +526,9 @@ struct Found {
 // Runs the exact scan.
 lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int K1, cudaStream_t s, Found* out,
                      CallProfile& prof, Begin begin = Begin{}, int force_splits = 0) {
-  KnnPlan p = plan_knn(ix, m, K1, ScanKind::Exact, force_splits);
+  KnnPlan p;
   char* ws = nullptr;
-  lnbnn_status st = scratch.admit(m, K1);
+  lnbnn_status st = scratch.plan(m, K1, ScanKind::Exact, force_splits, &p);
   if (st == LNBNN_OK) st = scratch.get(p.bytes, &ws);
   if (st != LNBNN_OK) return st;
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + p.off_qbf);
@@ -523,9 +553,9 @@ lnbnn_status run_knn(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_
 // The FP8 shortlist search's coarse pass, keeping the M1 smallest coarse keys.
 lnbnn_status run_knn_fp8(lnbnn_index* ix, Scratch& scratch, const uint8_t* q, int64_t m, int M1, cudaStream_t s,
                          Found* out, CallProfile& prof, Begin begin = Begin{}) {
-  KnnPlan p = plan_knn(ix, m, M1, ScanKind::Coarse);
+  KnnPlan p;
   char* ws = nullptr;
-  lnbnn_status st = scratch.admit(m, M1);
+  lnbnn_status st = scratch.plan(m, M1, ScanKind::Coarse, 0, &p);
   if (st == LNBNN_OK) st = scratch.get(p.bytes, &ws);
   if (st != LNBNN_OK) return st;
   // the BF16 query operand's space holds the E4M3 bytes (half its size)
@@ -981,7 +1011,7 @@ lnbnn_status lnbnn_autotune(lnbnn_index* index, void* stream, lnbnn_tuning* out)
   index->sched = saved;
   lnbnn_workspace w;
   w.index = index;
-  w.bytes = need;
+  w.bytes = w.room = need;
   uint8_t* q = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   lnbnn_status st = LNBNN_OK;
@@ -1415,7 +1445,8 @@ lnbnn_status lnbnn_workspace_create(lnbnn_index* index, int64_t max_queries, int
   w->index = index;
   const ScratchBound bound = scratch_bound(index, max_queries, std::min<int>(max_k + 1, LNBNN_MAX_K + 1));
   w->bytes = bound.bytes;
-  w->sized = bound.sized;
+  w->room = bound.room;
+  w->keys = round_up(max_queries, kQueryPad) * std::min<int>(max_k + 1, LNBNN_MAX_K + 1);
   cudaError_t e = lib_malloc(&w->base, w->bytes);
   if (e != cudaSuccess) {
     delete w;
