@@ -476,7 +476,8 @@ LNBNN_API lnbnn_status lnbnn_profile_read(lnbnn_index *index, lnbnn_profile *out
  * device (INVALID_ARG otherwise).  Every intermediate (BF16 operand copies,
  * squared norms, per-row neighbour lists and their shared bounds, the error
  * word) lives in one fixed-size array in device global memory that the
- * library defines at file scope: LNBNN_NOALLOC_SCRATCH_BYTES (64 MiB),
+ * library defines at file scope: LNBNN_NOALLOC_SCRATCH_BYTES (64 MiB) for a
+ * problem, and 64 MiB more for the scan's candidate buffers,
  * reserved on a device once the library's device code is loaded there (at
  * the latest by the first call there) and held until the process exits.  The
  * call makes no cudaMalloc, cudaFree or other allocating call.  n_ref or

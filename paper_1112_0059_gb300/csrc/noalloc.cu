@@ -18,9 +18,16 @@ namespace {
 
 using namespace lnbnn;
 
-// The fixed scratch: LNBNN_NOALLOC_SCRATCH_BYTES, reserved on a device once
-// the library's device code is loaded there, until the process exits.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[LNBNN_NOALLOC_SCRATCH_BYTES];
+// The fixed scratch, reserved on a device once the library's device code is
+// loaded there, until the process exits: LNBNN_NOALLOC_SCRATCH_BYTES for a
+// problem's operands and lists, and behind them room for the candidate buffers
+// of the CTAs that run at a time.  With the buffers in the rest of the 64 MiB a
+// large problem had few CTAs (200,000 references, 1,000 queries, k = 10: 22 for
+// 152 work items, 421 us against 199 before there were such buffers).  64 MiB
+// holds 13 entries a thread for 152 CTAs; a small problem leaves room for all 24.
+constexpr size_t kWorkBytes = size_t(64) << 20;
+constexpr size_t kScratchBytes = (size_t)LNBNN_NOALLOC_SCRATCH_BYTES + kWorkBytes;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -135,19 +142,16 @@ extern "C" LNBNN_API lnbnn_status knn_search_noalloc(const uint8_t* ref, int64_t
   const size_t o_merged = splits > 1 ? L.take<uint64_t>((size_t)m_pad * k) : o_lists;
   const size_t o_rowthr = L.take<int32_t>((size_t)m_pad);  // the bound the lists of a row share
   const size_t o_queue = L.take<uint32_t>(1);
-  // candidate buffers of the lists in progress: one set per CTA, as many CTAs as the rest
-  // of the scratch has room for (those take the work items from a queue)
-  const size_t o_work = L.take<char>((size_t)tc_work_bytes(kTcMinEntries));
   if (L.off > (size_t)LNBNN_NOALLOC_SCRATCH_BYTES) return LNBNN_ERR_SCRATCH_LIMIT;
+  // the candidate buffers take what is left: of fewer entries, and on a chip of
+  // more SMs than these make do for, of fewer CTAs (which take the work items
+  // from a queue)
+  const size_t o_work = L.take<char>(0);
   const int64_t items = (m_pad / kTcQueryTile) * splits;
+  const TcWork fit = tc_fit_work(k, std::min<int64_t>(items, sm_count), (int64_t)(kScratchBytes - o_work));
   TcSched sched;
-  auto areas = [&](int entries) {
-    const int64_t room = (int64_t)((size_t)LNBNN_NOALLOC_SCRATCH_BYTES - o_work) / tc_work_bytes(entries);
-    return std::min<int64_t>(std::min<int64_t>(items, sm_count), room);
-  };
-  sched.entries = tc_entries(k);
-  while (sched.entries > kTcMinEntries && areas(sched.entries) < areas(kTcMinEntries)) sched.entries -= 2;
-  sched.work_slots = areas(sched.entries);
+  sched.entries = fit.entries;
+  sched.work_slots = fit.slots;
 
   char* b = static_cast<char*>(base);
   uint32_t* err = reinterpret_cast<uint32_t*>(b + o_err);
