@@ -45,7 +45,7 @@ def test_made_and_used_under_different_schedules(lnbnn, made, used):
         ix.set_schedule(**made)
         with ix.workspace(M, k) as ws:
             ix.set_schedule(**used)
-            _check(ix, ws, ref, q, qd, k, rows)
+            _check(ix, ws, ref, q, qd, k + 1, rows)  # lists of max_k + 1, as a classify call keeps
             _check(ix, ws, ref, q[:999], qd[:999].contiguous(), k, np.arange(0, 999, 3))
 
 
