@@ -169,11 +169,16 @@ cudaError_t launch_rerank(const uint64_t* shortlist, int64_t m, int M1, const ui
 // class minima (which it overwrites), per image and class the sum of the
 // increments (all, or only those > 0), per image the number of increments
 // added (counts may be null) and the class of the largest sum, the lowest on
-// ties.  totals and counts are zeroed by the caller.  prepare_logodds sets the
-// kernel's shared-memory size on the current device (once, as prepare_tc_kernels).
+// ties.  totals and counts are zeroed by the caller; rowstat is scratch of
+// logodds_rowstat_bytes(m, C).  *launches: how many kernels it launched.
+// prepare_logodds sets the kernel's shared-memory size on the current device
+// (once, as prepare_tc_kernels).
+constexpr int64_t kLogoddsRowStatBytes = 24;
+int64_t logodds_rowstat_bytes(int64_t m, int32_t C);
 cudaError_t prepare_logodds();
-cudaError_t launch_logodds(int32_t* mins, int64_t m, int32_t C, double beta, bool positive_only, const int64_t* offsets,
-                           int64_t n_img, double* totals, int64_t* counts, int32_t* classes, cudaStream_t s);
+cudaError_t launch_logodds(int32_t* mins, void* rowstat, int64_t m, int32_t C, double beta, bool positive_only,
+                           const int64_t* offsets, int64_t n_img, double* totals, int64_t* counts, int32_t* classes,
+                           cudaStream_t s, int* launches);
 // argmin over classes per image, lowest class on ties.
 cudaError_t launch_argmin(const int64_t* totals, int64_t n_img, int32_t C, int32_t* classes, cudaStream_t s);
 

@@ -451,7 +451,7 @@ struct Scratch {
 
 struct NbnnPlan {
   KnnPlan k;
-  size_t off_qbf, off_qext, off_mins, off_queue, bytes;
+  size_t off_qbf, off_qext, off_mins, off_rowstat, off_queue, bytes;
 };
 
 NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
@@ -461,6 +461,7 @@ NbnnPlan plan_nbnn(const lnbnn_index* ix, int64_t m, int splits = 0) {
   p.off_qbf = c.take<__nv_bfloat16>(p.k.m_pad * kDim);
   p.off_qext = c.take<__nv_bfloat16>(p.k.m_pad * kExt);
   p.off_mins = c.take<int32_t>((size_t)p.k.m_pad * ix->n_classes);
+  p.off_rowstat = c.take<char>((size_t)logodds_rowstat_bytes(p.k.m_pad, ix->n_classes));  // log-odds rule only
   p.off_queue = c.take<uint32_t>(1);
   p.k.off_queue = p.off_queue;
   p.k.seeded = false;
@@ -1303,10 +1304,10 @@ static lnbnn_status do_lnbnn_classify(lnbnn_index* index, lnbnn_workspace* w, co
 
 // The [m_pad, C] table of class minima NN_C(d), one row per query row, filled
 // by the tensor-core scan of the class-sorted references (Alg. 1's inner
-// loop).
+// loop), and the scratch for its rows' log-odds statistics.
 static lnbnn_status scan_class_minima(lnbnn_index* index, lnbnn_workspace* w, const uint8_t* queries,
                                       int64_t n_queries, Begin begin, cudaStream_t s, CallProfile& prof,
-                                      int32_t** mins) {
+                                      int32_t** mins, void** rowstat) {
   const NbnnPlan np = plan_nbnn(index, n_queries);
   const KnnPlan& p = np.k;
   Scratch scratch{index, w};
@@ -1316,6 +1317,7 @@ static lnbnn_status scan_class_minima(lnbnn_index* index, lnbnn_workspace* w, co
   __nv_bfloat16* qbf = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qbf);
   __nv_bfloat16* qext = reinterpret_cast<__nv_bfloat16*>(ws + np.off_qext);
   *mins = reinterpret_cast<int32_t*>(ws + np.off_mins);
+  if (rowstat) *rowstat = ws + np.off_rowstat;
   begin.fill(*mins, sizeof(int32_t) * (size_t)p.m_pad * index->n_classes, 0x7F7F7F7Fu);  // > any distance
   p.begin(ws, &begin);
   CK(launch_prep_query(queries, n_queries, p.m_pad, index->row_bytes, index->loc_w, qbf, qext, begin, s));
@@ -1354,7 +1356,7 @@ static lnbnn_status do_nbnn_classify(lnbnn_index* index, lnbnn_workspace* w, con
     prof.mark(2);
   } else {
     int32_t* mins = nullptr;
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins, nullptr);
     if (st != LNBNN_OK) return st;
     CK(launch_nbnn_sum(mins, n_queries, C, offsets, n_images, totals, s));
     prof.launched(1);
@@ -1385,18 +1387,20 @@ static lnbnn_status do_nbnn_logodds_classify(lnbnn_index* index, lnbnn_workspace
   begin.m = n_queries;
   begin.dev_err = index->dev_err;
   int32_t* mins = nullptr;
+  void* rowstat = nullptr;
   if (n_queries == 0) {
     CK(launch_begin(begin, s));
     prof.launched(1);
     prof.mark(1);
     prof.mark(2);
   } else {
-    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins);
+    lnbnn_status st = scan_class_minima(index, w, queries, n_queries, begin, s, prof, &mins, &rowstat);
     if (st != LNBNN_OK) return st;
-    prof.launched(1);
   }
-  CK(launch_logodds(mins, n_queries, C, beta, positive_only, offsets, n_images, totals, n_increments, classes, s));
-  prof.launched(1);
+  int launches = 0;
+  CK(launch_logodds(mins, rowstat, n_queries, C, beta, positive_only, offsets, n_images, totals, n_increments, classes,
+                    s, &launches));
+  prof.launched(launches);
   return LNBNN_OK;
 }
 
