@@ -130,9 +130,8 @@ __global__ void extract_knn_kernel(const uint64_t* __restrict__ lists, int64_t m
   dist[e] = (int32_t)key_dist(key);
 }
 
-// Image owning descriptor row i: the last image whose first row is <= i.
-__device__ __forceinline__ int64_t image_of(const int64_t* __restrict__ offsets, int64_t n_img, int64_t i) {
-  int64_t lo = 0, hi = n_img;  // answer in [0, n_img)
+// Image owning descriptor row i, one of [lo, hi): the last whose first row is <= i.
+__device__ __forceinline__ int64_t image_of(const int64_t* __restrict__ offsets, int64_t lo, int64_t hi, int64_t i) {
   while (lo + 1 < hi) {
     const int64_t mid = (lo + hi) >> 1;
     if (offsets[mid] <= i) lo = mid; else hi = mid;
@@ -176,11 +175,17 @@ __device__ __forceinline__ void argmin_of(const int64_t* t, int32_t C, int32_t* 
 // k = 100, 15k rows 1.78 ms).  A block takes consecutive rows; a stretch of at
 // least kTableRows of one image is summed in shared memory first (int32: the
 // block's rows times the largest distance stay below 2^31), the rest goes
-// straight to the totals.
+// straight to the totals, with a row per warp whatever its image (the rows of
+// one small image at a time left most warps idle: 20,000 images of one row
+// against 5,000 references, k = 10, 100 us of a call against 26 for 200 images).
 constexpr int kScoreWarps = 8;
 constexpr int kScoreMaxRows = 128;    // rows of a block: 128 x 14,565,600 < 2^31
 constexpr int kTableRows = 8;
 constexpr int kTableClasses = 8192;   // classes up to which the sums fit (32 KB)
+constexpr int64_t kMaxDistance = 14565600;
+static_assert(kMaxDistance == (int64_t)kDim * 255 * 255 + 2ll * LNBNN_MAX_LOCATION_WEIGHT * 255 * 255 &&
+                  kScoreMaxRows * kMaxDistance <= INT32_MAX,
+              "a block's sums stay within 32 bits");
 
 // The update of rows [row0, row1) by a block: update(i, add) is called by a warp
 // for row i and calls add(class, delta) from any of its lanes.
@@ -189,33 +194,39 @@ __device__ __forceinline__ void sum_rows(const int64_t* offsets, int64_t n_img, 
                                          bool table, int64_t* totals, uint32_t* dev_err, int32_t* sums, Update update) {
   const int warp = threadIdx.x >> 5;
   unsigned long long* t = reinterpret_cast<unsigned long long*>(totals);
-  for (int64_t r = row0; r < row1;) {  // stretches of one image (the same for the block)
-    const int64_t img = image_of(offsets, n_img, r);
+  const int64_t first = image_of(offsets, 0, n_img, row0), last = image_of(offsets, first, n_img, row1 - 1);
+  for (int64_t r = row0; r < row1;) {  // stretches of one image (the same for the block), or of small images
+    const int64_t img = image_of(offsets, first, last + 1, r);
     const int64_t end = min(offsets[img + 1], row1);
-    if (r < offsets[img] || r >= end) {  // only with invalid offsets
-      if (threadIdx.x == 0) atomicOr(dev_err, kDevErrOffsets);
-      ++r;
-      continue;
-    }
-    const bool summed = table && end - r >= kTableRows;
+    const bool summed = table && r >= offsets[img] && end - r >= kTableRows;
+    const int64_t stop = summed ? end : min(row1, table ? r + 4 * kScoreWarps : row1);
     if (summed) {
       for (int32_t c = threadIdx.x; c < C; c += 32 * kScoreWarps) sums[c] = 0;
       __syncthreads();
     }
-    auto add = [&](int32_t c, int32_t delta) {
-      if (summed)
-        atomicAdd(sums + c, delta);
-      else
-        atomicAdd(t + img * C + c, (unsigned long long)(int64_t)delta);
-    };
-    for (int64_t i = r + warp; i < end; i += kScoreWarps) update(i, add);
+    for (int64_t i = r + warp; i < stop; i += kScoreWarps) {
+      int64_t own = img;
+      if (!summed) {
+        own = image_of(offsets, first, last + 1, i);
+        if (i < offsets[own] || i >= offsets[own + 1]) {  // only with invalid offsets
+          if ((threadIdx.x & 31) == 0) atomicOr(dev_err, kDevErrOffsets);
+          continue;
+        }
+      }
+      update(i, [&](int32_t c, int32_t delta) {
+        if (summed)
+          atomicAdd(sums + c, delta);
+        else
+          atomicAdd(t + own * C + c, (unsigned long long)(int64_t)delta);
+      });
+    }
     if (summed) {
       __syncthreads();
       for (int32_t c = threadIdx.x; c < C; c += 32 * kScoreWarps)
         if (sums[c] != 0) atomicAdd(t + img * C + c, (unsigned long long)(int64_t)sums[c]);
       __syncthreads();
     }
-    r = end;
+    r = stop;
   }
 }
 
@@ -410,17 +421,23 @@ __global__ void __launch_bounds__(32 * kScoreWarps) row_end_kernel(const __grid_
 }
 
 // Alg. 1's sums: totals[img][c] += the sum over the image's descriptor rows of
-// mins[row][c] (= NN_c of that descriptor).  A block takes 32 rows and 128
-// classes, whatever the images (a block per image left most SMs idle: 20
-// images, 162 us); integer addition is exact in any order.
+// mins[row][c] (= NN_c of that descriptor).  A block takes up to 32 rows and
+// 128 classes, whatever the images (a block per image left most SMs idle: 20
+// images, 162 us).  Rows of several images are added one after another, so it
+// takes no more rows than an image has on average unless there are many blocks
+// anyway (20,000 images of one row: 10 classes, 32 rows 45 us, one row 13;
+// 4,000 classes, images of 3 rows, whole calls of 6.72 and 6.99 ms); integer
+// addition is exact in any order.
 constexpr int kSumRows = 32;
+constexpr int64_t kSumBlocks = 16 * 152;
 __global__ void nbnn_sum_kernel(const int32_t* __restrict__ mins, int64_t m, int32_t C,
-                                const int64_t* __restrict__ offsets, int64_t n_img, int64_t* __restrict__ totals) {
+                                const int64_t* __restrict__ offsets, int64_t n_img, int rows,
+                                int64_t* __restrict__ totals) {
   const int32_t c = blockIdx.y * blockDim.x + threadIdx.x;
   if (c >= C) return;
-  const int64_t row1 = min(m, ((int64_t)blockIdx.x + 1) * kSumRows);
-  for (int64_t r = (int64_t)blockIdx.x * kSumRows; r < row1;) {
-    const int64_t img = image_of(offsets, n_img, r);
+  const int64_t row0 = (int64_t)blockIdx.x * rows, row1 = min(m, row0 + rows);
+  for (int64_t r = row0; r < row1;) {
+    const int64_t img = image_of(offsets, 0, n_img, r);
     const int64_t end = min(offsets[img + 1], row1);
     if (r < offsets[img] || r >= end) {  // only with invalid offsets, flagged elsewhere
       ++r;
@@ -500,7 +517,9 @@ cudaError_t launch_row_end(const RowLists& in, const RowRerank* rerank, const Ro
     p.dev_err = score->dev_err;
     p.classes = score->classes;
     // one block takes the argmin of up to 64 images x 256 classes in a few us
-    p.counter = score->n_img * score->C <= 16384 ? score->counter : nullptr;
+    // (an image's is one round trip to memory for a warp, whatever its classes:
+    // 400 images x 10 classes took 20 us that way, 3 as a launch of their own)
+    p.counter = score->n_img <= 64 && score->n_img * score->C <= 16384 ? score->counter : nullptr;
     if (argmin_done) *argmin_done = p.counter != nullptr;
     smem = p.table ? sizeof(int32_t) * (size_t)score->C : 0;
   } else {
@@ -552,8 +571,11 @@ cudaError_t launch_lnbnn_score(const uint64_t* lists, int64_t m, int K1, int k, 
 cudaError_t launch_nbnn_sum(const int32_t* mins, int64_t m, int32_t C, const int64_t* offsets, int64_t n_img,
                             int64_t* totals, cudaStream_t s) {
   if (n_img == 0 || m == 0) return cudaSuccess;
-  dim3 grid((unsigned)((m + kSumRows - 1) / kSumRows), (unsigned)((C + 127) / 128));
-  nbnn_sum_kernel<<<grid, 128, 0, s>>>(mins, m, C, offsets, n_img, totals);
+  const int64_t ranges = (C + 127) / 128;
+  const int rows =
+      (int)std::min<int64_t>(kSumRows, std::max<int64_t>(1, std::max<int64_t>(m / n_img, m * ranges / kSumBlocks)));
+  dim3 grid((unsigned)((m + rows - 1) / rows), (unsigned)ranges);
+  nbnn_sum_kernel<<<grid, 128, 0, s>>>(mins, m, C, offsets, n_img, rows, totals);
   return cudaGetLastError();
 }
 
