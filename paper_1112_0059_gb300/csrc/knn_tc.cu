@@ -94,10 +94,12 @@ template <class Epilogue>
 constexpr int kMaxRegsOf = 65536 / kThreadsOf<Epilogue> / 8 * 8;
 // Lists of more than 64 registers a thread: the inserter warps take registers
 // that the first warpgroup, whose roles need few, gives up (the epilogue's two
-// warpgroups keep theirs).
+// warpgroups keep theirs).  What counts is that an insertion has no spilled
+// operand: k = 50, 20,000 rows x 1.5 million, 184 registers and the spills that
+// went with them 7.4 and 9.3 ms, 192 6.4, 200 6.4.
 template <class Epilogue, int QT>
 constexpr bool kWideLists = Epilogue::KMAX * QT > 32;
-constexpr int kRegsFirst = 72, kRegsLaunch = 128, kRegsInserter = 184;
+constexpr int kRegsFirst = 64, kRegsLaunch = 128, kRegsInserter = 192;
 static_assert(kRegsFirst + 2 * kRegsLaunch + kRegsInserter <= 4 * kRegsLaunch, "what is taken has been given up");
 constexpr uint32_t kAccCols = kTcRefTile;  // FP32 columns per accumulator (one step)
 constexpr uint32_t kTmemCols = 2 * kAccCols;
@@ -776,15 +778,17 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   };
   static_assert(!Claim || (QT == 1 && Epilogue::kClaimsChunks), "the claimed-chunk form: one query tile per CTA, kNN lists");
   constexpr bool chunked = Claim;
+  // (after a timeout reported earlier and not yet collected by lnbnn_sync, no
+  // tiles are scanned: every item's lists are still written, empty; the
+  // inserters, whose registers are short, need not know)
+  auto scanned_tiles = [&](int ntiles) -> int { return *stale_slot != 0u ? 0 : ntiles; };
   auto item_tiles = [&](int64_t w, int64_t* m0, int64_t* j_begin) -> int {
     const int64_t x = chunked ? (int64_t)blockIdx.x / work.group : w % work.T;
     const int64_t y = chunked ? w : w / work.T;
     *m0 = x * (int64_t)(kBM * QT);
     *j_begin = y * work.split_len;
     const int64_t j_end = min(*j_begin + work.split_len, n_ref);
-    // a timeout reported earlier and not yet collected by lnbnn_sync: scan no
-    // tiles (every item's lists are still written, empty)
-    return *stale_slot != 0u ? 0 : (int)((j_end - *j_begin + kTileN - 1) / kTileN);
+    return (int)((j_end - *j_begin + kTileN - 1) / kTileN);
   };
   // The tiles run twice at the start of this CTA's item i: none where the
   // lists go on from the previous chunk or split.
@@ -829,7 +833,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           }
           if (w >= work.n_items) break;
           int64_t m0, j_begin;
-          const int ntiles = item_tiles(w, &m0, &j_begin);
+          const int ntiles = scanned_tiles(item_tiles(w, &m0, &j_begin));
           // the query tiles: once the previous item's MMAs have read theirs (in
           // the claimed-chunk form, once for the whole launch)
           if (!chunked || a_loads == 0) {
@@ -894,7 +898,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           }
           if (w >= work.n_items) break;
           int64_t m0, j_begin;
-          int ntiles = item_tiles(w, &m0, &j_begin);
+          int ntiles = scanned_tiles(item_tiles(w, &m0, &j_begin));
           ntiles += warm_tiles(i, w, ntiles).tiles;
           if ((!chunked || i == 0) && !mbar_wait(bars.afull(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
             flag_timeout(abort_flag, dev_err);
@@ -1043,7 +1047,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
       }
       if (w >= work.n_items) break;
       int64_t m0, j_begin;
-      const int ntiles = item_tiles(w, &m0, &j_begin);
+      const int ntiles = scanned_tiles(item_tiles(w, &m0, &j_begin));
       if constexpr (kAsync) {
         if (!Claim || i == 0) {
           const WarmUp wu = warm_tiles(i, w, ntiles);
@@ -1135,7 +1139,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           if (w >= work.n_items) break;
         }
         int64_t m0, j_begin;
-        const int ntiles = item_tiles(w, &m0, &j_begin);
+        item_tiles(w, &m0, &j_begin);
         const int64_t y = Claim ? (int64_t)(blockIdx.x % (unsigned)work.group) : w / work.T;
         // the previous split of these rows, if it has finished: start from its
         // list.  Its flag says 2 when every earlier split of the rows was
@@ -1143,7 +1147,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         // the item's slot (cleared by the thread that publishes the slot's
         // previous item before that item's slot is released)
         const bool chain = !Claim && out.done != nullptr;
-        const uint32_t prev = chain && y > 0 && ntiles > 0 ? ld_acquire_gpu(out.done + (w - out.T)) : 0u;
+        const uint32_t prev = chain && y > 0 ? ld_acquire_gpu(out.done + (w - out.T)) : 0u;
         const bool carried = __all_sync(0xffffffffu, prev != 0u);
         if (chain && y > 0 && !__all_sync(0xffffffffu, prev == 2u) && lane == 0) chain_broken[i & 1] = 1u;
         bool ok = __all_sync(0xffffffffu, mbar_wait(bars.warmed(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag));
