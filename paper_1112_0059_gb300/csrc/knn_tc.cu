@@ -283,48 +283,87 @@ __device__ __forceinline__ void release_slot(const ScanOut& out, int32_t s) {
 //
 // Warm-up: a list that starts empty would copy every column until its first
 // merge.  So the first tiles of an item are run twice, first for a limit alone:
-// the columns fall into groups of 32, each group's least value is the distance
-// of another column, and so the K1-th smallest of these minima bounds the K1-th
-// smallest distance.  A thread keeps the least ceil(K1 / 2) minima of its column
-// half sorted (QT = 2: K1), and the larger of the two halves' last ones is the
-// limit ("ranked").  Lists too long for that take the largest minimum of
-// exactly as many groups, of a tile's column half where the item is long
-// enough.
-constexpr int32_t kNoBound = 0x7F7F7F7F;  // row_thr's initial value: above every distance
+// the columns fall into groups, each group's least value is the distance of
+// another column, and so the K1-th smallest of these minima bounds the K1-th
+// smallest distance.  A thread keeps the least minima of its column half sorted,
+// half of K1 (QT = 2: K1), and the larger of the two halves' last ones is the
+// limit.  With 32 columns a group the minimum comes with the load; where that is
+// too few groups for a useful limit, eight.  Where a thread cannot keep as many
+// minima (lists of more than 128 keys), a group's second-least value stands for
+// two columns.  (QT = 2 with the longest lists has no registers for any: the
+// largest minimum of exactly as many groups.)
+// (row_thr starts at 0x7F7F7F7F, above everything.)  A list's own bound starts
+// between the distances (and coarse values) and those of padding rows, so that
+// these are never collected: a last split of one tile, mostly padding, held up
+// calls of short items by 20 of 45 us.
+constexpr int32_t kRealBound = 0x4B7FFFFF;  // bits of 2^24 - 1
 
 struct WarmUp {
-  int tiles;     // tiles run twice
-  bool fine;     // groups of 32 columns
-  bool ranked;   // the limit is the K1-th (per column half) smallest of the minima
+  int tiles;    // tiles run twice
+  bool octets;  // groups of 8 columns, not 32 (unranked: of 32, not the thread's part of a tile)
+  bool pairs;   // a group's second-least value, for two columns
 };
-// How many minima a thread can keep sorted, for the ranked limit.
+// How many minima a thread can keep sorted (0: the limit is the largest).
 template <int KMAX, int QT>
 constexpr int kRankedMax = KMAX > 0 ? KMAX * QT / 2 : QT == 1 ? 64 : 0;
+// rows: of the item's query tile; share: other lists of the rows run meanwhile
+// and share their bound.
+//
+// A tile run twice costs a step; W of an item's n tiles leave about
+// K1 (1 + ln(n / W)) columns a row to insert.  The least sum is at W ~ K1 for
+// lists in registers (8 K1 for the 64-key ones, whose insertions are dear), a
+// few K1 where a merge is paid by the row, whatever n: so a short item runs all
+// of its tiles twice.  Whole calls, one GB300, with the tiles limited to a
+// quarter or a sixteenth of the item (and none where they had fewer than K1
+// groups of 32) against now: 20,000 queries, 2,000 references, k = 10, 24, 100
+// and 200 171, 298, 3,351 and 5,552 us / 102, 161, 1,104 and 2,582 us; 20,000
+// references, k = 50 and 100 1.88 and 3.76 / 0.57 and 1.45 ms; 500,000, k = 50
+// 5.1 / 3.2 ms.  Lists that share a bound get most of it from one another, so
+// their items keep that limit, but for a few tiles: 128 queries, 5,000
+// references, k = 10 and 100 74 and 1,484 / 56 and 668 us, 11.5 million, k = 40
+// all tiles 975, a sixteenth 650 us.
 template <int KMAX, int QT, bool Claim>
-__device__ __forceinline__ WarmUp warm_up(int ntiles, int K1) {
-  constexpr int kHalves = QT == 2 ? 1 : 2;  // column halves of a row per tile
-  const int wide = (K1 + kHalves - 1) / kHalves, fine = (K1 + 4 * kHalves - 1) / (4 * kHalves);
-  if (ntiles < fine) return {0, false, false};
-  if (wide <= kRankedMax<KMAX, QT>) {
-    // A tile more costs a step; twice as many save K1 ln 2 candidates a row,
-    // which cost more the longer the list.  Whole calls (one GB300), against
-    // the largest minimum of ceil(K1 / 2) tiles: 2,000 queries x 5,000 rows
-    // 81 / 68 us; FP8 shortlist 24, one image of 632 rows, K1 / 4, K1 / 2, K1
-    // and 2 K1 tiles 802, 780, 777 and 786 us (before: 802); 20-NN of 3,001 rows
-    // with locations 855 / 830 us; k = 50, 200k rows x 1.5 million, K1 / 4, K1, 4 K1
-    // and 8 K1 tiles of 5,918 63.4, 61.7, 61.7 and 56.3 ms (63.8), one image
-    // against 11.5 million (items of 1,500 tiles) 102, 204 and 375 tiles 1.38,
-    // 1.48 and 1.59 ms (1.50); k = 100, 15k rows, items of 9,000 tiles, 2 K1,
-    // 4 K1 and 8 K1 tiles 32.3, 31.8 and 32.5 ms (32.9), FP8 shortlist 128
-    // 26.5, 26.8 and 27.7 ms (27.2).  At least 16 tiles, and hand-overs from two
-    // entries on for lists of less than 8 keys: 37,271 queries x 27,412 rows
-    // (items of 107 tiles), k = 1, 2, 5 and 10 476, 503, 546 and 598 us with K1
-    // tiles, 451, 488, 542 and 584 us with at least 8, 397, 449, 499 and 573 us
-    // with at least 16.
-    const int want = K1 <= 32 ? max(K1, 16) : (K1 <= 64 ? 8 : 3) * K1;
-    return {max(fine, min(want, ntiles / (Claim || K1 <= 32 ? 4 : 16))), true, true};
+__device__ __forceinline__ WarmUp warm_up(int ntiles, int K1, int64_t rows, bool share) {
+  constexpr int kRanked = kRankedMax<KMAX, QT>;
+  if constexpr (kRanked == 0) {
+    const int fine = (K1 + 3) / 4;
+    return ntiles >= 2 * K1 ? WarmUp{K1, false, false} : WarmUp{ntiles < fine ? 0 : fine, true, false};
   }
-  return ntiles >= 2 * wide ? WarmUp{wide, false, false} : WarmUp{fine, true, false};
+  const int need = (K1 * QT + 1) / 2;
+  const bool wide = K1 > 32, pairs = need > kRanked;
+  const int want = !wide      ? max(K1, 16)
+                   : pairs    ? K1 / 2
+                   : KMAX > 0 ? 8 * K1
+                              : max(16, 3 * K1 * (int)min(rows, int64_t(32)) / 32);
+  const int tiles =
+      min(want, share ? max(ntiles / (Claim || !wide || pairs ? 4 : 16), min(ntiles, wide ? 16 : 8)) : ntiles);
+  const int ranks = pairs ? (need + 1) / 2 : need;
+  const bool octets = 4 * tiles < 2 * ranks;
+  return {(octets ? 16 : 4) * tiles < ranks ? 0 : tiles, octets, pairs};
+}
+
+// The four octets' least (pairs: second-least) values, or the one of all 32.
+__device__ __forceinline__ void group_values(const uint32_t (&v)[32], bool octets, bool pairs, int32_t (&y)[4]) {
+  int32_t a[4], b[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    a[o] = (int32_t)v[8 * o];
+    b[o] = INT32_MAX;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+      const int32_t x = (int32_t)v[8 * o + i];
+      b[o] = min(b[o], max(a[o], x));
+      a[o] = min(a[o], x);
+    }
+    y[o] = pairs ? b[o] : a[o];
+  }
+  if (octets) return;
+#pragma unroll
+  for (int o = 1; o < 4; ++o) {
+    b[0] = min(min(b[0], b[o]), max(a[0], a[o]));
+    a[0] = min(a[0], a[o]);
+  }
+  y[0] = pairs ? b[0] : a[0];
 }
 
 // Shared memory of the hand-over between epilogue and inserter warps.
@@ -792,9 +831,9 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   };
   // The tiles run twice at the start of this CTA's item i: none where the
   // lists go on from the previous chunk or split.
-  auto warm_tiles = [&](int i, int64_t w, int ntiles) -> WarmUp {
+  auto warm_tiles = [&](int i, int64_t w, int64_t m0, int ntiles) -> WarmUp {
     if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false, false};
-    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1);
+    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1, m - m0, out.bound_per_tile && out.row_thr != nullptr);
   };
 
   if (warp < kEpiWarp0) {
@@ -851,7 +890,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
             ++a_loads;
           }
           bool ok = true;
-          const int warm = warm_tiles(i, w, ntiles).tiles;
+          const int warm = warm_tiles(i, w, m0, ntiles).tiles;
           for (int t = -warm; ok && t < ntiles && !*abort_flag; ++t) {
             const int32_t row = (int32_t)(j_begin + (int64_t)(t < 0 ? t + warm : t) * kTileN);
             for (int kc = 0; kc < KC; ++kc, ++it) {
@@ -899,7 +938,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           if (w >= work.n_items) break;
           int64_t m0, j_begin;
           int ntiles = scanned_tiles(item_tiles(w, &m0, &j_begin));
-          ntiles += warm_tiles(i, w, ntiles).tiles;
+          ntiles += warm_tiles(i, w, m0, ntiles).tiles;
           if ((!chunked || i == 0) && !mbar_wait(bars.afull(), (uint32_t)(i & 1), kWaitLimitNs, abort_flag)) {
             flag_timeout(abort_flag, dev_err);
             break;
@@ -1050,12 +1089,13 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
       const int ntiles = scanned_tiles(item_tiles(w, &m0, &j_begin));
       if constexpr (kAsync) {
         if (!Claim || i == 0) {
-          const WarmUp wu = warm_tiles(i, w, ntiles);
-          // ranked: the least minima, sorted, behind slots that nothing displaces
+          const WarmUp wu = warm_tiles(i, w, m0, ntiles);
+          // the least minima, sorted, behind slots that nothing displaces
           constexpr int kRanked = kRankedMax<Epilogue::KMAX, QT>;
+          const int need = (out.K1 * QT + 1) / 2, ranks = wu.pairs ? (need + 1) / 2 : need;
           int32_t ranked[kRanked > 0 ? kRanked : 1];
 #pragma unroll
-          for (int j = 0; j < kRanked; ++j) ranked[j] = j < kRanked - (out.K1 * QT + 1) / 2 ? INT32_MIN : INT32_MAX;
+          for (int j = 0; j < kRanked; ++j) ranked[j] = j < kRanked - ranks ? INT32_MIN : INT32_MAX;
           int32_t most = wu.tiles > 0 ? INT32_MIN : INT32_MAX;
           bool ok = true;
           for (int u = 0; u < wu.tiles; ++u, ++tg) {
@@ -1067,19 +1107,29 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
               uint32_t v[32], mn;
               tmem_ld_min_32x32b_x32(taddr + c, v, mn);
               tmem_ld_wait(v, mn);
-              if (kRanked > 0 && wu.ranked) {
+              if constexpr (kRanked > 0) {
+                int32_t y[4] = {(int32_t)mn, INT32_MAX, INT32_MAX, INT32_MAX};
+                if (wu.octets || wu.pairs) group_values(v, wu.octets, wu.pairs, y);
+#pragma unroll 1
+                for (int g = 0; g < (wu.octets ? 4 : 1); ++g) {
+                  const int32_t x = y[0];
+                  y[0] = y[1];
+                  y[1] = y[2];
+                  y[2] = y[3];
+                  if (!__any_sync(0xffffffffu, x < ranked[kRanked - 1])) continue;
 #pragma unroll
-                for (int j = kRanked - 1; j > 0; --j) ranked[j] = max(ranked[j - 1], min(ranked[j], (int32_t)mn));
-                ranked[0] = min(ranked[0], (int32_t)mn);
+                  for (int j = kRanked - 1; j > 0; --j) ranked[j] = max(ranked[j - 1], min(ranked[j], x));
+                  ranked[0] = min(ranked[0], x);
+                }
               } else {
-                if (wu.fine) most = max(most, (int32_t)mn);
+                if (wu.octets) most = max(most, (int32_t)mn);
                 least = min(least, (int32_t)mn);
               }
             }
             release_tile();
-            if (!wu.fine) most = max(most, least);
+            if (kRanked == 0 && !wu.octets) most = max(most, least);
           }
-          if (kRanked > 0 && wu.ranked) most = ranked[kRanked - 1];
+          if (kRanked > 0 && wu.tiles > 0) most = ranked[kRanked - 1];
           if (!ok) break;
           st_shared_u32(ho.warm(t), (uint32_t)most);
           __syncwarp();
@@ -1173,7 +1223,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           const uint32_t t = (uint32_t)(q * kBM) + quarter * 32 + (uint32_t)lane;
           int32_t bound = (int32_t)ld_shared_u32(ins.ho.warm(t));
           if (QT == 1) bound = max(bound, (int32_t)ld_shared_u32(ins.ho.warm(t + kBM)));
-          ins.shared[q] = ins.rthr[q] ? __ldcg(ins.rthr[q]) : kNoBound;
+          ins.shared[q] = ins.rthr[q] ? min(__ldcg(ins.rthr[q]), kRealBound) : kRealBound;
           if (bound < ins.shared[q]) {
             ins.shared[q] = bound;
             if (share && ins.rthr[q]) atomicMin(ins.rthr[q], bound);

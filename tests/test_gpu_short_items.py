@@ -1,0 +1,93 @@
+"""Scans of few reference tiles, whose lists start from a limit taken over groups of 8
+or 32 columns (of pairs of columns for the longest lists): every list kind, tiles
+that are mostly padding, falling distances and ties, against the oracle; and what
+longer lists cost on a small index."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def lnbnn():
+    from paper_1112_0059_gb300 import build, lnbnn
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    build.build()
+    lnbnn.load_library()
+    return lnbnn
+
+
+def _refs(rng, N, kind):
+    if kind == "falling":  # every later row is nearer: all of them pass the limit
+        ref = np.zeros((N, 128), np.uint8)
+        level = np.linspace(255, 0, N)[:, None]
+        ref[:] = np.clip(level + rng.integers(0, 3, (N, 128)), 0, 255)
+        return ref
+    if kind == "ties":  # few different rows
+        return np.repeat(rng.integers(0, 256, (max(1, N // 40), 128)), 41, axis=0)[:N].astype(np.uint8)
+    return rng.integers(0, 256, (N, 128)).astype(np.uint8)
+
+
+@pytest.mark.parametrize("kind", ["random", "falling", "ties"])
+@pytest.mark.parametrize("N,M", [(257, 3), (600, 130), (785, 40), (2000, 300), (4100, 17), (10_000, 300)])
+def test_every_list_length(lnbnn, N, M, kind):
+    rng = np.random.default_rng(N + M)
+    ref = _refs(rng, N, kind)
+    N = len(ref)
+    q = rng.integers(0, 256, (M, 128)).astype(np.uint8) if kind != "falling" else np.zeros((M, 128), np.uint8)
+    with lnbnn.Index(torch.from_numpy(ref).cuda(), torch.zeros(N, dtype=torch.int32, device="cuda"), 1) as ix:
+        ix.prepare_fp8()
+        qd = torch.from_numpy(q).cuda()
+        wd, wi = oracle.knn(ref, q, min(255, N))
+        for k in (1, 2, 16, 17, 32, 33, 64, 65, 128, 129, 200, 255):
+            if k > N:
+                continue
+            i, d = ix.knn_search(qd, k)
+            ix.sync()
+            assert np.array_equal(d.cpu().numpy(), wd[:, :k]) and np.array_equal(i.cpu().numpy(), wi[:, :k]), k
+        for s in (10, 24, 64, 128, 256):
+            i, d = ix.knn_search(qd, 7, shortlist=s)
+            ix.sync()
+            cd, ci = oracle.knn_coarse(ref, q, 7, min(s, N))
+            assert np.array_equal(d.cpu().numpy(), cd) and np.array_equal(i.cpu().numpy(), ci), s
+
+
+@pytest.mark.parametrize("query_tiles", [1, 2])
+def test_more_query_tiles_than_sms(lnbnn, query_tiles):
+    N, M = 1030, 160 * 128 + 5
+    rng = np.random.default_rng(9)
+    ref, q = _refs(rng, N, "random"), rng.integers(0, 256, (M, 128)).astype(np.uint8)
+    rows = np.concatenate([np.arange(70), rng.choice(M, 300, replace=False), np.arange(M - 70, M)])
+    with lnbnn.Index(torch.from_numpy(ref).cuda(), torch.zeros(N, dtype=torch.int32, device="cuda"), 1) as ix:
+        ix.set_schedule(query_tiles=query_tiles)
+        qd = torch.from_numpy(q).cuda()
+        wd, wi = oracle.knn(ref, q[rows], 255)
+        for k in (1, 10, 24, 32, 50, 100, 255):
+            i, d = ix.knn_search(qd, k)
+            ix.sync()
+            assert np.array_equal(d.cpu().numpy()[rows], wd[:, :k]) and np.array_equal(i.cpu().numpy()[rows], wi[:, :k]), k
+
+
+def test_time_of_longer_lists(lnbnn):
+    """20,000 queries against 20,000 references: k = 50 takes about as long as k = 32,
+    k = 100 two to three times that (3 and 6 times where short items start from no limit)."""
+    rng = np.random.default_rng(3)
+    ref = torch.from_numpy(_refs(rng, 20_000, "random")).cuda()
+    q = torch.from_numpy(_refs(rng, 20_000, "random")).cuda()
+    us = {}
+    with lnbnn.Index(ref, torch.zeros(len(ref), dtype=torch.int32, device="cuda"), 1) as ix:
+        for k in (32, 50, 100):
+            times = []
+            for _ in range(5):
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                a.record()
+                ix.knn_search(q, k)
+                b.record()
+                torch.cuda.synchronize()
+                times.append(a.elapsed_time(b) * 1e3)
+            us[k] = min(times)
+    assert us[50] < 1.9 * us[32] and us[100] < 4.2 * us[32], us
