@@ -1493,7 +1493,7 @@ cudaError_t launch_lists(const TcTensorMaps& maps, bool sorted_copy, const void*
                          int64_t m, int64_t m_pad, int64_t n_ref, int splits, int64_t split_len, int K1,
                          const ScanOut& out, uint32_t* dev_err, unsigned long long* stats, const TcSched& sched,
                          cudaStream_t s) {
-  switch (tc_list_max(K1)) {
+  switch (tc_list_max(K1, m)) {
     case kTcRegListMax:
       return launch_shape<Fmt, KnnEpilogue<kTcRegListMax>>(maps, sorted_copy, qop, qext, m, m_pad, n_ref, splits,
                                                            split_len, out, dev_err, stats, sched, s);

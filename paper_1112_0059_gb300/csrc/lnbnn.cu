@@ -360,12 +360,13 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   p.m_pad = round_up(m, kQueryPad);
   p.K1 = K1;
   const int64_t T1 = p.m_pad / kTcQueryTile;
-  const bool qt2_ok = kind == ScanKind::Nbnn || K1 <= kTcCoarseRegListMax || K1 > kTcWideRegListMax;
+  const bool wide = kind != ScanKind::Nbnn && tc_list_max(K1, m) == kTcWideRegListMax;
+  const bool qt2_ok = !wide;
   p.qt = qt2_ok && (o.query_tiles == 2 || (o.query_tiles == 0 && auto_query_tiles(ix, kind, T1) == 2)) ? 2 : 1;
   const int64_t T = (T1 + p.qt - 1) / p.qt;
   if (splits <= 0) splits = o.splits;
   // The claimed-chunk form for launches of fewer query-tile groups than SMs
-  // (automatic split count; lists of up to 32 keys or more than 64): on a class-sorted
+  // (automatic split count; no lists of 64 registers): on a class-sorted
   // index the few reference ranges that hold a query's own class carry most
   // of the list inserts, and with fixed splits the CTAs that draw them set
   // the launch's time.  Instead each of P / T CTAs per group keeps the
@@ -376,8 +377,7 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
   // (256-class data, shortlist 24, 632 descriptors: 854 us a call against 908
   // with splits; with fewer CTAs a tile the rest of the SMs idle); the exact
   // scan for a lone query tile only (100 descriptors: 530 against 560 us).
-  const bool claim_kind = kind != ScanKind::Nbnn && (K1 <= kTcCoarseRegListMax || K1 > kTcWideRegListMax) &&
-                          (kind == ScanKind::Coarse ? T * 8 <= P : T == 1);
+  const bool claim_kind = kind != ScanKind::Nbnn && !wide && (kind == ScanKind::Coarse ? T * 8 <= P : T == 1);
   const int64_t ref_tiles = (ix->n_ref + kTcRefTile - 1) / kTcRefTile;
   p.group = may_claim && splits <= 0 && T < P && p.qt == 1 && claim_kind && o.persistent != 0 && o.bound_per_tile != 0
                 // chunks of >= 4 tiles each, and no more lists than the split
@@ -940,8 +940,9 @@ lnbnn_status lnbnn_plan_search(const lnbnn_index* index, int64_t n_queries, int3
   r.splits = p.splits;
   r.lists_per_row = p.splits;
   r.split_len = p.split_len;
-  r.list_storage = tc_list_max(k1) > 0 ? 0 : 2;
-  r.list_capacity = tc_list_max(k1) > 0 ? tc_list_max(k1) : k1;
+  const int list = tc_list_max(k1, n_queries);
+  r.list_storage = list > 0 ? 0 : 2;
+  r.list_capacity = list > 0 ? list : k1;
   r.tile_m = kTcQueryTile * p.qt;
   r.tile_n = kTcRefTile / p.qt;
   r.persistent = p.persistent ? 1 : 0;

@@ -72,6 +72,24 @@ def test_more_query_tiles_than_sms(lnbnn, query_tiles):
             assert np.array_equal(d.cpu().numpy()[rows], wd[:, :k]) and np.array_equal(i.cpu().numpy()[rows], wi[:, :k]), k
 
 
+@pytest.mark.parametrize("M", [1, 4, 5])
+def test_few_rows_keep_long_lists_in_memory(lnbnn, M):
+    rng = np.random.default_rng(M)
+    for N in (600, 30_000):
+        ref, q = _refs(rng, N, "random"), rng.integers(0, 256, (M, 128)).astype(np.uint8)
+        with lnbnn.Index(torch.from_numpy(ref).cuda(), torch.zeros(N, dtype=torch.int32, device="cuda"), 1) as ix:
+            ix.prepare_fp8()
+            for k in (33, 50, 64):
+                assert (ix.plan_search(M, k)["list_storage"] == "registers") == (M > 4)
+                i, d = ix.knn_search(torch.from_numpy(q).cuda(), k)
+                fi, fd = ix.knn_search(torch.from_numpy(q).cuda(), 5, shortlist=k)
+                ix.sync()
+                wd, wi = oracle.knn(ref, q, k)
+                assert np.array_equal(d.cpu().numpy(), wd) and np.array_equal(i.cpu().numpy(), wi)
+                cd, ci = oracle.knn_coarse(ref, q, 5, k)
+                assert np.array_equal(fd.cpu().numpy(), cd) and np.array_equal(fi.cpu().numpy(), ci)
+
+
 def test_time_of_longer_lists(lnbnn):
     """20,000 queries against 20,000 references: k = 50 takes about as long as k = 32,
     k = 100 two to three times that (3 and 6 times where short items start from no limit)."""
