@@ -255,6 +255,18 @@ bool auto_persistent(const lnbnn_index* ix, ScanKind k, int64_t T1) {
   return T1 >= ix->sm_count && ix->auto_persistent[(int)k] == 1;
 }
 
+// Exact scans of at least a full wave of short items take a persistent grid
+// whatever was measured on large batches: a CTA's start and its inserters' last
+// merge then overlap the next item.  One CTA per item / persistent, 100,000
+// queries: 600 references, k = 20 346 / 297 us, 5,000, k = 10 360 / 298, 20,000
+// 1,203 / 1,125, 60,000 1,961 / 1,877; from about 400 tiles on it is the number of
+// waves that decides (200,000 references, k = 10, 20,000 queries 1,007 / 938 us, k = 50
+// 2,213 / 2,327).
+constexpr int64_t kShortItemTiles = 256;
+bool short_items(ScanKind k, int64_t T1, int64_t sm_count, int64_t split_len) {
+  return k == ScanKind::Exact && T1 >= sm_count && split_len <= kShortItemTiles * kTcRefTile;
+}
+
 // Splits for the exact scan of a launch of at least a full wave whose lists
 // are longer than 16 keys: with the splits run one after another and their
 // lists carried across, the later splits insert little, and a last wave that
@@ -402,7 +414,8 @@ KnnPlan plan_knn(const lnbnn_index* ix, int64_t m, int K1, ScanKind kind, int sp
     }
     p.split_len = round_up((ix->n_ref + splits - 1) / splits, kTcRefTile);
     p.splits = (int)((ix->n_ref + p.split_len - 1) / p.split_len);
-    p.persistent = o.persistent == 1 || (o.persistent == -1 && auto_persistent(ix, kind, T1));
+    p.persistent = o.persistent == 1 || (o.persistent == -1 && (auto_persistent(ix, kind, T1) ||
+                                                              short_items(kind, T1, P, p.split_len)));
     p.bound_per_tile = o.bound_per_tile >= 0 ? o.bound_per_tile == 1 : T < P;
   }
   p.items = T * p.splits;
