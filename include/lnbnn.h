@@ -294,7 +294,7 @@ LNBNN_API lnbnn_status lnbnn_classify_fp8_ws(lnbnn_index *index, lnbnn_workspace
  * on whether it has).  A launch of few query tiles with an automatic split
  * count takes the claimed-chunk form instead of splits (the FP8 coarse pass
  * while there are at least 8 SMs per query tile, the exact scan for a lone
- * query tile; lists of up to 32 or more than 64 keys, for at most 4 queries of
+ * query tile; lists of up to 32 or more than 64 keys, for at most 8 queries of
  * any length): each of P / T CTAs per
  * query tile keeps that tile's lists for the whole launch and claims short
  * reference chunks, in increasing order, from a counter the tile's CTAs

@@ -721,6 +721,15 @@ struct Work {
 
 // Claim: the claimed-chunk form (Work::group > 0), a separate instantiation
 // so that the split form's kernels carry none of its code.
+// Query rows of each TMEM lane quarter: 32, or for a launch of at most 96 rows a
+// quarter of them each, since a quarter's rows have one inserter warp.  Its 32
+// lanes hold consecutive operand rows either way, and lanes past the quarter's
+// rows are inactive.  FP8 shortlist 100, 1.5 million references, 16, 32, 64 and 96
+// rows, 32 to a quarter / spread: 602, 922, 956 and 998 / 349, 454, 645 and 841 us;
+// 2,000 references, k = 100, 32 rows 618 / 259 us.
+constexpr int kSpreadRows = 96;
+__host__ __device__ constexpr int quarter_rows(int64_t m) { return m <= kSpreadRows ? (int)((m + 3) / 4) : 32; }
+
 template <class Fmt, class Epilogue, int QT, bool Claim>
 __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
     tc_scan_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_qe,
@@ -833,7 +842,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   // lists go on from the previous chunk or split.
   auto warm_tiles = [&](int i, int64_t w, int64_t m0, int ntiles) -> WarmUp {
     if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false, false};
-    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1, m - m0, out.bound_per_tile && out.row_thr != nullptr);
+    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1, min(m - m0, (int64_t)quarter_rows(m)), out.bound_per_tile && out.row_thr != nullptr);
   };
 
   if (warp < kEpiWarp0) {
@@ -883,9 +892,13 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
             mbar_arrive_expect_tx(bars.afull(), QT * (KC * kAChunkBytes + kAExtBytes));
             for (int q = 0; q < QT; ++q) {
               const uint32_t a = sbase + L::kOffA + q * L::kAQueryBytes;
-              const int32_t qrow = (int32_t)(m0 + q * kBM);
-              for (int kc = 0; kc < KC; ++kc) tma_load_2d(a + kc * kAChunkBytes, &tmap_q, kc * kBK, qrow, bars.afull());
-              tma_load_2d(a + KC * kAChunkBytes, &tmap_qe, 0, qrow, bars.afull());
+              const int boxes = m <= kSpreadRows ? 4 : 1;  // (of 32 rows each, or one of 128)
+              for (int b = 0; b < boxes; ++b) {
+                const int32_t qrow = (int32_t)(m0 + q * kBM) + b * quarter_rows(m);
+                for (int kc = 0; kc < KC; ++kc)
+                  tma_load_2d(a + kc * kAChunkBytes + b * (kAChunkBytes / 4), &tmap_q, kc * kBK, qrow, bars.afull());
+                tma_load_2d(a + KC * kAChunkBytes + b * (kAExtBytes / 4), &tmap_qe, 0, qrow, bars.afull());
+              }
             }
             ++a_loads;
           }
@@ -1146,8 +1159,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
           if (lane == 0) mbar_arrive(bars.queued());
         }
       } else {
-        const int64_t row = m0 + (QT == 2 ? half * kBM : 0) + quarter * 32 + lane;
-        Epilogue epi(out, row, row < m, j_begin + c_off);
+        const int64_t row = m0 + (QT == 2 ? half * kBM : 0) + quarter * quarter_rows(m) + lane;
+        Epilogue epi(out, row, lane < quarter_rows(m) && row < m, j_begin + c_off);
         const bool ok = scan_tiles(epi, ntiles, j_begin + c_off);
         epi.finish();
         if (!ok) break;
@@ -1204,9 +1217,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         if (!ok) flag_timeout(abort_flag, dev_err);  // (the lists are written all the same, empty)
 #pragma unroll
         for (int q = 0; q < QT; ++q) {
-          const int64_t row = m0 + q * kBM + quarter * 32 + lane;
-          const bool active = row < m;
-          const int64_t first = m0 + q * kBM + quarter * 32;
+          const int64_t first = m0 + q * kBM + quarter * quarter_rows(m), row = first + lane;
+          const bool active = lane < quarter_rows(m) && row < m;
           ins.list[q] = out.lists + (y * out.stride + first) * out.K1;
           ins.seed[q] = carried ? ins.list[q] - out.stride * out.K1 : nullptr;
           ins.listed[q] = 0u;
@@ -1262,8 +1274,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         }
 #pragma unroll
         for (int q = 0; q < QT; ++q) {
-          const int64_t left = m - (m0 + q * kBM + quarter * 32);
-          ins.finish(q, (uint32_t)max(int64_t(0), min(left, int64_t(32))));
+          const int64_t left = m - (m0 + q * kBM + quarter * quarter_rows(m));
+          ins.finish(q, (uint32_t)max(int64_t(0), min(left, (int64_t)quarter_rows(m))));
           if (ins.rthr[q] && !out.bound_per_tile && ins.kth[q] < ins.shared[q]) atomicMin(ins.rthr[q], ins.kth[q]);
         }
         if (chain) {
@@ -1383,10 +1395,11 @@ cudaError_t launch_scan(const CUtensorMap& tr, const CUtensorMap& tre, const voi
   if (m_pad % kBM != 0 || split_len % kTcRefTile != 0 || splits < 1) return cudaErrorInvalidValue;
   if (sched.persistent_ctas > 0 && sched.queue == nullptr) return cudaErrorInvalidValue;
   CUtensorMap tq, tqe;
+  const uint32_t box = m <= kSpreadRows ? 32 : kBM;
   const bool ok = Fmt::kChunks == 1
-                      ? encode_e4m3(&tq, qop, (uint64_t)m_pad, kBM) &&
-                            encode_bf16(&tqe, qext, (uint64_t)m_pad, kExt, kExt, kBM, CU_TENSOR_MAP_SWIZZLE_32B)
-                      : encode_operand(&tq, &tqe, qop, qext, (uint64_t)m_pad, kBM);
+                      ? encode_e4m3(&tq, qop, (uint64_t)m_pad, box) &&
+                            encode_bf16(&tqe, qext, (uint64_t)m_pad, kExt, kExt, box, CU_TENSOR_MAP_SWIZZLE_32B)
+                      : encode_operand(&tq, &tqe, qop, qext, (uint64_t)m_pad, box);
   if (!ok) return cudaErrorInvalidValue;
   Work work;
   work.T = (m_pad + kBM * QT - 1) / (kBM * QT);

@@ -49,10 +49,10 @@ inline TcWork tc_fit_work(int K1, int64_t ctas, int64_t bytes) {
 // The kernel instantiation for lists of K1 keys of m queries: the longest list
 // it takes, 0 for the longest.  An insertion into 64 registers a thread is the
 // same work for one row as for 32, a merge into lists in global memory is paid
-// by the row, so few rows keep 33..64 keys that way: 20,000 references, k = 50,
-// 1, 4 and 8 queries 97, 121 and 150 us, in registers 124, 122 and 137; 1.5
-// million, k = 63 173, 231 and 299 us, in registers 206, 230 and 239.
-constexpr int64_t kTcFewRows = 4;
+// by the row, so few rows keep 33..64 keys that way: 2,000 references, k = 63, 1, 4,
+// 8 and 16 queries 99, 108, 126 and 148 us, in registers 132, 142, 167 and 179; 20,000
+// references, k = 40 90, 98, 113 and 129 us, in registers 100, 100, 111 and 118.
+constexpr int64_t kTcFewRows = 8;
 inline int tc_list_max(int K1, int64_t m) {
   if (K1 > kTcCoarseRegListMax && m <= kTcFewRows) return 0;
   return K1 <= kTcRegListMax         ? kTcRegListMax
