@@ -717,27 +717,22 @@ struct Work {
   // split_len rows, in increasing order, from the group's counter
   // queue[c / group]; n_items is then the number of chunks.
   int group;
+  // Query rows of each TMEM lane quarter: 32, or for a launch of at most
+  // kSpreadRows a quarter of them each, since a quarter's rows have one inserter
+  // warp.  Only in the instantiations that such launches have (it cost the others
+  // up to 1%: NBNN, the FP8 pass of large batches).  Its 32 lanes
+  // hold consecutive operand rows either way, and lanes past the quarter's rows
+  // are inactive.  FP8 shortlist 100, 1.5 million references, 16, 32, 64 and 96
+  // rows, 32 to a quarter / spread: 602, 922, 956 and 998 / 349, 454, 645 and 841 us;
+  // 2,000 references, k = 100, 32 rows 618 / 259 us.
+  int quarter;
 };
+constexpr int64_t kSpreadRows = 96;
+template <class Epilogue, bool Claim>
+constexpr bool kSpreads = Epilogue::kInserterWarps > 0 && (Claim || Epilogue::KMAX == kTcWideRegListMax);
 
 // Claim: the claimed-chunk form (Work::group > 0), a separate instantiation
 // so that the split form's kernels carry none of its code.
-// Query rows of each TMEM lane quarter: 32, or for a launch of at most 96 rows a
-// quarter of them each, since a quarter's rows have one inserter warp (not where
-// there are none: it cost the NBNN scan 0.5%).  Its 32
-// lanes hold consecutive operand rows either way, and lanes past the quarter's
-// rows are inactive.  FP8 shortlist 100, 1.5 million references, 16, 32, 64 and 96
-// rows, 32 to a quarter / spread: 602, 922, 956 and 998 / 349, 454, 645 and 841 us;
-// 2,000 references, k = 100, 32 rows 618 / 259 us.
-constexpr int kSpreadRows = 96;
-template <class Epilogue>
-__host__ __device__ constexpr bool spread_rows(int64_t m) {
-  return Epilogue::kInserterWarps > 0 && m <= kSpreadRows;
-}
-template <class Epilogue>
-__host__ __device__ constexpr int quarter_rows(int64_t m) {
-  return spread_rows<Epilogue>(m) ? (int)((m + 3) / 4) : 32;
-}
-
 template <class Fmt, class Epilogue, int QT, bool Claim>
 __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
     tc_scan_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_qe,
@@ -756,6 +751,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   // tile cost the MMA thread 2-10% of a step.
   static_assert(kStages >= 2 * KC, "the ring holds two tiles");
   constexpr bool kAsync = Epilogue::kInserterWarps > 0;  // lists kept by inserter warps
+  const int quarter_rows = kSpreads<Epilogue, Claim> ? work.quarter : 32;
   constexpr int kListWarps = 4;                        // inserter warps
   constexpr int kEpiPerQuarter = kEpiWarps / 4;
   constexpr int kEpiCols = kAccCols / kEpiPerQuarter;  // accumulator columns per epilogue warp
@@ -850,7 +846,7 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
   // lists go on from the previous chunk or split.
   auto warm_tiles = [&](int i, int64_t w, int64_t m0, int ntiles) -> WarmUp {
     if (!kAsync || (Claim && i > 0) || (!Claim && out.done != nullptr && w >= work.T)) return WarmUp{0, false, false};
-    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1, min(m - m0, (int64_t)quarter_rows<Epilogue>(m)), out.bound_per_tile && out.row_thr != nullptr);
+    return warm_up<Epilogue::KMAX, QT, Claim>(ntiles, out.K1, min(m - m0, (int64_t)quarter_rows), out.bound_per_tile && out.row_thr != nullptr);
   };
 
   if (warp < kEpiWarp0) {
@@ -900,9 +896,9 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
             mbar_arrive_expect_tx(bars.afull(), QT * (KC * kAChunkBytes + kAExtBytes));
             for (int q = 0; q < QT; ++q) {
               const uint32_t a = sbase + L::kOffA + q * L::kAQueryBytes;
-              const int boxes = spread_rows<Epilogue>(m) ? 4 : 1;  // (of 32 rows each, or one of 128)
+              const int boxes = quarter_rows < 32 ? 4 : 1;  // (of 32 rows each, or one of 128)
               for (int b = 0; b < boxes; ++b) {
-                const int32_t qrow = (int32_t)(m0 + q * kBM) + b * quarter_rows<Epilogue>(m);
+                const int32_t qrow = (int32_t)(m0 + q * kBM) + b * quarter_rows;
                 for (int kc = 0; kc < KC; ++kc)
                   tma_load_2d(a + kc * kAChunkBytes + b * (kAChunkBytes / 4), &tmap_q, kc * kBK, qrow, bars.afull());
                 tma_load_2d(a + KC * kAChunkBytes + b * (kAExtBytes / 4), &tmap_qe, 0, qrow, bars.afull());
@@ -1225,8 +1221,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         if (!ok) flag_timeout(abort_flag, dev_err);  // (the lists are written all the same, empty)
 #pragma unroll
         for (int q = 0; q < QT; ++q) {
-          const int64_t first = m0 + q * kBM + quarter * quarter_rows<Epilogue>(m), row = first + lane;
-          const bool active = lane < quarter_rows<Epilogue>(m) && row < m;
+          const int64_t first = m0 + q * kBM + quarter * quarter_rows, row = first + lane;
+          const bool active = lane < quarter_rows && row < m;
           ins.list[q] = out.lists + (y * out.stride + first) * out.K1;
           ins.seed[q] = carried ? ins.list[q] - out.stride * out.K1 : nullptr;
           ins.listed[q] = 0u;
@@ -1282,8 +1278,8 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
         }
 #pragma unroll
         for (int q = 0; q < QT; ++q) {
-          const int64_t left = m - (m0 + q * kBM + quarter * quarter_rows<Epilogue>(m));
-          ins.finish(q, (uint32_t)max(int64_t(0), min(left, (int64_t)quarter_rows<Epilogue>(m))));
+          const int64_t left = m - (m0 + q * kBM + quarter * quarter_rows);
+          ins.finish(q, (uint32_t)max(int64_t(0), min(left, (int64_t)quarter_rows)));
           if (ins.rthr[q] && !out.bound_per_tile && ins.kth[q] < ins.shared[q]) atomicMin(ins.rthr[q], ins.kth[q]);
         }
         if (chain) {
@@ -1403,7 +1399,8 @@ cudaError_t launch_scan(const CUtensorMap& tr, const CUtensorMap& tre, const voi
   if (m_pad % kBM != 0 || split_len % kTcRefTile != 0 || splits < 1) return cudaErrorInvalidValue;
   if (sched.persistent_ctas > 0 && sched.queue == nullptr) return cudaErrorInvalidValue;
   CUtensorMap tq, tqe;
-  const uint32_t box = spread_rows<Epilogue>(m) ? 32 : kBM;
+  const bool spread = (sched.group > 0 ? kSpreads<Epilogue, true> : kSpreads<Epilogue, false>) && m <= kSpreadRows;
+  const uint32_t box = spread ? 32 : kBM;
   const bool ok = Fmt::kChunks == 1
                       ? encode_e4m3(&tq, qop, (uint64_t)m_pad, box) &&
                             encode_bf16(&tqe, qext, (uint64_t)m_pad, kExt, kExt, box, CU_TENSOR_MAP_SWIZZLE_32B)
@@ -1415,6 +1412,7 @@ cudaError_t launch_scan(const CUtensorMap& tr, const CUtensorMap& tre, const voi
   work.split_len = split_len;
   work.queue = sched.persistent_ctas > 0 ? sched.queue : nullptr;
   work.group = 0;
+  work.quarter = spread ? (int)((m + 3) / 4) : 32;
   ScanOut o = out;
   o.done = splits > 1 ? sched.done : nullptr;
   o.T = work.T;

@@ -177,22 +177,9 @@ __device__ __forceinline__ bool chunk_of(const int64_t* __restrict__ offsets, in
   return true;
 }
 
-// Adds the increments of rows [r, r + rows) of class c to acc, in row order;
-// e(i): exp(-x) of row r + i.
-template <class Exp>
-__device__ __forceinline__ double add_rows(const int32_t* mins, int64_t r, int rows, int32_t C, int32_t c, double beta,
-                                           double log_c1, int positive_only, const RowStat* st, Exp e, double acc,
-                                           unsigned long long* n) {
-#pragma unroll 4
-  for (int i = 0; i < rows; ++i) {
-    const double x = beta * (double)(mins[(r + i) * C + c] - st[i].dmin);
-    const double inc = c == st[i].cstar ? st[i].inc : -x - log(st[i].s - e(i, x)) + log_c1;
-    if (!positive_only || inc > 0.0) {
-      acc += inc;
-      ++*n;
-    }
-  }
-  return acc;
+// The increment of a row with statistics t to class c, x = beta (D_c - Dmin), e = exp(-x).
+__device__ __forceinline__ double increment(const RowStat& t, int32_t c, double x, double e, double log_c1) {
+  return c == t.cstar ? t.inc : -x - log(t.s - e) + log_c1;
 }
 
 __device__ __forceinline__ void add_count(unsigned long long* counts, int64_t img, unsigned long long n) {
@@ -203,7 +190,7 @@ __device__ __forceinline__ void add_count(unsigned long long* counts, int64_t im
 }
 
 // Up to kTableClasses classes: statistics and sums of a chunk.  kFull: kThreads
-// threads (a stride known to the compiler: 147 us of a call, 150 without).
+// threads (a stride known to the compiler).
 template <bool kFull>
 __global__ void __launch_bounds__(kThreads)
     logodds_chunk_kernel(int32_t* __restrict__ mins, int64_t m, int32_t C, double beta, double log_c1, int positive_only,
@@ -227,8 +214,17 @@ __global__ void __launch_bounds__(kThreads)
     __syncthreads();
     for (int32_t c = threadIdx.x; c < C; c += threads) {
       double* sum = split ? part + c : totals + img * C + c;
-      *sum = add_rows(mins, r, rows, C, c, beta, log_c1, positive_only, st,
-                      [&](int i, double) { return table[(int64_t)i * C + c]; }, r == r0 ? 0.0 : *sum, &n);
+      double acc = r == r0 ? 0.0 : *sum;
+#pragma unroll 4
+      for (int i = 0; i < rows; ++i) {
+        const double x = beta * (double)(mins[(r + i) * C + c] - st[i].dmin);
+        const double inc = increment(st[i], c, x, table[(int64_t)i * C + c], log_c1);
+        if (!positive_only || inc > 0.0) {
+          acc += inc;
+          ++n;
+        }
+      }
+      *sum = acc;
     }
   }
   add_count(counts, img, n);
@@ -261,31 +257,22 @@ __global__ void __launch_bounds__(kThreads)
   unsigned long long n = 0;
   const int32_t c = (int32_t)blockIdx.y * kThreads + threadIdx.x;
   if (c < C) {
-    const double acc = add_rows(mins, r0, (int)(r1 - r0), C, c, beta, log_c1, positive_only, stat + r0,
-                                [](int, double x) { return exp(-x); }, 0.0, &n);
+    double acc = 0.0;
+#pragma unroll 4
+    for (int64_t r = r0; r < r1; ++r) {
+      const double x = beta * (double)(mins[r * C + c] - stat[r].dmin);
+      const double inc = increment(stat[r], c, x, exp(-x), log_c1);
+      if (!positive_only || inc > 0.0) {
+        acc += inc;
+        ++n;
+      }
+    }
     if (split)
       put_partial(mins, r0, C, c, acc);
     else
       totals[img * C + c] = acc;
   }
   add_count(counts, img, n);
-}
-
-// v(0) + ... + v(chunks - 1) in that order, eight loads at a time (125 chunks of
-// 256 classes: 25 us, 33 as one loop).
-template <class Value>
-__device__ __forceinline__ double ordered_sum(int64_t chunks, Value v) {
-  double sum = 0.0;
-  int64_t j = 0;
-  for (; j + 8 <= chunks; j += 8) {
-    double x[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = v(j + u);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) sum += x[u];
-  }
-  for (; j < chunks; ++j) sum += v(j);
-  return sum;
 }
 
 // and these sums in the chunks' order, an image and kThreads classes a block.
@@ -296,26 +283,33 @@ __global__ void __launch_bounds__(kThreads)
   const int32_t c = (int32_t)blockIdx.y * kThreads + threadIdx.x;
   const int64_t o0 = max(offsets[img], (int64_t)0), o1 = min(offsets[img + 1], m);
   const int64_t chunks = o1 <= o0 ? 0 : (o1 - o0) / kChunk;
-  if (c < C && chunks > 1)
-    totals[img * C + c] = ordered_sum(chunks, [&](int64_t j) { return partial(mins, o0 + j * kChunk, C, c); });
+  if (c >= C || chunks < 2) return;
+  double v = 0.0;
+#pragma unroll 8
+  for (int64_t j = 0; j < chunks; ++j) v += partial(mins, o0 + j * kChunk, C, c);
+  totals[img * C + c] = v;
 }
 
 // One block per image: the chunks' sums (unless summed), then the argmax over
-// classes, the lowest class on ties.
+// classes, the lowest class on ties.  kFull: kThreads threads.
+template <bool kFull>
 __global__ void __launch_bounds__(kThreads)
     logodds_finish_kernel(int32_t* __restrict__ mins, int64_t m, int32_t C, const int64_t* __restrict__ offsets,
                           bool summed, double* __restrict__ totals, int32_t* __restrict__ classes) {
   __shared__ double best_s[kWarps];
   __shared__ int32_t class_s[kWarps];
+  const int threads = kFull ? kThreads : (int)blockDim.x;
   const int64_t img = blockIdx.x;
   const int64_t o0 = max(offsets[img], (int64_t)0), o1 = min(offsets[img + 1], m);
   const int64_t chunks = summed || o1 <= o0 ? 0 : (o1 - o0) / kChunk;
   double best = -INFINITY;
   int32_t bc = INT32_MAX;
-  for (int32_t c = threadIdx.x; c < C; c += blockDim.x) {
+  for (int32_t c = threadIdx.x; c < C; c += threads) {
     double v;
     if (chunks > 1) {
-      v = ordered_sum(chunks, [&](int64_t j) { return __ldcg(partials(mins, o0 + j * kChunk, C) + c); });
+      v = 0.0;
+#pragma unroll 8
+      for (int64_t j = 0; j < chunks; ++j) v += partials(mins, o0 + j * kChunk, C)[c];
       totals[img * C + c] = v;
     } else {
       v = totals[img * C + c];
@@ -340,7 +334,7 @@ __global__ void __launch_bounds__(kThreads)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+    for (int w = 1; w < (threads >> 5); ++w)
       if (class_s[w] != INT32_MAX && (bc == INT32_MAX || best_s[w] > best || (best_s[w] == best && class_s[w] < bc))) {
         best = best_s[w];
         bc = class_s[w];
@@ -403,8 +397,10 @@ cudaError_t launch_logodds(int32_t* mins, void* rowstat, int64_t m, int32_t C, d
     }
     if (e != cudaSuccess) return e;
   }
-  logodds_finish_kernel<<<(unsigned)n_img, (unsigned)(32 * class_warps), 0, s>>>(mins, m, C, offsets, !tabled || m == 0,
-                                                                                 totals, classes);
+  // (blocks of fewer threads only where there are many: see the chunks)
+  const unsigned finish = n_img > 1024 ? (unsigned)(32 * class_warps) : kThreads;
+  (finish == kThreads ? logodds_finish_kernel<true> : logodds_finish_kernel<false>)<<<(unsigned)n_img, finish, 0, s>>>(
+      mins, m, C, offsets, !tabled || m == 0, totals, classes);
   return launched();
 }
 
