@@ -57,10 +57,10 @@ __host__ __device__ __forceinline__ bool row_layout_ok(int row_bytes, int loc_w)
 
 // Reference preparation (rows of row_bytes bytes): exact BF16 copy of the
 // centred appearance coordinates x - 128 (padding rows up to n_pad: zero),
-// squared norms as fp32 (padding rows get kPadNorm; not if null) and the K-extension
-// [n_pad, kExt] (norm digits, location columns).
+// and the K-extension [n_pad, kExt] (digits of the squared norm, kPadNorm for
+// padding rows; location columns).
 cudaError_t launch_prep_ref(const uint8_t* ref, int64_t n_ref, int64_t n_pad, int row_bytes, int loc_w,
-                            __nv_bfloat16* ref_bf, float* rnorm, __nv_bfloat16* ref_ext, cudaStream_t s);
+                            __nv_bfloat16* ref_bf, __nv_bfloat16* ref_ext, cudaStream_t s);
 // What else the first kernel of a call does beside the query preparation: words
 // of memory set to a value, and the offsets validation.  Each as a launch of
 // its own cost 2-4 us: 2,000 queries against 5,000 rows took 95 us before,
@@ -90,15 +90,9 @@ cudaError_t launch_prep_query(const uint8_t* q, int64_t m, int64_t m_pad, int ro
 // Label histogram; sets *bad when a label is outside [0, C).
 cudaError_t launch_label_hist(const int32_t* labels, int64_t n, int32_t C, unsigned long long* counts,
                               uint32_t* bad, cudaStream_t s);
-// Gather rows: dst[i] = src[perm[i]] for bf16 operand rows, norm-digit rows,
-// norms and labels.
+// Gather rows: dst[i] = src[perm[i]] for bf16 operand rows and norm-digit rows.
 cudaError_t launch_gather_ref(const int64_t* perm, int64_t n, const __nv_bfloat16* src_bf, __nv_bfloat16* dst_bf,
-                              const __nv_bfloat16* src_ext,
-                              __nv_bfloat16* dst_ext, const float* src_norm, float* dst_norm,
-                              const int32_t* src_lab, int32_t* dst_lab, cudaStream_t s);
-
-// dst[0..n) = v
-cudaError_t launch_fill_float(float* dst, int64_t n, float v, cudaStream_t s);
+                              const __nv_bfloat16* src_ext, __nv_bfloat16* dst_ext, cudaStream_t s);
 
 // Merge `splits` sorted lists per row into one sorted list of K1 keys
 // (at most 32 * kMaxListsPerLane lists).  With `chain.done` set (the scan's

@@ -90,7 +90,7 @@ struct TcSched {
   // lists for the whole launch and claiming reference chunks of split_len
   // rows in increasing order from the group's counter queue[group index]
   // (T counters zeroed before the launch); the launch writes `group` x lists
-  // per CTA lists per query row.  kNN register lists and heaps only; never
+  // per CTA lists per query row.  kNN lists only; never
   // with `done`.
   int group = 0;
   // kNN: candidate buffers of the lists in progress, tc_work_bytes(entries)

@@ -28,14 +28,11 @@ struct lnbnn_index {
   uint8_t* ref_u8 = nullptr;         // [n_ref, row_bytes] the descriptors as given
   __nv_bfloat16* ref_bf = nullptr;   // [n_pad, 128] exact BF16 copy, zero padding rows
   __nv_bfloat16* ref_ext = nullptr;  // [n_pad, 16] squared-norm digits (K-extension)
-  float* rnorm = nullptr;            // [n_pad] squared norms, kPadNorm on padding rows
   int32_t* labels = nullptr;        // [n_ref]
   // class-sorted view (aliases the above when the labels are already grouped)
   bool sorted = true;
   __nv_bfloat16* sref_bf = nullptr;
   __nv_bfloat16* sref_ext = nullptr;
-  float* srnorm = nullptr;
-  int32_t* slabels = nullptr;
   std::vector<int64_t> class_off_h;  // [C+1]
   int64_t* class_off_d = nullptr;
   bool has_empty_class = false;
@@ -116,15 +113,12 @@ void free_index(lnbnn_index* ix) {
   if (!ix->sorted) {
     cudaFree(ix->sref_bf);
     cudaFree(ix->sref_ext);
-    cudaFree(ix->srnorm);
-    cudaFree(ix->slabels);
   }
   cudaFree(ix->ref_f8);
   cudaFree(ix->ref_f8_ext);
   cudaFree(ix->ref_u8);
   cudaFree(ix->ref_bf);
   cudaFree(ix->ref_ext);
-  cudaFree(ix->rnorm);
   cudaFree(ix->labels);
   cudaFree(ix->class_off_d);
   cudaFree(ix->dev_err);
@@ -704,7 +698,6 @@ static lnbnn_status create_index(const uint8_t* ref, const int32_t* labels, int6
   CKF(dmalloc(&ix->ref_u8, (size_t)n_ref * row_bytes));
   CKF(dmalloc(&ix->ref_bf, (size_t)ix->n_pad * kDim));
   CKF(dmalloc(&ix->ref_ext, (size_t)ix->n_pad * kExt));
-  CKF(dmalloc(&ix->rnorm, (size_t)ix->n_pad));
   CKF(dmalloc(&ix->labels, (size_t)n_ref));
   CKF(dmalloc(&ix->dev_err, 1));
   CKF(dmalloc(&counts, (size_t)n_classes));
@@ -715,7 +708,7 @@ static lnbnn_status create_index(const uint8_t* ref, const int32_t* labels, int6
   CKF(cudaMemcpyAsync(ix->ref_u8, ref, (size_t)n_ref * row_bytes, cudaMemcpyDeviceToDevice, s));
   CKF(cudaMemcpyAsync(ix->labels, labels, sizeof(int32_t) * n_ref, cudaMemcpyDeviceToDevice, s));
   CKF(launch_label_hist(ix->labels, n_ref, n_classes, counts, bad, s));
-  CKF(launch_prep_ref(ix->ref_u8, n_ref, ix->n_pad, row_bytes, loc_w, ix->ref_bf, ix->rnorm, ix->ref_ext, s));
+  CKF(launch_prep_ref(ix->ref_u8, n_ref, ix->n_pad, row_bytes, loc_w, ix->ref_bf, ix->ref_ext, s));
   std::vector<unsigned long long> cnt(n_classes);
   uint32_t bad_h = 0;
   std::vector<int32_t> lab_h(n_ref);
@@ -736,8 +729,6 @@ static lnbnn_status create_index(const uint8_t* ref, const int32_t* labels, int6
   if (ix->sorted) {
     ix->sref_bf = ix->ref_bf;
     ix->sref_ext = ix->ref_ext;
-    ix->srnorm = ix->rnorm;
-    ix->slabels = ix->labels;
   } else {
     // stable counting sort by class: rows of one class keep their order
     std::vector<int64_t> next(ix->class_off_h.begin(), ix->class_off_h.end() - 1);
@@ -746,17 +737,13 @@ static lnbnn_status create_index(const uint8_t* ref, const int32_t* labels, int6
     CKF(dmalloc(&perm_d, (size_t)n_ref));
     CKF(dmalloc(&ix->sref_bf, (size_t)ix->n_pad * kDim));
     CKF(dmalloc(&ix->sref_ext, (size_t)ix->n_pad * kExt));
-    CKF(dmalloc(&ix->srnorm, (size_t)ix->n_pad));
-    CKF(dmalloc(&ix->slabels, (size_t)n_ref));
     CKF(cudaMemcpyAsync(perm_d, perm.data(), sizeof(int64_t) * n_ref, cudaMemcpyHostToDevice, s));
-    CKF(launch_gather_ref(perm_d, n_ref, ix->ref_bf, ix->sref_bf, ix->ref_ext, ix->sref_ext, ix->rnorm, ix->srnorm,
-                          ix->labels, ix->slabels, s));
+    CKF(launch_gather_ref(perm_d, n_ref, ix->ref_bf, ix->sref_bf, ix->ref_ext, ix->sref_ext, s));
     // padding rows are the same in both orders
     CKF(cudaMemcpyAsync(ix->sref_bf + (size_t)n_ref * kDim, ix->ref_bf + (size_t)n_ref * kDim,
                         sizeof(__nv_bfloat16) * (size_t)(ix->n_pad - n_ref) * kDim, cudaMemcpyDeviceToDevice, s));
     CKF(cudaMemcpyAsync(ix->sref_ext + (size_t)n_ref * kExt, ix->ref_ext + (size_t)n_ref * kExt,
                         sizeof(__nv_bfloat16) * (size_t)(ix->n_pad - n_ref) * kExt, cudaMemcpyDeviceToDevice, s));
-    CKF(launch_fill_float(ix->srnorm + n_ref, ix->n_pad - n_ref, kPadNorm, s));
     CKF(cudaStreamSynchronize(s));  // perm (host vector) must outlive the copy
   }
   if (!make_tc_tensor_maps(ix->ref_bf, ix->sref_bf, ix->ref_ext, ix->sref_ext, ix->n_pad, &ix->tc))

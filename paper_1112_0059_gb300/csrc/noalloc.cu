@@ -178,7 +178,7 @@ extern "C" LNBNN_API lnbnn_status knn_search_noalloc(const uint8_t* ref, int64_t
   begin.fill(err, sizeof(uint32_t), 0u);
   if (sched.queue) begin.fill(sched.queue, sizeof(uint32_t), 0u);
   if (splits > 1) begin.fill(row_thr, sizeof(int32_t) * (size_t)m_pad, 0x7F7F7F7Fu);
-  cudaError_t e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, nullptr, ref_ext, s);
+  cudaError_t e = launch_prep_ref(ref, n_ref, n_pad, kDim, 0, ref_bf, ref_ext, s);
   if (e == cudaSuccess) e = launch_prep_query(queries, n_queries, m_pad, kDim, 0, qbf, qext, begin, s);
   if (e == cudaSuccess)
     e = launch_knn_tc(maps, false, qbf, qext, n_queries, m_pad, n_ref, (int)splits, split_len, k, lists, m_pad,

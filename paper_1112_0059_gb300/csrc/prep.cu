@@ -63,7 +63,7 @@ __device__ __forceinline__ void load8(const uint8_t* p, int row_bytes, uint8_t (
 }
 
 __global__ void prep_ref_kernel(const uint8_t* __restrict__ ref, int64_t n_ref, int64_t n_pad, int row_bytes,
-                                int loc_w, __nv_bfloat16* __restrict__ ref_bf, float* __restrict__ rnorm,
+                                int loc_w, __nv_bfloat16* __restrict__ ref_bf,
                                 __nv_bfloat16* __restrict__ ref_ext) {
   const int sub = threadIdx.x % kThreadsPerRow;
   const int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.x / kThreadsPerRow;
@@ -90,7 +90,6 @@ __global__ void prep_ref_kernel(const uint8_t* __restrict__ ref, int64_t n_ref, 
     ly = (int32_t)ref[row * row_bytes + kDim + 1] - 128;
   }
   const int32_t norm = real ? ss + loc_w * (lx * lx + ly * ly) : (int32_t)kPadNorm;
-  if (rnorm) rnorm[row] = (float)norm;
   // base-256 digits: d2 <= 56 for real rows, 512 for padding rows
   const float v[kExt] = {(float)(norm & 255), (float)((norm >> 8) & 255), (float)(norm >> 16), 1.0f, 256.0f,
                          65536.0f, (float)lx, (float)lx, (float)ly, (float)ly, 0, 0, 0, 0, 0, 0};
@@ -160,9 +159,7 @@ __global__ void label_hist_kernel(const int32_t* __restrict__ labels, int64_t n,
 
 __global__ void gather_ref_kernel(const int64_t* __restrict__ perm, int64_t n, const __nv_bfloat16* __restrict__ src_bf,
                                   __nv_bfloat16* __restrict__ dst_bf, const __nv_bfloat16* __restrict__ src_ext,
-                                  __nv_bfloat16* __restrict__ dst_ext, const float* __restrict__ src_norm,
-                                  float* __restrict__ dst_norm, const int32_t* __restrict__ src_lab,
-                                  int32_t* __restrict__ dst_lab) {
+                                  __nv_bfloat16* __restrict__ dst_ext) {
   // one warp per row: 32 lanes x 8 bytes of bf16
   const int lane = threadIdx.x & 31;
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -171,15 +168,6 @@ __global__ void gather_ref_kernel(const int64_t* __restrict__ perm, int64_t n, c
   reinterpret_cast<uint2*>(dst_bf + row * kDim)[lane] = reinterpret_cast<const uint2*>(src_bf + from * kDim)[lane];
   if (lane < 2)
     reinterpret_cast<uint4*>(dst_ext + row * kExt)[lane] = reinterpret_cast<const uint4*>(src_ext + from * kExt)[lane];
-  if (lane == 0) {
-    dst_norm[row] = src_norm[from];
-    dst_lab[row] = src_lab[from];
-  }
-}
-
-__global__ void fill_float_kernel(float* __restrict__ dst, int64_t n, float v) {
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    dst[j] = v;
 }
 
 __global__ void begin_kernel(const __grid_constant__ Begin begin) { begin_part(begin, blockIdx.x, gridDim.x); }
@@ -195,20 +183,12 @@ cudaError_t launch_begin(const Begin& begin, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_fill_float(float* dst, int64_t n, float v, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > 1024) blocks = 1024;
-  fill_float_kernel<<<(unsigned)blocks, 256, 0, s>>>(dst, n, v);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_prep_ref(const uint8_t* ref, int64_t n_ref, int64_t n_pad, int row_bytes, int loc_w,
-                            __nv_bfloat16* ref_bf, float* rnorm, __nv_bfloat16* ref_ext, cudaStream_t s) {
+                            __nv_bfloat16* ref_bf, __nv_bfloat16* ref_ext, cudaStream_t s) {
   if (!row_layout_ok(row_bytes, loc_w)) return cudaErrorInvalidValue;
   const int64_t blocks = (n_pad + kRowsPerBlock - 1) / kRowsPerBlock;
   prep_ref_kernel<<<(unsigned)blocks, kRowsPerBlock * kThreadsPerRow, 0, s>>>(ref, n_ref, n_pad, row_bytes, loc_w,
-                                                                               ref_bf, rnorm, ref_ext);
+                                                                               ref_bf, ref_ext);
   return cudaGetLastError();
 }
 
@@ -231,12 +211,9 @@ cudaError_t launch_label_hist(const int32_t* labels, int64_t n, int32_t C, unsig
 }
 
 cudaError_t launch_gather_ref(const int64_t* perm, int64_t n, const __nv_bfloat16* src_bf, __nv_bfloat16* dst_bf,
-                              const __nv_bfloat16* src_ext,
-                              __nv_bfloat16* dst_ext, const float* src_norm, float* dst_norm,
-                              const int32_t* src_lab, int32_t* dst_lab, cudaStream_t s) {
+                              const __nv_bfloat16* src_ext, __nv_bfloat16* dst_ext, cudaStream_t s) {
   const int64_t blocks = (n * 32 + 255) / 256;
-  gather_ref_kernel<<<(unsigned)blocks, 256, 0, s>>>(perm, n, src_bf, dst_bf, src_ext, dst_ext, src_norm, dst_norm,
-                                                     src_lab, dst_lab);
+  gather_ref_kernel<<<(unsigned)blocks, 256, 0, s>>>(perm, n, src_bf, dst_bf, src_ext, dst_ext);
   return cudaGetLastError();
 }
 

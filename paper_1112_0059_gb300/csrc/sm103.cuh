@@ -202,22 +202,8 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Each thread of the warp reads 32 consecutive 32-bit columns of its TMEM lane.
-__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-
-// The same load with a reduction: mn also receives the minimum of the 32
-// columns as unsigned 32-bit integers (which orders non-negative float bit
+// Each thread of the warp reads 32 consecutive 32-bit columns of its TMEM lane;
+// mn receives the minimum of the 32 columns as unsigned 32-bit integers (which orders non-negative float bit
 // patterns like the floats).
 __device__ __forceinline__ void tmem_ld_min_32x32b_x32(uint32_t taddr, uint32_t (&r)[32], uint32_t& mn) {
   asm volatile(
@@ -231,8 +217,6 @@ __device__ __forceinline__ void tmem_ld_min_32x32b_x32(uint32_t taddr, uint32_t 
       : "r"(taddr)
       : "memory");
 }
-
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Wait for this thread's TMEM loads; the registers are passed through the
 // wait so no use of them can be scheduled before it.
