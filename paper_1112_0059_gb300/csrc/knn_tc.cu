@@ -1127,17 +1127,17 @@ __global__ void __launch_bounds__(kThreadsOf<Epilogue>, 1)
               if constexpr (kRanked > 0) {
                 int32_t y[4] = {(int32_t)mn, INT32_MAX, INT32_MAX, INT32_MAX};
                 if (wu.octets || wu.pairs) group_values(v, wu.octets, wu.pairs, y);
+                int left = wu.octets ? 4 : 1;
 #pragma unroll 1
-                for (int g = 0; g < (wu.octets ? 4 : 1); ++g) {
+                do {
                   const int32_t x = y[0];
                   y[0] = y[1];
                   y[1] = y[2];
                   y[2] = y[3];
-                  if (!__any_sync(0xffffffffu, x < ranked[kRanked - 1])) continue;
 #pragma unroll
                   for (int j = kRanked - 1; j > 0; --j) ranked[j] = max(ranked[j - 1], min(ranked[j], x));
                   ranked[0] = min(ranked[0], x);
-                }
+                } while (--left > 0);
               } else {
                 if (wu.octets) most = max(most, (int32_t)mn);
                 least = min(least, (int32_t)mn);
